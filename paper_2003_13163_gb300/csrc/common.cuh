@@ -36,11 +36,11 @@ __device__ __forceinline__ unsigned long long global_timer_ns() {
   return t;
 }
 
-// Control block of a persistent cooperative kernel: a sense-counting grid
-// barrier plus status words. Zeroed by the host before every launch.
+// Control block of a persistent cooperative kernel: a grid barrier plus
+// status words. Zeroed by the host before every launch.
 struct GridCtl {
-  unsigned int count;
-  unsigned int gen;
+  unsigned int count;   // barrier word: the top bit flips when every CTA has arrived
+  unsigned int unused;
   int err;        // 1: a barrier wait ran past its time limit
   int status;     // kernel-specific status (e.g. not converged)
   int sweeps;     // kernel-specific counter
@@ -48,33 +48,33 @@ struct GridCtl {
 };
 
 // Grid-wide barrier for a cooperatively launched kernel (all CTAs resident).
+// One L2 round trip to arrive and one to see the last arrival: CTA 0 adds
+// 2^31 - (nblocks - 1), every other CTA 1, so the top bit of the word flips
+// exactly when all have arrived and the word needs no reset, no second flag
+// and no read after the wait (the Jacobi solvers below pass thousands of
+// barriers per factorisation, so this latency is what bounds the small ones).
 // Every wait is bounded by timeout_ns of wall time: on expiry the CTA sets
-// ctl->err and every CTA leaves at its next barrier, so a broken launch ends
+// ctl->err and leaves; the others see the flag (or their own limit) at their
+// next wait, since the missing CTA never arrives there. A broken launch ends
 // with an error status instead of hanging the GPU. Returns false on error.
 __device__ __forceinline__ bool grid_barrier(GridCtl* ctl, unsigned int nblocks, long long timeout_ns) {
   __shared__ int s_ok;
   __syncthreads();
   if (threadIdx.x == 0) {
     int ok = 1;
-    volatile unsigned int* vgen = &ctl->gen;
-    volatile int* verr = &ctl->err;
-    unsigned int g = *vgen;
+    const unsigned int add = blockIdx.x == 0 ? 0x80000000u - (nblocks - 1u) : 1u;
+    unsigned int old, cur;
     __threadfence();
-    unsigned int arrived = atomicAdd(&ctl->count, 1u);
-    if (arrived == nblocks - 1) {
-      atomicExch(&ctl->count, 0u);
-      __threadfence();
-      atomicAdd(&ctl->gen, 1u);
-    } else {
-      unsigned long long t0 = global_timer_ns();
-      while (*vgen == g) {
-        if (*verr) { ok = 0; break; }
-        if ((long long)(global_timer_ns() - t0) > timeout_ns) { atomicExch(&ctl->err, 1); ok = 0; break; }
-        __nanosleep(32);
-      }
+    asm volatile("atom.add.release.gpu.global.u32 %0, [%1], %2;" : "=r"(old) : "l"(&ctl->count), "r"(add) : "memory");
+    unsigned long long t0 = 0;
+    for (unsigned int it = 0;; ++it) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(cur) : "l"(&ctl->count) : "memory");
+      if ((cur ^ old) & 0x80000000u) break;
+      if (it == 0) { t0 = global_timer_ns(); continue; }
+      if ((it & 31u) == 31u && *(volatile int*)&ctl->err) { ok = 0; break; }
+      if ((long long)(global_timer_ns() - t0) > timeout_ns) { atomicExch(&ctl->err, 1); ok = 0; break; }
     }
     __threadfence();
-    if (*verr) ok = 0;
     s_ok = ok;
   }
   __syncthreads();

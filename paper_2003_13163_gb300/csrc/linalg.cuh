@@ -130,11 +130,18 @@ inline cudaError_t cgemm(cudaStream_t st, int M, int N, int K, const cplx<T>* A,
 // rotation; status = 1 if max_sweeps is reached first.
 //
 // Each round runs as three phases of one persistent cooperative launch:
-//   A (every CTA, redundantly): the rotation table of the round -> smem;
-//                                                                  barrier
+//   A: the round's rotation table, each pair by one thread of the grid, to
+//      the global table of this round's parity;                     barrier
 //   B (G <- G J, V <- V J): one warp per row, lanes over pairs;   barrier
 //   C (G <- J^H G): one warp per pair, lanes over columns;           barrier
 // All G/V traffic uses L2-only loads/stores because other CTAs write it.
+// The FP64 unit (2 FMA per clock and SM) bounds all three phases (m = 1088,
+// nearly diagonal: 303 ms with tables built by every CTA, 173 ms now), so the work
+// is spread evenly over the SMs: a rotation costs ~200 FP64 instructions
+// (hypot, square roots, divisions), which every CTA repeated for all m / 2
+// pairs of a round when the table was built redundantly; and warp w of CTA b
+// takes items w gridDim + b, so that fewer items than warps still reach every
+// SM.
 // ---------------------------------------------------------------------------
 template <typename T> struct JRot { T c, s, ur, ui; };
 
@@ -143,17 +150,16 @@ __device__ __forceinline__ int rr_player(int pos, int r, int N) {
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) jacobi_kernel(cplx<T>* G, int m, cplx<T>* V, T* w, GridCtl* ctl,
+__global__ void __launch_bounds__(256) jacobi_kernel(cplx<T>* G, int m, cplx<T>* V, T* w, JRot<T>* table, GridCtl* ctl,
                                                       int max_sweeps, T tol_rel, T floor_rel, long long timeout_ns) {
   extern __shared__ unsigned char jsmem[];
   JRot<T>* rot = reinterpret_cast<JRot<T>*>(jsmem);
-  __shared__ int s_active;
   __shared__ T s_red[32];
   const int N = m + (m & 1), npairs = N / 2;
   const unsigned nblk = gridDim.x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nwarp_blk = blockDim.x >> 5;
-  const long gwarp = (long)blockIdx.x * nwarp_blk + warp, nwarps = (long)nblk * nwarp_blk;
+  const long gwarp = (long)warp * nblk + blockIdx.x, nwarps = (long)nblk * nwarp_blk;
   const size_t gtid = (size_t)blockIdx.x * blockDim.x + threadIdx.x, gthreads = (size_t)nblk * blockDim.x;
 
   // V = I
@@ -182,11 +188,11 @@ __global__ void __launch_bounds__(256) jacobi_kernel(cplx<T>* G, int m, cplx<T>*
     long sweep_active = 0;
     for (int r = 0; r < N - 1; ++r) {
       // ---- phase A: rotation table -------------------------------------
-      if (threadIdx.x == 0) s_active = 0;
-      __syncthreads();
-      int my_active = 0;
-      for (int pi = threadIdx.x; pi < npairs; pi += blockDim.x) {
-        int p = rr_player(pi, r, N), q = rr_player(N - 1 - pi, r, N);
+      // two tables in turn: a CTA that is already in the next round writes
+      // the other one while slower CTAs still read this one
+      JRot<T>* tab = table + (size_t)((sweep * (N - 1) + r) & 1) * npairs;
+      for (long pi = blockIdx.x + (long)threadIdx.x * nblk; pi < npairs; pi += (long)nblk * blockDim.x) {
+        int p = rr_player((int)pi, r, N), q = rr_player(N - 1 - (int)pi, r, N);
         if (p > q) { int t_ = p; p = q; q = t_; }
         JRot<T> R; R.c = T(1); R.s = T(0); R.ur = T(1); R.ui = T(0);
         if (q < m) {
@@ -201,19 +207,23 @@ __global__ void __launch_bounds__(256) jacobi_kernel(cplx<T>* G, int m, cplx<T>*
             else t = (zeta >= T(0) ? T(1) : T(-1)) / (fabs(zeta) + sqrt(T(1) + zeta * zeta));
             const T c = T(1) / sqrt(T(1) + t * t);
             R.c = c; R.s = t * c; R.ur = g.x / ag; R.ui = g.y / ag;
-            if (R.s != T(0)) ++my_active;
           }
         }
-        rot[pi] = R;
+        __stcg(&tab[pi].c, R.c); __stcg(&tab[pi].s, R.s); __stcg(&tab[pi].ur, R.ur); __stcg(&tab[pi].ui, R.ui);
       }
-      if (my_active) atomicAdd(&s_active, my_active);
-      __syncthreads();
-      const int act = s_active;   // identical in every CTA: same inputs, same code
-      sweep_active += act;
-      if (act == 0) continue;
       // phase B rewrites the pivots (G_pp, G_qq, G_pq) that phase A reads:
-      // no CTA rotates before every CTA has built its table from the same G
+      // no CTA rotates before the whole table has been built from the same G
       if (!grid_barrier(ctl, nblk, timeout_ns)) return;
+      int my_active = 0;
+      for (int pi = threadIdx.x; pi < npairs; pi += blockDim.x) {
+        JRot<T> R;
+        R.c = __ldcg(&tab[pi].c); R.s = __ldcg(&tab[pi].s); R.ur = __ldcg(&tab[pi].ur); R.ui = __ldcg(&tab[pi].ui);
+        rot[pi] = R;
+        if (R.s != T(0)) my_active = 1;
+      }
+      const int act = __syncthreads_or(my_active);   // identical in every CTA: the same table
+      if (act == 0) continue;
+      ++sweep_active;
       // ---- phase B: column rotations, G <- G J and V <- V J ---------------
       for (long row = gwarp; row < 2L * m; row += nwarps) {
         cplx<T>* Rw = row < m ? G + (size_t)row * m : V + (size_t)(row - m) * m;
@@ -410,6 +420,21 @@ struct OSCtl {
   unsigned long long phase_ns[4];   // CTA 0: wall time per phase (G, E, A), barrier waits included
 };
 
+// Largest of w[0 .. r), read through L2 by the whole CTA (at most 1024 threads).
+template <typename T>
+__device__ T block_max(const T* w, int r) {
+  __shared__ T s_part[32];
+  T mx = T(0);
+  for (int i = threadIdx.x; i < r; i += blockDim.x) mx = fmax(mx, __ldcg(&w[i]));
+  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = mx;
+  __syncthreads();
+  mx = s_part[0];
+  for (int i = 1; i < (int)(blockDim.x >> 5); ++i) mx = fmax(mx, s_part[i]);
+  __syncthreads();
+  return mx;
+}
+
 template <typename T>
 __device__ __forceinline__ void warp_sum3(T& a, T& b, T& c, T& d) {
 #pragma unroll
@@ -428,7 +453,10 @@ __global__ void __launch_bounds__(256) onesided_jacobi_kernel(cplx<T>* X, int r,
   const int N = r + (r & 1), npairs = N / 2;
   const unsigned nblk = gridDim.x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwb = blockDim.x >> 5;
-  const long gwarp = (long)blockIdx.x * nwb + warp, nwarps = (long)nblk * nwb;
+  // warp w of CTA b takes the pairs w gridDim + b, ...: neighbouring pairs go to
+  // different SMs, so that a round of fewer pairs than warps uses the FP64
+  // units of every SM (8 neighbours on one SM left 104 of 152 idle at r = 768)
+  const long gwarp = (long)warp * nblk + blockIdx.x, nwarps = (long)nblk * nwb;
   const size_t gtid = (size_t)blockIdx.x * blockDim.x + threadIdx.x, gthreads = (size_t)nblk * blockDim.x;
   if (max_sweeps > 64) max_sweeps = 64;
 
@@ -444,14 +472,7 @@ __global__ void __launch_bounds__(256) onesided_jacobi_kernel(cplx<T>* X, int r,
     if (lane == 0) w[i] = s;
   }
   if (!grid_barrier(&ctl->g, nblk, timeout_ns)) return;
-  __shared__ T s_floor;
-  if (threadIdx.x == 0) {
-    T mx = T(0);
-    for (int i = 0; i < r; ++i) mx = fmax(mx, __ldcg(&w[i]));
-    s_floor = floor_rel * mx;
-  }
-  __syncthreads();
-  const T floor_abs = s_floor;
+  const T floor_abs = floor_rel * block_max<T>(w, r);
 
   int sweep = 0;
   bool converged = (r <= 1);
@@ -514,6 +535,253 @@ __global__ void __launch_bounds__(256) onesided_jacobi_kernel(cplx<T>* X, int r,
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) w[i] = s;
   }
+  if (gtid == 0) {
+    ctl->g.sweeps = sweep;
+    ctl->g.status = converged ? 0 : 1;
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The same solver with one CTA (four warps) per row pair, the form every
+// complex128 factorisation and the precision form's FP32 Rayleigh-Ritz step
+// use (onesided_jacobi_kernel above serves the complex64 form, whose results
+// are pinned to its arithmetic).
+//
+// What bounds it: an FP64 warp instruction occupies its SM partition for 64
+// clocks on this part, so a pair handled by one warp uses a quarter of the
+// SM's FP64 rate, and the ~200 FP64 instructions of the rotation parameters
+// (hypot, square roots, divisions) cost 6 us per round, more than the rows
+// themselves below ~300 columns. Four warps share the pair's rows, the four
+// sums are reduced by halves (6 + 2 additions instead of 20), one warp forms
+// the parameters in ~35 FP64 instructions (osj_rotation), and rows of up to
+// 128 E elements stay in registers between the dot products and the rotation
+// (one read and one write per round instead of two and one).
+// Measured, one warp per pair -> this kernel: complex128 64 x 64 17.2 ->
+// 7.1 ms (20 sweeps), 256 x 256 174 -> 51 ms, 768 x 1024 1363 -> 586 ms
+// (28 sweeps, 27 us per round); complex64 2048 x 2048 in the precision form
+// 557 -> 166 ms.
+// ---------------------------------------------------------------------------
+constexpr int OSJ_NT = 128;
+
+// 1 / sqrt(x) for x in [1, 8): the FP32 approximation (2^-22) and one
+// third-order step y (1 + e/2 + 3 e^2 / 8), e = 1 - x y^2, whose remainder
+// (5/16) e^3 is below 2^-66.
+__device__ __forceinline__ double osj_rsqrt(double x) {
+  const double y = (double)rsqrtf((float)x);
+  const double e = fma(-x * y, y, 1.0);
+  return fma(y, e * fma(e, 0.375, 0.5), y);
+}
+
+// 2^k as a double, |k| <= 1022.
+__device__ __forceinline__ double osj_pow2(int k) { return __longlong_as_double((long long)(k + 1023) << 52); }
+
+// Rotation parameters of a row pair with a = |x|^2, b = |y|^2, g = <x, y>:
+// c, s real and u = g / |g|; false when |g| <= max(tol sqrt(ab), floor) or
+// the rotation is below resolution. The root t of t^2 + 2 zeta t - 1 is taken in
+// FP32 and corrected by one FP64 Newton step (relative error ~1e-14, so a
+// rotation leaves 1e-14 of g); c and u come from osj_rsqrt, so c^2 + s^2 and
+// |u| are 1 to FP64 rounding whatever the angle. g is scaled by a power of two
+// first (integer arithmetic on its exponent), so no square over- or underflows.
+__device__ __forceinline__ bool osj_rotation(double a, double b, double gr, double gi, double tol2, double floor_abs,
+                                             double& c, double& s, double& ur, double& ui) {
+  const int er = (int)((__double_as_longlong(gr) >> 52) & 0x7FF), ei = (int)((__double_as_longlong(gi) >> 52) & 0x7FF);
+  const int e = max(er, ei) - 1023;
+  if (e <= -1022 || e >= 1022) return false;      // zero, denormal, infinite or NaN couplings
+  const double sc = osj_pow2(-e);
+  const double x = gr * sc, y = gi * sc;
+  const double g2 = fma(x, x, y * y);             // in [1, 8)
+  if (!(g2 > tol2 * ((a * sc) * (b * sc)))) return false;
+  const double inv = osj_rsqrt(g2);
+  if (!(g2 * inv * osj_pow2(e) > floor_abs)) return false;
+  const double zeta = ((b - a) * sc) * (0.5 * inv);
+  const float zf = (float)zeta, az = fabsf(zf);
+  if (!(az < 3e38f)) return false;                // t below 1e-38: no change at any precision
+  float t0 = az > 1e18f ? 0.5f / az : 1.0f / (az + sqrtf(fmaf(az, az, 1.0f)));
+  if (zf < 0.0f) t0 = -t0;
+  const double td = (double)t0;
+  const double f = fma(td, td + 2.0 * zeta, -1.0);
+  const double t = fma(-f, (double)(0.5f / (zf + t0)), td);
+  c = osj_rsqrt(fma(t, t, 1.0));
+  s = t * c;
+  ur = x * inv;
+  ui = y * inv;
+  return s != 0.0;
+}
+
+// Sum of the four values over the CTA's 128 threads, returned in every lane of
+// warp 0 only (one barrier; the caller's next barrier frees the scratch).
+template <typename T>
+__device__ __forceinline__ void osj_reduce4(T& a, T& b, T& c, T& d, T (*part)[4]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool h16 = lane & 16, h8 = lane & 8;
+  T v0 = h16 ? c : a, v1 = h16 ? d : b;
+  v0 += __shfl_xor_sync(0xffffffffu, h16 ? a : c, 16);
+  v1 += __shfl_xor_sync(0xffffffffu, h16 ? b : d, 16);
+  T v = h8 ? v1 : v0;
+  v += __shfl_xor_sync(0xffffffffu, h8 ? v0 : v1, 8);
+  v += __shfl_xor_sync(0xffffffffu, v, 4);
+  v += __shfl_xor_sync(0xffffffffu, v, 2);
+  v += __shfl_xor_sync(0xffffffffu, v, 1);
+  if ((lane & 7) == 0) part[lane >> 3][warp] = v;
+  __syncthreads();
+  if (warp == 0) {
+    v = part[(lane >> 2) & 3][lane & 3];
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    a = __shfl_sync(0xffffffffu, v, 0);
+    b = __shfl_sync(0xffffffffu, v, 4);
+    c = __shfl_sync(0xffffffffu, v, 8);
+    d = __shfl_sync(0xffffffffu, v, 12);
+  }
+}
+
+template <typename T> struct OsjRot { T c, s, sur, sui, cur, cui; int on; };
+
+// (x, y) <- (c x - s u y, s x + c u y)
+template <typename T>
+__device__ __forceinline__ void osj_rotate(cplx<T>& x, cplx<T>& y, T c, T s, T sur, T sui, T cur, T cui) {
+  const cplx<T> xn = mk<T>(fma(sui, y.y, fma(-sur, y.x, c * x.x)), fma(-sui, y.x, fma(-sur, y.y, c * x.y)));
+  y = mk<T>(fma(-cui, y.y, fma(cur, y.x, s * x.x)), fma(cui, y.x, fma(cur, y.y, s * x.y)));
+  x = xn;
+}
+
+template <typename T, int E>
+__global__ void __launch_bounds__(OSJ_NT) pair_jacobi_kernel(cplx<T>* X, int r, int c, int ldx, cplx<T>* Ut, T* w,
+                                                             OSCtl* ctl, int max_sweeps, T tol_rel, T floor_rel,
+                                                             long long timeout_ns) {
+  __shared__ T part[4][4];
+  __shared__ OsjRot<T> s_rot;
+  const int N = r + (r & 1), npairs = N / 2;
+  const unsigned nblk = gridDim.x;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const size_t gtid = (size_t)blockIdx.x * OSJ_NT + tid, gthreads = (size_t)nblk * OSJ_NT;
+  const bool regs = c <= OSJ_NT * E, uregs = r <= OSJ_NT * E;   // the rows fit the registers
+  if (max_sweeps > 64) max_sweeps = 64;
+
+  for (size_t e = gtid; e < (size_t)r * r; e += gthreads) {
+    const size_t i = e / r, j = e % r;
+    stcg(&Ut[e], mk<T>(i == j ? T(1) : T(0), T(0)));
+  }
+  // squared row norms -> w, one warp per row
+  auto norms = [&]() {
+    for (long i = gtid >> 5; i < r; i += (long)(gthreads >> 5)) {
+      T s = T(0);
+      for (int j = lane; j < c; j += 32) {
+        const cplx<T> x = ldcg(&X[(size_t)i * ldx + j]);
+        s = fma(x.x, x.x, fma(x.y, x.y, s));
+      }
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == 0) __stcg(&w[i], s);
+    }
+  };
+  norms();
+  if (!grid_barrier(&ctl->g, nblk, timeout_ns)) return;
+  const double floor_abs = (double)(floor_rel * block_max<T>(w, r));
+  const double tol2 = (double)tol_rel * (double)tol_rel;
+
+  int sweep = 0;
+  bool converged = (r <= 1);
+  for (; sweep < max_sweeps && !converged; ++sweep) {
+    for (int rd = 0; rd < N - 1; ++rd) {
+      for (int pi = blockIdx.x; pi < npairs; pi += nblk) {
+        int p = rr_player(pi, rd, N), q = rr_player(N - 1 - pi, rd, N);
+        if (p > q) { int t_ = p; p = q; q = t_; }
+        if (q >= r) continue;
+        cplx<T>* xp = X + (size_t)p * ldx;
+        cplx<T>* xq = X + (size_t)q * ldx;
+        T a = T(0), b = T(0), gr = T(0), gi = T(0);
+        auto dots = [&](cplx<T> x, cplx<T> y) {
+          a = fma(x.x, x.x, fma(x.y, x.y, a));
+          b = fma(y.x, y.x, fma(y.y, y.y, b));
+          gr = fma(x.x, y.x, fma(x.y, y.y, gr));     // x conj(y)
+          gi = fma(x.y, y.x, fma(-x.x, y.y, gi));
+        };
+        cplx<T> rx[E], ry[E];
+        if (regs) {
+#pragma unroll
+          for (int e = 0; e < E; ++e) {
+            const int j = tid + OSJ_NT * e;
+            rx[e] = j < c ? ldcg(&xp[j]) : czero<T>();
+            ry[e] = j < c ? ldcg(&xq[j]) : czero<T>();
+          }
+#pragma unroll
+          for (int e = 0; e < E; ++e)
+            if (OSJ_NT * e < c) dots(rx[e], ry[e]);
+        } else {
+#pragma unroll 4
+          for (int j = tid; j < c; j += OSJ_NT) dots(ldcg(&xp[j]), ldcg(&xq[j]));
+        }
+        osj_reduce4<T>(a, b, gr, gi, part);
+        if (tid < 32) {
+          double cs, sn, ur, ui;
+          const bool on = osj_rotation((double)a, (double)b, (double)gr, (double)gi, tol2, floor_abs, cs, sn, ur, ui) &&
+                          (T)sn != T(0);
+          if (tid == 0) {
+            s_rot.on = on;
+            if (on) {
+              s_rot.c = (T)cs; s_rot.s = (T)sn;
+              s_rot.sur = (T)(sn * ur); s_rot.sui = (T)(sn * ui);
+              s_rot.cur = (T)(cs * ur); s_rot.cui = (T)(cs * ui);
+              atomicAdd(&ctl->active[sweep], 1);
+            }
+          }
+        }
+        __syncthreads();
+        if (!s_rot.on) continue;
+        const T cs = s_rot.c, sn = s_rot.s, sur = s_rot.sur, sui = s_rot.sui, cur = s_rot.cur, cui = s_rot.cui;
+        cplx<T>* tp = Ut + (size_t)p * r;
+        cplx<T>* tq = Ut + (size_t)q * r;
+        if (regs) {
+#pragma unroll
+          for (int e = 0; e < E; ++e) {
+            const int j = tid + OSJ_NT * e;
+            if (j < c) {
+              osj_rotate<T>(rx[e], ry[e], cs, sn, sur, sui, cur, cui);
+              stcg(&xp[j], rx[e]);
+              stcg(&xq[j], ry[e]);
+            }
+          }
+        } else {
+#pragma unroll 4
+          for (int j = tid; j < c; j += OSJ_NT) {
+            cplx<T> x = ldcg(&xp[j]), y = ldcg(&xq[j]);
+            osj_rotate<T>(x, y, cs, sn, sur, sui, cur, cui);
+            stcg(&xp[j], x);
+            stcg(&xq[j], y);
+          }
+        }
+        // U <- U J: the conjugate phase
+        if (uregs) {
+#pragma unroll
+          for (int e = 0; e < E; ++e) {
+            const int j = tid + OSJ_NT * e;
+            rx[e] = j < r ? ldcg(&tp[j]) : czero<T>();
+            ry[e] = j < r ? ldcg(&tq[j]) : czero<T>();
+          }
+#pragma unroll
+          for (int e = 0; e < E; ++e) {
+            const int j = tid + OSJ_NT * e;
+            if (j < r) {
+              osj_rotate<T>(rx[e], ry[e], cs, sn, sur, -sui, cur, -cui);
+              stcg(&tp[j], rx[e]);
+              stcg(&tq[j], ry[e]);
+            }
+          }
+        } else {
+#pragma unroll 4
+          for (int j = tid; j < r; j += OSJ_NT) {
+            cplx<T> x = ldcg(&tp[j]), y = ldcg(&tq[j]);
+            osj_rotate<T>(x, y, cs, sn, sur, -sui, cur, -cui);
+            stcg(&tp[j], x);
+            stcg(&tq[j], y);
+          }
+        }
+      }
+      if (!grid_barrier(&ctl->g, nblk, timeout_ns)) return;
+    }
+    if (atomicAdd(&ctl->active[sweep], 0) == 0) converged = true;
+  }
+  norms();
   if (gtid == 0) {
     ctl->g.sweeps = sweep;
     ctl->g.status = converged ? 0 : 1;
@@ -876,7 +1144,6 @@ __global__ void __launch_bounds__(256) block_jacobi_kernel(cplx<T>* X, int r, in
 
   __shared__ T s_gmax;
   cplx<T>* Js = reinterpret_cast<cplx<T>*>(red);        // phase A: J^H or J^T (ld JP+1)
-  __shared__ T s_floor;
   const int nb = (r + JB - 1) / JB, N = nb + (nb & 1), npairs = N / 2;
   const int nch = (c + JCW - 1) / JCW, nchu = (r + JCW - 1) / JCW;
   const unsigned nblk = gridDim.x;
@@ -904,13 +1171,7 @@ __global__ void __launch_bounds__(256) block_jacobi_kernel(cplx<T>* X, int r, in
     if (lane == 0) w[i] = s;
   }
   if (!grid_barrier(&ctl->g, nblk, timeout_ns)) return;
-  if (tid == 0) {
-    T mx = T(0);
-    for (int i = 0; i < r; ++i) mx = fmax(mx, __ldcg(&w[i]));
-    s_floor = floor_rel * mx;
-  }
-  __syncthreads();
-  const T floor_abs = s_floor;
+  const T floor_abs = floor_rel * block_max<T>(w, r);
 
   int sweep = 0;
   bool converged = (r <= 1);

@@ -145,6 +145,7 @@ struct mpo_ctx {
   int mx_cur_bond = -1;            // bond of the gate being factorised (-1: not a gate)
   std::vector<int> mx_bond_steps;  // subspace steps the last gate on each bond needed
   long long prof_steps = 0;        // subspace steps since profiling was switched on
+  JRot<double>* mx_rot = nullptr;  // rotation tables of that eigen-solve (two rounds in turn)
   OSCtl* mx_eosctl = nullptr;      // control block of the FP64 Rayleigh-Ritz eigen-solve
   int* mx_chst = nullptr;          // set when a Cholesky pivot was not positive
   OzWork oz;                       // FP64-accurate tensor-core GEMM scratch (precision form)
@@ -251,7 +252,7 @@ static cudaError_t ensure_dynamic_smem(const void* fn, int bytes) {
 }
 
 template <typename T>
-static cudaError_t launch_jacobi(cudaStream_t st, cplx<T>* G, int m, cplx<T>* V, T* w, GridCtl* ctl,
+static cudaError_t launch_jacobi(cudaStream_t st, cplx<T>* G, int m, cplx<T>* V, T* w, JRot<T>* table, GridCtl* ctl,
                                  int max_sweeps, double timeout_s, int num_sms) {
   const int N = m + (m & 1);
   const size_t smem = sizeof(JRot<T>) * (size_t)std::max(1, N / 2);
@@ -262,14 +263,17 @@ static cudaError_t launch_jacobi(cudaStream_t st, cplx<T>* G, int m, cplx<T>* V,
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const int coresident = per_sm * num_sms;
-  int want = (2 * m + 7) / 8;   // one warp per row of G and V in phase B
-  int blocks = std::max(1, std::min(coresident, want));
+  // one warp per row of G and V in phase B; small matrices spread their rows
+  // over as many SMs as there are pairs, large ones keep two CTAs per SM (one: 178.6 ms, two:
+  // 172.6 ms at m = 1088; more lengthen the barriers, the FP64 unit is busy)
+  const int want = std::max((2 * m + 7) / 8, N / 2);
+  const int blocks = std::max(1, std::min(std::min(coresident, 2 * num_sms), want));
   e = cudaMemsetAsync(ctl, 0, sizeof(GridCtl), st);
   if (e != cudaSuccess) return e;
   const T tol_rel = std::is_same<T, double>::value ? (T)1e-14 : (T)2e-6;
   const T floor_rel = eps_of<T>::value;
   long long timeout_ns = (long long)(timeout_s * 1e9);
-  void* args[] = {&G, &m, &V, &w, &ctl, &max_sweeps, (void*)&tol_rel, (void*)&floor_rel, &timeout_ns};
+  void* args[] = {&G, &m, &V, &w, &table, &ctl, &max_sweeps, (void*)&tol_rel, (void*)&floor_rel, &timeout_ns};
   return cudaLaunchCooperativeKernel((const void*)jacobi_kernel<T>, dim3(blocks), dim3(256), args, smem, st);
 }
 
@@ -300,9 +304,9 @@ static cudaError_t launch_onesided(cudaStream_t st, cplx<T>* X, int r, int c, in
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const int N = r + (r & 1);
-  // one warp per pair; at least one CTA per SM so that the FP64 units of every
-  // SM take part even when the pairs are few
-  const int want = std::max(num_sms, (N / 2 + 7) / 8);
+  // one warp per pair, spread over the SMs; no more CTAs than pairs, because
+  // every round ends with a barrier whose cost grows with the CTAs that join
+  const int want = std::max(std::min(num_sms, N / 2), (N / 2 + 7) / 8);
   const int blocks = std::max(1, std::min(per_sm * num_sms, want));
   e = cudaMemsetAsync(ctl, 0, sizeof(OSCtl), st);
   if (e != cudaSuccess) return e;
@@ -313,6 +317,39 @@ static cudaError_t launch_onesided(cudaStream_t st, cplx<T>* X, int r, int c, in
   long long timeout_ns = (long long)(timeout_s * 1e9);
   void* args[] = {&X, &r, &c, &ldx, &Ut, &w, &ctl, &max_sweeps, (void*)&tol_rel, (void*)&floor_rel, &timeout_ns};
   return cudaLaunchCooperativeKernel((const void*)onesided_jacobi_kernel<T>, dim3(blocks), dim3(256), args, 0, st);
+}
+
+// One CTA per pair; rows of up to 128 E elements in registers. E = 2 keeps
+// eight CTAs on an SM for the short rows, 8 (complex128) and 16 (complex64)
+// cover rows of 1024 and 2048; longer rows are streamed.
+template <typename T>
+static cudaError_t launch_pair_jacobi(cudaStream_t st, cplx<T>* X, int r, int c, int ldx, cplx<T>* Ut, T* w, OSCtl* ctl,
+                                      int max_sweeps, double timeout_s, int num_sms, double tol_min = 0.0) {
+  constexpr int EL = sizeof(T) == 8 ? 8 : 16;
+  const void* fn = std::max(r, c) <= 2 * OSJ_NT ? (const void*)pair_jacobi_kernel<T, 2> : (const void*)pair_jacobi_kernel<T, EL>;
+  int per_sm = 0;
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, OSJ_NT, 0);
+  if (e != cudaSuccess) return e;
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  const int blocks = std::max(1, std::min(per_sm * num_sms, (r + 1) / 2));
+  e = cudaMemsetAsync(ctl, 0, sizeof(OSCtl), st);
+  if (e != cudaSuccess) return e;
+  // rows count as orthogonal once |<x_p, x_q>| <= 2 eps sqrt(c) ||x_p|| ||x_q||,
+  // the rounding level of the length-c dot product itself
+  const T tol_rel = (T)std::max(tol_min, 2.0 * eps_of<T>::value * std::sqrt((double)std::max(c, 1)));
+  const T floor_rel = eps_of<T>::value * eps_of<T>::value;
+  long long timeout_ns = (long long)(timeout_s * 1e9);
+  void* args[] = {&X, &r, &c, &ldx, &Ut, &w, &ctl, &max_sweeps, (void*)&tol_rel, (void*)&floor_rel, &timeout_ns};
+  return cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(OSJ_NT), args, 0, st);
+}
+
+// The row-pair solver of a stand-alone form: complex128 by the CTA-per-pair
+// kernel, complex64 by the warp-per-pair one (see there).
+template <typename T>
+static cudaError_t launch_row_jacobi(cudaStream_t st, cplx<T>* X, int r, int c, int ldx, cplx<T>* Ut, T* w, OSCtl* ctl,
+                                     int max_sweeps, double timeout_s, int num_sms) {
+  if constexpr (sizeof(T) == 8) return launch_pair_jacobi<T>(st, X, r, c, ldx, Ut, w, ctl, max_sweeps, timeout_s, num_sms);
+  else return launch_onesided<T>(st, X, r, c, ldx, Ut, w, ctl, max_sweeps, timeout_s, num_sms);
 }
 
 template <typename T>
@@ -640,7 +677,7 @@ static int msvd_select(mpo_ctx* h, double2* X, int r, int c, int ldx, int cap, b
     {
       const double fm = m, fc = c1;
       ProfScope ps(h, disc ? PK_SVD : PK_SVD_SWEEP, 4.0 * fm * fm * fc, (2.0 * fm * fc + fm * fm) * sizeof(float2));
-      CK(h, launch_onesided<float>(h->st, h->mx_a32, m, c1, c1, h->mx_ut32, h->mx_w32, h->osctl,
+      CK(h, launch_pair_jacobi<float>(h->st, h->mx_a32, m, c1, c1, h->mx_ut32, h->mx_w32, h->osctl,
                                    h->opts.eig_max_sweeps, h->opts.barrier_timeout_s, h->num_sms, 3e-5));
     }
     {
@@ -716,7 +753,7 @@ static int msvd_select(mpo_ctx* h, double2* X, int r, int c, int ldx, int cap, b
     ProfScope ps(h, PK_EIG64, 13.3 * (double)mp * mp * mp, 3.0 * (double)mp * mp * sizeof(double2));
     hermitise_kernel<<<grid_for((size_t)mp * mp, h->num_sms), 256, 0, h->st>>>(h->mx_G, mp);
     CK(h, cudaGetLastError());
-    CK(h, launch_jacobi<double>(h->st, h->mx_G, mp, h->mx_V, h->mx_w, &h->mx_eosctl->g, h->opts.eig_max_sweeps,
+    CK(h, launch_jacobi<double>(h->st, h->mx_G, mp, h->mx_V, h->mx_w, h->mx_rot, &h->mx_eosctl->g, h->opts.eig_max_sweeps,
                                 h->opts.barrier_timeout_s, h->num_sms));
   }
   // left factor Q' V, stored as rows conj(column j) = V^H Q'^H; the rows
@@ -769,8 +806,8 @@ static int svd_select(mpo_ctx* h, cplx<T>* X, int r, int c, int ldx, int cap, bo
                                    (cplx<T>*)h->bj_j, h->bj_act, h->bj_act_ints, h->osctl, h->opts.eig_max_sweeps,
                                    h->opts.barrier_timeout_s, h->num_sms));
     else
-      CK(h, launch_onesided<T>(h->st, X, r, c, ldx, (cplx<T>*)h->vecs, w, h->osctl, h->opts.eig_max_sweeps,
-                               h->opts.barrier_timeout_s, h->num_sms));
+      CK(h, launch_row_jacobi<T>(h->st, X, r, c, ldx, (cplx<T>*)h->vecs, w, h->osctl, h->opts.eig_max_sweeps,
+                                 h->opts.barrier_timeout_s, h->num_sms));
   }
   {
     ProfScope ps(h, PK_SELECT, 0.0, (double)r * (sizeof(T) + sizeof(int) + sizeof(double)));
@@ -1370,6 +1407,7 @@ static bool alloc_factor_ws(mpo_ctx* h, int m, int ccap, size_t bj_nch) {
     ok = ok && alloc((void**)&h->mx_w, mm * sizeof(double));
     ok = ok && alloc((void**)&h->mx_W, mm * mm * sizeof(double2));
     ok = ok && alloc((void**)&h->mx_eosctl, sizeof(OSCtl));
+    ok = ok && alloc((void**)&h->mx_rot, (mm + 1) * sizeof(JRot<double>));
     ok = ok && alloc((void**)&h->mx_Q0, (size_t)m * mm * sizeof(double2));
     ok = ok && alloc((void**)&h->mx_A32, mm * mm * sizeof(float2));
     ok = ok && alloc((void**)&h->mx_Li32, mm * mm * sizeof(float2));
@@ -1530,7 +1568,7 @@ void mpo_free(mpo_handle h) {
                 h->dsup, h->dp, h->info, h->ctl, h->scal, h->dS, h->dschmidt, h->tv0, h->tv1,
                 h->mx_a32, h->mx_ut32, h->mx_w32, h->mx_perm32, h->mx_lam32, h->mx_info32, h->mx_Q, h->mx_Q2,
                 h->mx_B, h->mx_T, h->mx_V, h->mx_G, h->mx_w,
-                h->mx_W, h->mx_A32, h->mx_Li32, h->mx_t32, h->mx_d, h->mx_chst, h->mx_eosctl, h->mx_Q0};
+                h->mx_W, h->mx_A32, h->mx_Li32, h->mx_t32, h->mx_d, h->mx_chst, h->mx_eosctl, h->mx_rot, h->mx_Q0};
   for (void* p : ps) if (p) cudaFree(p);
   if (h->hs) cudaFreeHost(h->hs);
   free_oz(h->oz);
@@ -1818,8 +1856,8 @@ int mpo_svd(int r, int c, void* X, void* w, void* Ut, mpo_precision prec, int ma
                                      (float2*)jb, act, bj_state_ints(r), ctl, ms, 5.0, sms);
   else
     e = prec == MPO_FP64
-        ? launch_onesided<double>(st, (double2*)X, r, c, c, (double2*)Ut, (double*)w, ctl, ms, 5.0, sms)
-        : launch_onesided<float>(st, (float2*)X, r, c, c, (float2*)Ut, (float*)w, ctl, ms, 5.0, sms);
+        ? launch_row_jacobi<double>(st, (double2*)X, r, c, c, (double2*)Ut, (double*)w, ctl, ms, 5.0, sms)
+        : launch_row_jacobi<float>(st, (float2*)X, r, c, c, (float2*)Ut, (float*)w, ctl, ms, 5.0, sms);
   OSCtl hctl{};
   if (e == cudaSuccess) e = cudaMemcpyAsync(&hctl, ctl, sizeof(OSCtl), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -2051,14 +2089,20 @@ int mpo_eigh(int m, void* A, void* w, void* V, mpo_precision prec, int max_sweep
   if (cudaGetDevice(&dev) != cudaSuccess) return MPO_ERR_CUDA;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   GridCtl* ctl = nullptr;
-  if (cudaMalloc(&ctl, sizeof(GridCtl)) != cudaSuccess) return MPO_ERR_OOM;
+  void* rot = nullptr;
+  if (cudaMalloc(&ctl, sizeof(GridCtl)) != cudaSuccess || cudaMalloc(&rot, (size_t)(m + 1) * sizeof(JRot<double>)) != cudaSuccess) {
+    cudaGetLastError();
+    cudaFree(ctl);
+    return MPO_ERR_OOM;
+  }
   cudaError_t e = prec == MPO_FP64
-      ? launch_jacobi<double>(st, (double2*)A, m, (double2*)V, (double*)w, ctl, max_sweeps > 0 ? max_sweeps : 40, 5.0, sms)
-      : launch_jacobi<float>(st, (float2*)A, m, (float2*)V, (float*)w, ctl, max_sweeps > 0 ? max_sweeps : 40, 5.0, sms);
+      ? launch_jacobi<double>(st, (double2*)A, m, (double2*)V, (double*)w, (JRot<double>*)rot, ctl, max_sweeps > 0 ? max_sweeps : 40, 5.0, sms)
+      : launch_jacobi<float>(st, (float2*)A, m, (float2*)V, (float*)w, (JRot<float>*)rot, ctl, max_sweeps > 0 ? max_sweeps : 40, 5.0, sms);
   GridCtl hc{};
   if (e == cudaSuccess) e = cudaMemcpyAsync(&hc, ctl, sizeof(GridCtl), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   cudaFree(ctl);
+  cudaFree(rot);
   if (e != cudaSuccess) { g_last_init_error = cudaGetErrorString(e); return MPO_ERR_CUDA; }
   if (hc.err) return MPO_ERR_TIMEOUT;
   if (hc.status) return MPO_ERR_NOCONV;
