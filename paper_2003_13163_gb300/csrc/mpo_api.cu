@@ -77,6 +77,13 @@ struct OzWork {
   int e_cap = 0;
 };
 
+// Workspace of the LQ-preconditioned SVD: the reflectors (m x ccap), the
+// accumulated W (m x m), the reflectors' factors and first entries.
+struct LqWork {
+  double2 *z = nullptr, *w = nullptr, *zd = nullptr;
+  double* f = nullptr;
+};
+
 struct mpo_ctx {
   BatchState* batch = nullptr;     // set on handles made by mpo_init_batch
   int n = 0, chi_max = 0;
@@ -103,6 +110,7 @@ struct mpo_ctx {
   OSCtl* osctl = nullptr;          // control block of the Jacobi launches (barriers, status, counts)
   void *bj_gpart = nullptr, *bj_j = nullptr;   // block Jacobi partial Grams and pair rotations
   int* bj_act = nullptr;                        // block Jacobi integer state (bj_state_ints)
+  LqWork lq;                       // FP64 form; all NULL when it did not fit (then no LQ step)
   size_t bj_slots = 0, bj_act_ints = 0;
   int block_min_rows = 0;
   bool tensor_cores = false;       // FP32 plain products on tcgen05
@@ -324,7 +332,9 @@ static cudaError_t launch_onesided(cudaStream_t st, cplx<T>* X, int r, int c, in
 // cover rows of 1024 and 2048; longer rows are streamed.
 template <typename T>
 static cudaError_t launch_pair_jacobi(cudaStream_t st, cplx<T>* X, int r, int c, int ldx, cplx<T>* Ut, T* w, OSCtl* ctl,
-                                      int max_sweeps, double timeout_s, int num_sms, double tol_min = 0.0) {
+                                      int max_sweeps, double timeout_s, int num_sms, double tol_min = 0.0,
+                                      bool clear = true,
+                                      double floor = eps_of<T>::value * eps_of<T>::value) {
   constexpr int EL = sizeof(T) == 8 ? 8 : 16;
   const void* fn = std::max(r, c) <= 2 * OSJ_NT ? (const void*)pair_jacobi_kernel<T, 2> : (const void*)pair_jacobi_kernel<T, EL>;
   int per_sm = 0;
@@ -332,15 +342,47 @@ static cudaError_t launch_pair_jacobi(cudaStream_t st, cplx<T>* X, int r, int c,
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const int blocks = std::max(1, std::min(per_sm * num_sms, (r + 1) / 2));
-  e = cudaMemsetAsync(ctl, 0, sizeof(OSCtl), st);
+  if (clear) e = cudaMemsetAsync(ctl, 0, sizeof(OSCtl), st);
   if (e != cudaSuccess) return e;
   // rows count as orthogonal once |<x_p, x_q>| <= 2 eps sqrt(c) ||x_p|| ||x_q||,
   // the rounding level of the length-c dot product itself
   const T tol_rel = (T)std::max(tol_min, 2.0 * eps_of<T>::value * std::sqrt((double)std::max(c, 1)));
-  const T floor_rel = eps_of<T>::value * eps_of<T>::value;
+  const T floor_rel = (T)floor;
   long long timeout_ns = (long long)(timeout_s * 1e9);
   void* args[] = {&X, &r, &c, &ldx, &Ut, &w, &ctl, &max_sweeps, (void*)&tol_rel, (void*)&floor_rel, &timeout_ns};
   return cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(OSJ_NT), args, 0, st);
+}
+
+// Rows below which the LQ step costs more than the sweeps it saves.
+constexpr int kLqMinRows = 8;
+
+// X (r x c, r <= c) <- the rows Sigma V^H, vecs (r x r) <- rows conj(column of
+// U), w <- sigma^2 (lq_kernel). A barrier that timed out in the first kernel
+// leaves its error in ctl, which the Jacobi launch does not clear.
+static cudaError_t launch_lq_jacobi(cudaStream_t st, double2* X, int r, int c, int ldx, double2* vecs, double* w,
+                                    const LqWork& q, OSCtl* ctl, int max_sweeps, double timeout_s, int num_sms) {
+  const bool small = c <= 2 * OSJ_NT;
+  const void* fn = small ? (const void*)lq_kernel<2> : (const void*)lq_kernel<8>;
+  int per_sm = 0;
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, OSJ_NT, 0);
+  if (e != cudaSuccess) return e;
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  const int blocks = std::max(1, std::min(std::min(per_sm, 4) * num_sms, r));
+  e = cudaMemsetAsync(ctl, 0, sizeof(OSCtl), st);
+  if (e != cudaSuccess) return e;
+  long long timeout_ns = (long long)(timeout_s * 1e9);
+  LqWork k = q;
+  void* args[] = {&X, &ldx, &r, &c, &k.z, &vecs, &k.f, &k.zd, &ctl, &timeout_ns};
+  e = cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(OSJ_NT), args, 0, st);
+  if (e != cudaSuccess) return e;
+  // the columns of U come from the rows of the result, so these are made
+  // orthogonal relative to their own size down to 1e-14 of the largest each
+  // (a floor of eps^2 would leave pairs at 1e-11 coupled by 1e-10)
+  e = launch_pair_jacobi<double>(st, vecs, r, r, r, k.w, w, ctl, max_sweeps, timeout_s, num_sms, 0.0, false, 1e-44);
+  if (e != cudaSuccess) return e;
+  if (small) lq_apply_kernel<2><<<r, OSJ_NT, 0, st>>>(k.z, r, c, k.f, k.zd, k.w, vecs, w, X, ldx);
+  else lq_apply_kernel<8><<<r, OSJ_NT, 0, st>>>(k.z, r, c, k.f, k.zd, k.w, vecs, w, X, ldx);
+  return cudaGetLastError();
 }
 
 // The row-pair solver of a stand-alone form: complex128 by the CTA-per-pair
@@ -805,7 +847,13 @@ static int svd_select(mpo_ctx* h, cplx<T>* X, int r, int c, int ldx, int cap, bo
       CK(h, launch_block_jacobi<T>(h->st, X, r, c, ldx, (cplx<T>*)h->vecs, w, (cplx<T>*)h->bj_gpart, h->bj_slots,
                                    (cplx<T>*)h->bj_j, h->bj_act, h->bj_act_ints, h->osctl, h->opts.eig_max_sweeps,
                                    h->opts.barrier_timeout_s, h->num_sms));
-    else
+    else if (h->lq.z && r >= kLqMinRows && r <= c) {
+      if constexpr (std::is_same<T, double>::value) {
+        CK(h, launch_lq_jacobi(h->st, X, r, c, ldx, (double2*)h->vecs, w, h->lq, h->osctl, h->opts.eig_max_sweeps,
+                               h->opts.barrier_timeout_s, h->num_sms));
+        h->vecs_conj = true;
+      }
+    } else
       CK(h, launch_row_jacobi<T>(h->st, X, r, c, ldx, (cplx<T>*)h->vecs, w, h->osctl, h->opts.eig_max_sweeps,
                                  h->opts.barrier_timeout_s, h->num_sms));
   }
@@ -1419,6 +1467,26 @@ static bool alloc_factor_ws(mpo_ctx* h, int m, int ccap, size_t bj_nch) {
   return ok;
 }
 
+// Workspace of the FP64 form's LQ step. It only saves time, so a handle whose
+// memory limit (arena_cap_bytes: `room` bytes left) or device has no room for
+// it goes without.
+static void alloc_lq(mpo_ctx* h, int m, int ccap, size_t room) {
+  if (h->prec != MPO_FP64) return;
+  const size_t z = (size_t)m * ccap * sizeof(double2), w = (size_t)m * m * sizeof(double2);
+  const size_t sum = z + w + (size_t)m * (sizeof(double2) + sizeof(double));
+  size_t freeb = 0, totb = 0;
+  if (sum > room || cudaMemGetInfo(&freeb, &totb) != cudaSuccess || sum > freeb) { cudaGetLastError(); return; }
+  LqWork q;
+  const size_t before = h->bytes;
+  if (ws_alloc(h, (void**)&q.z, z) && ws_alloc(h, (void**)&q.w, w) && ws_alloc(h, (void**)&q.zd, (size_t)m * sizeof(double2)) &&
+      ws_alloc(h, (void**)&q.f, (size_t)m * sizeof(double))) {
+    h->lq = q;
+    return;
+  }
+  cudaFree(q.z); cudaFree(q.w); cudaFree(q.zd); cudaFree(q.f);
+  h->bytes = before;
+}
+
 int mpo_init(mpo_handle* out, int n, int chi_max, mpo_precision prec, void* stream, const mpo_opts* opts) {
   if (!out) { g_last_init_error = "out is NULL"; return MPO_ERR_ARG; }
   *out = nullptr;
@@ -1526,6 +1594,7 @@ int mpo_init(mpo_handle* out, int n, int chi_max, mpo_precision prec, void* stre
   ok = ok && alloc((void**)&h->tv0, (size_t)(chi_max + 1) * sizeof(double2));
   ok = ok && alloc((void**)&h->tv1, (size_t)(chi_max + 1) * sizeof(double2));
   if (!ok) return init_fail(h, MPO_ERR_OOM, "cudaMalloc failed");
+  alloc_lq(h, m, mx_ccap, h->opts.arena_cap_bytes > 0 ? h->opts.arena_cap_bytes - need : ~(size_t)0);
   if (cudaMallocHost((void**)&h->hs, sizeof(HostSync)) != cudaSuccess) {
     cudaGetLastError();
     h->hs = nullptr;
@@ -1565,6 +1634,7 @@ void mpo_free(mpo_handle h) {
   if (h->batch) { batch_free(h); return; }
   for (void* p : h->site) if (p) cudaFree(p);
   void* ps[] = {h->spare, h->theta, h->theta2, h->osctl, h->tc_status, h->bj_gpart, h->bj_j, h->bj_act, h->vecs, h->tmp, h->wv, h->perm, h->lam2, h->Ms, h->dgates,
+                h->lq.z, h->lq.w, h->lq.zd, h->lq.f,
                 h->dsup, h->dp, h->info, h->ctl, h->scal, h->dS, h->dschmidt, h->tv0, h->tv1,
                 h->mx_a32, h->mx_ut32, h->mx_w32, h->mx_perm32, h->mx_lam32, h->mx_info32, h->mx_Q, h->mx_Q2,
                 h->mx_B, h->mx_T, h->mx_V, h->mx_G, h->mx_w,
@@ -1906,6 +1976,7 @@ int mpo_svd_truncated(int r, int c, const void* A, int cap, mpo_precision prec, 
   if (ok && h->use_oz) ok = alloc_oz(h->oz, c, &h->bytes);
   if (ok && cudaMallocHost((void**)&h->hs, sizeof(HostSync)) != cudaSuccess) { cudaGetLastError(); h->hs = nullptr; ok = false; }
   if (!ok) { mpo_free(h); g_last_init_error = "mpo_svd_truncated: allocation failed"; return MPO_ERR_OOM; }
+  alloc_lq(h, r, c, h->opts.arena_cap_bytes > 0 ? 0 : ~(size_t)0);
   int rc = MPO_OK, kk = 0;
   auto ck = [&](cudaError_t e) { if (rc == MPO_OK && e != cudaSuccess) { rc = MPO_ERR_CUDA; g_last_init_error = cudaGetErrorString(e); } };
   ck(cudaMemcpyAsync(h->theta, A, (size_t)r * c * h->esz, cudaMemcpyDeviceToDevice, h->st));
