@@ -467,30 +467,28 @@ static cudaError_t oz_gemm(cudaStream_t st, int M, int N, int K, const double2* 
                            int ldb, int opB, double2* C, int ldc, double alpha, int accumulate, const OzWork& w,
                            double timeout_s, int num_sms) {
   if (M <= 0 || N <= 0) return cudaSuccess;
-  const int K8 = (std::max(K, 1) + 31) / 32 * 32;
+  const int nkb = (std::max(K, 1) + 15) / 16;
   const int Mp = (M + oz::BM - 1) / oz::BM * oz::BM, Nrp = (2 * N + oz::BN - 1) / oz::BN * oz::BN;
-  const size_t Kp = 2 * (size_t)K8;
+  const size_t Kp = 32 * (size_t)nkb;
   if ((size_t)oz::S * Mp * Kp > w.a_cap || (size_t)oz::S * Nrp * Kp > w.b_cap || Mp > w.e_cap || Nrp / 2 > w.e_cap)
     return cudaErrorInvalidValue;
-  // scaling exponents: rows of op(A) are stored rows of A (op 0) or stored
-  // columns (op 1); columns of op(B) are stored columns of B (op 0) or rows
-  cudaError_t e0 = cudaMemsetAsync(w.ea, 0, sizeof(int) * (size_t)M, st);
-  if (e0 == cudaSuccess) e0 = cudaMemsetAsync(w.eb, 0, sizeof(int) * (size_t)N, st);
-  if (e0 != cudaSuccess) return e0;
-  {
-    const int Ra = opA ? K : M, Ca = opA ? M : K, Rb = opB ? N : K, Cb = opB ? K : N;
-    oz_exp_kernel<<<dim3((Ca + 31) / 32, (Ra + 255) / 256), dim3(32, 8), 0, st>>>(A, lda, Ra, Ca, opA ? 0 : 1, w.ea);
-    oz_exp_kernel<<<dim3((Cb + 31) / 32, (Rb + 255) / 256), dim3(32, 8), 0, st>>>(B, ldb, Rb, Cb, opB ? 1 : 0, w.eb);
-  }
-  oz_split_a_kernel<<<dim3(K8 / 32, Mp / 32), dim3(32, 8), 0, st>>>(A, lda, opA, M, K, K8, Mp, w.ea, w.a);
-  oz_split_b_kernel<<<dim3(K8 / 32, Nrp / 64), dim3(32, 8), 0, st>>>(B, ldb, opB, K, N, K8, Nrp, w.eb, w.b);
-  cudaError_t e = cudaGetLastError();
+  const OzOp a{A, lda, opA, M, w.ea, w.a}, b{B, ldb, opB, N, w.eb, w.b};
+  // scaling exponents (eb follows ea in one allocation), then the slices: one
+  // launch each for both operands
+  cudaError_t e = cudaMemsetAsync(w.ea, 0, sizeof(int) * ((size_t)w.e_cap + N), st);
+  if (e != cudaSuccess) return e;
+  auto scans = [&](int rows, int cols) { return ((cols + 31) / 32) * ((rows + 255) / 256); };
+  const int na = opA ? scans(K, M) : scans(M, K), nb = opB ? scans(N, K) : scans(K, N);
+  oz_exp_kernel<<<na + nb, dim3(32, 8), 0, st>>>(a, b, K, na);
+  const int sa = nkb * (Mp / 32), sb = nkb * (Nrp / 32);
+  oz_split_kernel<<<sa + sb, 128, 0, st>>>(a, b, K, nkb, sa);
+  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   e = ensure_dynamic_smem((const void*)oz_mma_kernel, oz::SMEM_BYTES);
   if (e != cudaSuccess) return e;
-  oz_mma_kernel<<<dim3(Nrp / oz::BN, Mp / oz::BM), oz::NT, oz::SMEM_BYTES, st>>>(
-      M, N, (int)Kp, w.a, (size_t)Mp * Kp, w.b, (size_t)Nrp * Kp, w.ea, w.eb, C, ldc, alpha, accumulate, w.status,
-      (long long)(timeout_s * 1e9));
+  const OzTiles tl{Mp / oz::BM, Nrp / oz::BN, nkb};
+  oz_mma_kernel<<<std::min(num_sms, tl.nrb * tl.ncb), oz::NT, oz::SMEM_BYTES, st>>>(tl, a, b, C, ldc, alpha, accumulate,
+                                                                                  w.status, (long long)(timeout_s * 1e9));
   return cudaGetLastError();
 }
 
@@ -505,17 +503,19 @@ static bool alloc_oz(OzWork& w, int dmax, size_t* bytes) {
   w.e_cap = (int)std::max(Mp, Nrp);
   bool ok = cudaMalloc((void**)&w.a, w.a_cap * sizeof(__nv_bfloat16)) == cudaSuccess &&
             cudaMalloc((void**)&w.b, w.b_cap * sizeof(__nv_bfloat16)) == cudaSuccess &&
-            cudaMalloc((void**)&w.ea, w.e_cap * sizeof(int)) == cudaSuccess &&
-            cudaMalloc((void**)&w.eb, w.e_cap * sizeof(int)) == cudaSuccess &&
-            cudaMalloc((void**)&w.status, sizeof(int)) == cudaSuccess &&
-            cudaMemset(w.status, 0, sizeof(int)) == cudaSuccess;
+            cudaMalloc((void**)&w.ea, (2 * (size_t)w.e_cap + 1) * sizeof(int)) == cudaSuccess &&
+            cudaMemset(w.ea + 2 * (size_t)w.e_cap, 0, sizeof(int)) == cudaSuccess;
   if (!ok) cudaGetLastError();
+  if (w.ea) {                      // one allocation: exponents of A, of B, status
+    w.eb = w.ea + w.e_cap;
+    w.status = w.ea + 2 * (size_t)w.e_cap;
+  }
   if (bytes) *bytes += (w.a_cap + w.b_cap) * sizeof(__nv_bfloat16) + 2 * w.e_cap * sizeof(int);
   return ok;
 }
 
 static void free_oz(OzWork& w) {
-  cudaFree(w.a); cudaFree(w.b); cudaFree(w.ea); cudaFree(w.eb); cudaFree(w.status);
+  cudaFree(w.a); cudaFree(w.b); cudaFree(w.ea);
   w = OzWork();
 }
 

@@ -27,43 +27,58 @@
 // every level is drained to double-float (hi, lo) FP32 registers; the tile's
 // value (hi + lo) 2^{e_i + f_j} is formed in FP64 once at the end.
 //
-// One CTA computes a 128 x 64 real tile (128 rows x 32 complex columns) with
-// S 64-column FP32 accumulators (512 TMEM columns allocated). Operand slices are
-// staged by cp.async into the K-major no-swizzle core-matrix layout (8 rows x
-// 16 bytes per core matrix, SBO = 128 B between 8-row groups, LBO = rows x
-// 16 B between the K groups of 8), two stages of 32 real K; one thread
-// issues tcgen05.mma (kind::f16, BF16 inputs, FP32 accumulate, M = 128,
-// N = 64) and commits each stage to an mbarrier; every wait is bounded.
+// Operand layout. The split kernels write the slices in the order in which the
+// MMA kernel reads them: one stage is 16 complex k, its real parts, then (the
+// next stage) its imaginary parts, 16 real K each, in the K-major no-swizzle
+// core-matrix layout (8 rows x 16 bytes per core matrix, SBO = 128 B between
+// 8-row groups, LBO between the two K groups of 8):
+//   A: [row block of 128][stage][slice][K group][128 rows][8]   24 KB per stage
+//   B: [column block of 64][stage][K group][slice][64 rows][8]  12 KB per stage
+// so a stage is three bulk copies, and the slices of B follow one another as
+// rows: one MMA multiplies an A slice by two neighbouring B slices (N = 128).
+//
+// Accumulators. Level t + u of a slice pair has 64 TMEM columns; pairs of
+// levels (2p, 2p + 1) are the fixed 128-column accumulators, so every MMA on an
+// accumulator has the same shape and they execute in issue order. A slice of
+// odd index meets the pair that starts one level lower with a zero slice
+// ahead of B's first one in shared memory: 12 MMAs (24 slice products, 3 of
+// them zero) per 16 real K. With N = 64, one product each, the A operand is
+// read from shared memory 21 times instead of 12, more than its bandwidth.
+//
+// A persistent CTA (grid <= SMs) walks over 128 x 64 real tiles (128 rows x 32
+// complex columns): one warp issues the bulk copies (five stages ahead), one
+// thread the MMAs, eight warps drain the accumulators and write C, so the
+// copies of the next tile run under the epilogue of this one. Every wait is
+// bounded.
+// What bounds it: shared memory bandwidth. A stage of 16 real K takes 768 clocks
+// of the tensor pipe, but the MMAs read 96 KB and the copies write 36 KB of
+// shared memory for it (1056 clocks at 128 B). 4096 x 2048 x 4096: 13.75 ms
+// with cp.async loads one stage ahead and N = 64 MMAs, 4.92 ms now (tensor pipe
+// 54 % active, 55.9 TFLOP/s of FP64-accurate work, L2 reads 7.9 TB/s).
 #pragma once
 #include <cuda_bf16.h>
 #include "common.cuh"
 #include "tcgemm.cuh"
 
-// 16 consecutive 32-bit TMEM columns of this warp's 32 lanes -> v[base .. base + 15]
-#define OZ_LD16(v, base, taddr)                                                                               \
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];" \
-               : "=r"(v[base + 0]), "=r"(v[base + 1]), "=r"(v[base + 2]), "=r"(v[base + 3]),                 \
-                 "=r"(v[base + 4]), "=r"(v[base + 5]), "=r"(v[base + 6]), "=r"(v[base + 7]),                 \
-                 "=r"(v[base + 8]), "=r"(v[base + 9]), "=r"(v[base + 10]), "=r"(v[base + 11]),               \
-                 "=r"(v[base + 12]), "=r"(v[base + 13]), "=r"(v[base + 14]), "=r"(v[base + 15])              \
-               : "r"(taddr))
-
 namespace oz {
 constexpr int S = 6;                         // slices per operand (about 43 bits)
 constexpr int BM = 128, BN = 64;             // real tile: 128 rows x 64 real (32 complex) columns
-constexpr int KS = 32;                       // real K per stage (two MMAs of K = 16)
-constexpr int KC = 256;                      // real K per exact chunk
+constexpr int KS = 16;                       // real K per stage: one MMA deep
+// real K per exact chunk: a level's products sum to at most 2^15 units per K
+// (|a_1| <= 128, |a_t| <= 64: 2 * 2^13 + 4 * 2^12 at level 7), 2^24 per chunk
+constexpr int KC = 512;
 constexpr int SPC = KC / KS;                 // stages per chunk
-constexpr int A_SLICE = BM * KS * 2;         // 8 KB: one A slice, 128 rows x 32 K
-constexpr int B_SLICE = BN * KS * 2;         // 4 KB: one B slice, 64 rows x 32 K
-constexpr int A_LBO = BM * 16, B_LBO = BN * 16;   // bytes between the K groups of 8
-constexpr int B_OFF = S * A_SLICE;           // B slices follow the A slices in a stage
-constexpr int STAGE_BYTES = S * (A_SLICE + B_SLICE);   // 72 KB
-constexpr int SMEM_BYTES = 2 * STAGE_BYTES + 1024;
-constexpr int NT = 512;                      // 16 warps: 4 TMEM lane groups x 4 column groups of 16
-constexpr int NACC = S;                      // one accumulator per level L = 2 .. S + 1
-constexpr int TCOLS = 512;                   // TMEM allocation (power of two >= NACC * BN)
-static_assert(NACC * BN <= TCOLS, "accumulators exceed the TMEM allocation");
+constexpr int A_STAGE = S * 2 * BM * 16;     // 24 KB in global and shared memory
+constexpr int B_STAGE = 2 * S * BN * 16;     // 12 KB in global memory
+constexpr int B_KG = (S + 1) * BN * 16;      // one K group of B in shared memory, zero slice first
+constexpr int STAGE_BYTES = A_STAGE + 2 * B_KG;
+constexpr int NSTAGE = 5;
+constexpr int SMEM_BYTES = NSTAGE * STAGE_BYTES + 1024;
+constexpr int A_LBO = BM * 16;               // byte step between the K groups of 8
+constexpr int NDRAIN = 8;                    // drain warps: 4 TMEM lane groups x 2 column halves
+constexpr int NT = 32 * (NDRAIN + 2);
+constexpr int TCOLS = 512;                   // TMEM allocation (power of two >= S * BN)
+static_assert(S * BN <= TCOLS, "accumulators exceed the TMEM allocation");
 
 // Shared-memory matrix descriptor, K-major, no swizzle: start address, LBO
 // (byte step between the core matrices of consecutive K groups), SBO = 128 B
@@ -86,24 +101,38 @@ __device__ __forceinline__ uint64_t desc(uint32_t addr, uint32_t lbo) {
 __device__ __forceinline__ int oz_ex(int raw) { return raw > 0 ? raw - 1022 : 0; }
 __device__ __forceinline__ int oz_bexp(double v) { return (int)((__double_as_longlong(v) >> 52) & 0x7FF); }
 
-// The stored matrix (R rows x C columns, leading dimension ld) is scanned in
-// 32-column x 256-row tiles, block (32, 8); by_row = 1 reduces along each
-// stored row (raw indexed by stored row), 0 along each stored column (raw
-// indexed by stored column). One atomic per warp-row or per tile column.
-__global__ void oz_exp_kernel(const double2* __restrict__ X, int ld, int R, int C, int by_row, int* __restrict__ raw) {
+// One operand of a product: the stored matrix, its form and its slices.
+struct OzOp {
+  const double2* X;
+  int ld, op;        // op 0: as stored, 1: conjugate transpose
+  int n;             // rows of op(A) / columns of op(B)
+  int* raw;          // exponents
+  __nv_bfloat16* sl;
+};
+
+// The stored matrices (R rows x C columns) are scanned in 32-column x 256-row
+// tiles, block (32, 8); by_row = 1 reduces along each stored row (raw indexed by
+// stored row), 0 along each stored column. One atomic per warp-row or per
+// tile column. Blocks below na scan A, the rest B.
+__global__ void oz_exp_kernel(OzOp a, OzOp b, int K, int na) {
   __shared__ int red[8][33];
-  const int c = blockIdx.x * 32 + threadIdx.x, r0 = blockIdx.y * 256, ty = threadIdx.y;
+  const bool isB = (int)blockIdx.x >= na;
+  const OzOp o = isB ? b : a;
+  const int by_row = isB ? o.op : 1 - o.op;              // the K index runs along the stored row
+  const int R = by_row ? o.n : K, C = by_row ? K : o.n;
+  const int id = isB ? blockIdx.x - na : blockIdx.x, nx = (C + 31) / 32;
+  const int c = (id % nx) * 32 + threadIdx.x, r0 = (id / nx) * 256, ty = threadIdx.y;
   int mcol = 0;
   for (int r = r0 + ty; r < min(R, r0 + 256); r += 8) {
     int v = 0;
     if (c < C) {
-      const double2 x = X[(size_t)r * ld + c];
+      const double2 x = o.X[(size_t)r * o.ld + c];
       v = max(oz_bexp(x.x), oz_bexp(x.y));
     }
     if (by_row) {
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-      if (threadIdx.x == 0 && v > 0) atomicMax(&raw[r], v);
+      for (int s = 16; s > 0; s >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, s));
+      if (threadIdx.x == 0 && v > 0) atomicMax(&o.raw[r], v);
     } else {
       mcol = max(mcol, v);
     }
@@ -115,7 +144,7 @@ __global__ void oz_exp_kernel(const double2* __restrict__ X, int ld, int R, int 
       int v = red[0][threadIdx.x];
 #pragma unroll
       for (int i = 1; i < 8; ++i) v = max(v, red[i][threadIdx.x]);
-      if (c < C && v > 0) atomicMax(&raw[c], v);
+      if (c < C && v > 0) atomicMax(&o.raw[c], v);
     }
   }
 }
@@ -147,81 +176,60 @@ __device__ __forceinline__ void oz_slices(double v, int ex, float* out) {
   out[0] = __int2float_rn((int)n) * __int_as_float((127 - 7) << 23);
 }
 
-// Slices of op(A)' = [Re | Im] into Asl[t][i][c] (S x Mp x Kp, row-major,
-// Kp = 2 K8): c < K8 real parts, K8 <= c < 2 K8 imaginary parts; zero
-// outside M x K. Tiles of 32 rows x 32 K through shared memory so that
-// both the reads (either op) and the writes are coalesced. grid (K8/32, Mp/32), block (32, 8).
-__global__ void oz_split_a_kernel(const double2* __restrict__ A, int lda, int op, int M, int K, int K8, int Mp,
-                                  const int* __restrict__ e, __nv_bfloat16* __restrict__ Asl) {
-  __shared__ double2 tile[32][33];
-  const int i0 = blockIdx.y * 32, k0 = blockIdx.x * 32, tx = threadIdx.x, ty = threadIdx.y;
-  for (int r = ty; r < 32; r += 8) {
+// Slices of both operands in the stage layout above, zero outside the matrix.
+// One block of 128 threads takes 16 complex k (both stages) of 32 rows of
+// op(A), or of 16 columns of op(B): the 32 interleaved rows 2j = [Re b_j |
+// -Im b_j], 2j + 1 = [Im b_j | Re b_j]. Through shared memory, so that either
+// form is read coalesced; a thread then forms 8 K values of one row and stage
+// and writes 16 bytes per slice, 512 consecutive bytes per warp. Blocks below
+// na take A (nka = stages / 2 blocks per 32 rows), the rest B.
+__global__ void __launch_bounds__(128) oz_split_kernel(OzOp a, OzOp b, int K, int nkb, int na) {
+  __shared__ double2 tile[32][17];
+  const bool isB = (int)blockIdx.x >= na;
+  const OzOp o = isB ? b : a;
+  const int id = isB ? blockIdx.x - na : blockIdx.x, kb = id % nkb, rb = id / nkb;
+  const int tid = threadIdx.x, k0 = kb * 16, i0 = rb * (isB ? 16 : 32), ni = isB ? 16 : 32;
+  const bool along = isB ? o.op == 1 : o.op == 0;   // k runs along the stored row
+  for (int e = tid; e < ni * 16; e += 128) {
+    const int i = along ? e >> 4 : e % ni, k = along ? e & 15 : e / ni;
     double2 v = make_double2(0.0, 0.0);
-    if (op == 0) {                       // tile[i][k] from row i0 + r
-      const int i = i0 + r, k = k0 + tx;
-      if (i < M && k < K) v = A[(size_t)i * lda + k];
-      tile[r][tx] = v;
-    } else {                             // tile[i][k] = conj(A[k][i]) from row k0 + r of A
-      const int k = k0 + r, i = i0 + tx;
-      if (i < M && k < K) { v = A[(size_t)k * lda + i]; v.y = -v.y; }
-      tile[tx][r] = v;
+    if (i0 + i < o.n && k0 + k < K) {
+      v = along ? o.X[(size_t)(i0 + i) * o.ld + k0 + k] : o.X[(size_t)(k0 + k) * o.ld + i0 + i];
+      if (o.op) v.y = -v.y;
     }
+    tile[i][k] = v;
   }
   __syncthreads();
-  const size_t Kp = 2 * (size_t)K8, sstride = (size_t)Mp * Kp;
-  for (int r = ty; r < 32; r += 8) {
-    const int i = i0 + r, k = k0 + tx;
-    const double2 v = tile[r][tx];
-    const int ex = i < M ? oz_ex(e[i]) : 0;
-    float sr[oz::S], si[oz::S];
-    oz_slices(v.x, ex, sr);
-    oz_slices(v.y, ex, si);
+  const int q = tid & 31, cg = (tid >> 5) & 1, im = tid >> 6;   // row, K group of 8, stage
+  const int i = isB ? q >> 1 : q;
+  const int ex = i0 + i < o.n ? oz_ex(o.raw[i0 + i]) : 0;
+  const bool take_im = isB ? ((q & 1) != im) : im != 0;         // B: even rows [Re, -Im], odd rows [Im, Re]
+  const float sign = isB && im && !(q & 1) ? -1.0f : 1.0f;
+  uint32_t pk[oz::S][4];
+#pragma unroll
+  for (int h = 0; h < 4; ++h) {
+    float s0[oz::S], s1[oz::S];
+    const double2 v0 = tile[i][8 * cg + 2 * h], v1 = tile[i][8 * cg + 2 * h + 1];
+    oz_slices(take_im ? v0.y : v0.x, ex, s0);
+    oz_slices(take_im ? v1.y : v1.x, ex, s1);
 #pragma unroll
     for (int t = 0; t < oz::S; ++t) {
-      Asl[t * sstride + (size_t)i * Kp + k] = __float2bfloat16_rn(sr[t]);
-      Asl[t * sstride + (size_t)i * Kp + K8 + k] = __float2bfloat16_rn(si[t]);
+      const __nv_bfloat162 p2 = __floats2bfloat162_rn(sign * s0[t], sign * s1[t]);
+      pk[t][h] = *reinterpret_cast<const uint32_t*>(&p2);
     }
   }
-}
-
-// Slices of the interleaved rows of op(B)'^T into Bsl[t][q][c] (S x Nrp x Kp):
-// row 2j = [Re b_j | -Im b_j], row 2j + 1 = [Im b_j | Re b_j] (b_j = column j
-// of op(B)); zero outside. grid (K8/32, Nrp/64), block (32, 8): 32 complex
-// columns (64 rows of Bsl) x 32 K per CTA.
-__global__ void oz_split_b_kernel(const double2* __restrict__ B, int ldb, int op, int K, int N, int K8, int Nrp,
-                                  const int* __restrict__ f, __nv_bfloat16* __restrict__ Bsl) {
-  __shared__ double2 tile[32][33];   // tile[j][k]
-  const int j0 = blockIdx.y * 32, k0 = blockIdx.x * 32, tx = threadIdx.x, ty = threadIdx.y;
-  for (int r = ty; r < 32; r += 8) {
-    double2 v = make_double2(0.0, 0.0);
-    if (op == 0) {                       // row k0 + r of B holds op(B)[k][j0 + tx]
-      const int k = k0 + r, j = j0 + tx;
-      if (j < N && k < K) v = B[(size_t)k * ldb + j];
-      tile[tx][r] = v;
-    } else {                             // op(B)[k][j] = conj(B[j][k]): row j0 + r of B
-      const int j = j0 + r, k = k0 + tx;
-      if (j < N && k < K) { v = B[(size_t)j * ldb + k]; v.y = -v.y; }
-      tile[r][tx] = v;
-    }
-  }
-  __syncthreads();
-  const size_t Kp = 2 * (size_t)K8, sstride = (size_t)Nrp * Kp;
-  for (int r = ty; r < 32; r += 8) {
-    const int j = j0 + r, k = k0 + tx;
-    const double2 v = tile[r][tx];
-    const int ex = j < N ? oz_ex(f[j]) : 0;
-    float sr[oz::S], si[oz::S];
-    oz_slices(v.x, ex, sr);
-    oz_slices(v.y, ex, si);
-    const size_t q0 = (size_t)(2 * j) * Kp, q1 = (size_t)(2 * j + 1) * Kp;
+  unsigned char* base = reinterpret_cast<unsigned char*>(o.sl);
+  const int stage = 2 * kb + im;
+  if (!isB) {
+    base += ((size_t)(rb >> 2) * (2 * nkb) + stage) * oz::A_STAGE + cg * oz::A_LBO + ((rb & 3) * 32 + q) * 16;
 #pragma unroll
-    for (int t = 0; t < oz::S; ++t) {
-      __nv_bfloat16* base = Bsl + t * sstride;
-      base[q0 + k] = __float2bfloat16_rn(sr[t]);
-      base[q0 + K8 + k] = __float2bfloat16_rn(-si[t]);
-      base[q1 + k] = __float2bfloat16_rn(si[t]);
-      base[q1 + K8 + k] = __float2bfloat16_rn(sr[t]);
-    }
+    for (int t = 0; t < oz::S; ++t)
+      *reinterpret_cast<uint4*>(base + t * 2 * oz::A_LBO) = make_uint4(pk[t][0], pk[t][1], pk[t][2], pk[t][3]);
+  } else {
+    base += ((size_t)(rb >> 1) * (2 * nkb) + stage) * oz::B_STAGE + cg * (oz::B_STAGE / 2) + ((rb & 1) * 32 + q) * 16;
+#pragma unroll
+    for (int t = 0; t < oz::S; ++t)
+      *reinterpret_cast<uint4*>(base + t * oz::BN * 16) = make_uint4(pk[t][0], pk[t][1], pk[t][2], pk[t][3]);
   }
 }
 
@@ -235,152 +243,200 @@ __device__ __forceinline__ void df_add(float& hi, float& lo, float x) {
   lo = __fadd_rn(lo, err);
 }
 
-// grid (Nrp / 64, Mp / 128), 512 threads, dynamic smem oz::SMEM_BYTES.
-// Kp: real K (2 K8), a multiple of oz::KS. status: set to 1 if an mbarrier
-// wait ran past timeout_ns (the tile is then left unwritten).
-__global__ void __launch_bounds__(512, 1) oz_mma_kernel(int M, int N, int Kp, const __nv_bfloat16* __restrict__ Asl,
-                                                        size_t a_sstride, const __nv_bfloat16* __restrict__ Bsl,
-                                                        size_t b_sstride, const int* __restrict__ eA,
-                                                        const int* __restrict__ eB, double2* __restrict__ C, int ldc,
-                                                        double alpha, int accumulate, int* status, long long timeout_ns) {
+// The tile list of a product. Row blocks go in groups of 16 and the column
+// blocks of a group in turn, so the tiles in flight at one time share their
+// operands in L2.
+struct OzTiles {
+  int nrb, ncb, nkb;      // row blocks, column blocks, blocks of 16 complex k
+  __device__ __forceinline__ int count() const { return nrb * ncb; }
+  __device__ __forceinline__ void tile(int id, int& rb, int& cb) const {
+    const int per = 16 * ncb, g = id / per, h = min(16, nrb - 16 * g), w = id - g * per;
+    rb = 16 * g + w % h;
+    cb = w / h;
+  }
+  __device__ __forceinline__ int stages(int) const { return 2 * nkb; }
+};
+
+#define OZ_LD32(v, taddr)                                                                                      \
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15," \
+               "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"                      \
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),           \
+                 "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),       \
+                 "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]),    \
+                 "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]),    \
+                 "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])                                            \
+               : "r"(taddr))
+
+// grid <= SMs, oz::NT threads, dynamic smem oz::SMEM_BYTES. status: set to 1 if
+// an mbarrier wait ran past timeout_ns (the CTA's remaining tiles are then left
+// unwritten).
+__global__ void __launch_bounds__(oz::NT, 1) oz_mma_kernel(OzTiles tl, OzOp a, OzOp b, double2* __restrict__ C, int ldc,
+                                                           double alpha, int accumulate, int* status,
+                                                           long long timeout_ns) {
   using namespace oz;
   extern __shared__ __align__(1024) unsigned char oz_raw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>(((uintptr_t)oz_raw + 1023) & ~(uintptr_t)1023);
-  __shared__ __align__(8) uint64_t bars[3];   // [0], [1]: stage buffers; [2]: chunk drained-ready
+  __shared__ __align__(8) uint64_t full[NSTAGE], empty[NSTAGE], acc_full, acc_empty;
   __shared__ uint32_t tmem_base;
   __shared__ int s_fail;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int row0 = blockIdx.y * BM, rcol0 = blockIdx.x * BN;
-  const int lg = warp & 3, cg = warp >> 2;   // TMEM lane group (rows 32 lg ..), accumulator column group
 
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(tcg::saddr(&tmem_base)), "n"(TCOLS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (tid == 0) {
-    for (int b = 0; b < 3; ++b) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(tcg::saddr(&bars[b])));
+    for (int i = 0; i < NSTAGE; ++i) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(tcg::saddr(&full[i])));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(tcg::saddr(&empty[i])));
+    }
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(tcg::saddr(&acc_full)));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(tcg::saddr(&acc_empty)), "n"(NDRAIN));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     s_fail = 0;
   }
+  // the zero slice ahead of B's first one, in both K groups of every stage
+  for (int e = tid; e < NSTAGE * 2 * BN; e += NT) {
+    unsigned char* z = sm + (e / (2 * BN)) * STAGE_BYTES + A_STAGE + ((e / BN) & 1) * B_KG + (e % BN) * 16;
+    *reinterpret_cast<uint4*>(z) = make_uint4(0, 0, 0, 0);
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tbase = tmem_base;
-  // kind::f16 instruction descriptor: D FP32 (bit 4), A and B BF16 (bits 7, 10), K-major, N >> 3, M >> 4
-  const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+  const int ntiles = tl.count();
+  volatile int* fail = &s_fail;
 
-  const int nst = Kp / KS;
-  // A stage holds, per slice, the 128 A rows and the 64 B rows of 32 real K
-  // as 16-byte pieces (row, K group c) in the core-matrix layout.
-  auto load_stage = [&](int s) {
-    const uint32_t st = tcg::saddr(sm) + (uint32_t)((s & 1) * STAGE_BYTES);
-    const size_t k0 = (size_t)s * KS;
-    for (int q = tid; q < S * (BM + BN) * 4; q += NT) {
-      const int c = q & 3, rr = q >> 2;            // rr over S x (BM + BN) rows
-      const int t = rr / (BM + BN), r = rr % (BM + BN);
-      const bool isA = r < BM;
-      const int rb = isA ? r : r - BM;
-      const __nv_bfloat16* src = isA ? Asl + (size_t)t * a_sstride + (size_t)(row0 + rb) * Kp
-                                     : Bsl + (size_t)t * b_sstride + (size_t)(rcol0 + rb) * Kp;
-      src += k0 + 8 * c;
-      const uint32_t dst = st + (isA ? t * A_SLICE + c * A_LBO : B_OFF + t * B_SLICE + c * B_LBO) +
-                           (rb >> 3) * 128 + (rb & 7) * 16;
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" :: "r"(dst), "l"(src) : "memory");
+  if (warp == NDRAIN) {
+    // ---- producer: three bulk copies per stage --------------------------
+    if (lane == 0) {
+      int it = 0;
+      bool ok = true;
+      for (int id = blockIdx.x; id < ntiles && ok; id += gridDim.x) {
+        int rb, cb;
+        tl.tile(id, rb, cb);
+        const int nst = tl.stages(cb);
+        const unsigned char* pa = reinterpret_cast<const unsigned char*>(a.sl) + (size_t)rb * 2 * tl.nkb * A_STAGE;
+        const unsigned char* pb = reinterpret_cast<const unsigned char*>(b.sl) + (size_t)cb * 2 * tl.nkb * B_STAGE;
+        for (int s = 0; s < nst; ++s, ++it) {
+          const int slot = it % NSTAGE;
+          if (it >= NSTAGE && !tcg::wait_parity(tcg::saddr(&empty[slot]), (uint32_t)(it / NSTAGE - 1) & 1u, timeout_ns)) ok = false;
+          if (!ok || *fail) { ok = false; break; }
+          const uint32_t st = tcg::saddr(sm + slot * STAGE_BYTES), bar = tcg::saddr(&full[slot]);
+          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(bar), "n"(A_STAGE + B_STAGE) : "memory");
+          asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                       :: "r"(st), "l"(pa + (size_t)s * A_STAGE), "n"(A_STAGE), "r"(bar) : "memory");
+#pragma unroll
+          for (int g = 0; g < 2; ++g)
+            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                         :: "r"(st + A_STAGE + g * B_KG + BN * 16), "l"(pb + (size_t)s * B_STAGE + g * (B_STAGE / 2)),
+                            "n"(B_STAGE / 2), "r"(bar) : "memory");
+        }
+      }
+      if (!ok) s_fail = 1;
+      // copies still in flight land before the CTA may end
+      for (int j = max(0, it - NSTAGE); j < it; ++j)
+        (void)tcg::wait_parity(tcg::saddr(&full[j % NSTAGE]), (uint32_t)(j / NSTAGE) & 1u, timeout_ns);
     }
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
-  };
-
-  // double-float sums of all levels for this thread's 16 accumulator columns
-  float hi[16], lo[16];
+  } else if (warp == NDRAIN + 1) {
+    // ---- MMA issue --------------------------------------------------------
+    if (lane == 0) {
+      // kind::f16 instruction descriptor: D FP32 (bit 4), A and B BF16 (bits 7, 10), K-major, N >> 3, M >> 4
+      constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)((2 * BN) >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+      int it = 0, chunk = 0;
+      bool ok = true;
+      for (int id = blockIdx.x; id < ntiles && ok; id += gridDim.x) {
+        int rb, cb;
+        tl.tile(id, rb, cb);
+        const int nst = tl.stages(cb);
+        for (int s = 0; s < nst; ++s, ++it) {
+          const int slot = it % NSTAGE;
+          const bool first = s % SPC == 0;
+          if (first && chunk > 0) {     // the drain warps have read the previous chunk
+            if (!tcg::wait_parity(tcg::saddr(&acc_empty), (uint32_t)(chunk - 1) & 1u, timeout_ns)) ok = false;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          }
+          if (!ok || *fail || !tcg::wait_parity(tcg::saddr(&full[slot]), (uint32_t)(it / NSTAGE) & 1u, timeout_ns)) { ok = false; break; }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t st = tcg::saddr(sm + slot * STAGE_BYTES);
 #pragma unroll
-  for (int j = 0; j < 16; ++j) { hi[j] = 0.f; lo[j] = 0.f; }
-  uint32_t phase[2] = {0u, 0u}, cphase = 0u;
-  uint32_t fresh = (1u << NACC) - 1u;   // accumulators whose next MMA overwrites
-  const uint32_t tl = tbase + ((uint32_t)(32 * lg) << 16) + 16 * cg;
-  bool ok = true;
-
-  // Per stage s: wait for its operands, issue its MMAs (they run while the
-  // next stage is loaded), then wait for the MMAs of stage s - 1 (the other
-  // buffer) and refill that buffer with stage s + 1. At the end of a K chunk
-  // every thread waits for the chunk's MMAs and drains levels 2..4.
-  load_stage(0);
-  for (int s = 0; s < nst; ++s) {
-    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    if (!ok) s_fail = 1;
-    __syncthreads();
-    if (s_fail) break;
-    const bool chunk_end = ((s + 1) % SPC == 0) || (s + 1 == nst);
-    if (tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t st = tcg::saddr(sm + (s & 1) * STAGE_BYTES);
+          for (int p = 0; p < S / 2; ++p) {
 #pragma unroll
-      for (int kk = 0; kk < KS / 16; ++kk) {
-        for (int t = 0; t < S; ++t) {
-          for (int u = 0; t + u + 2 <= S + 1; ++u) {
-            const int acc = t + u;           // level L = t + u + 2
-            const uint32_t en = (fresh >> acc) & 1u ? 0u : 1u;
-            fresh &= ~(1u << acc);
-            const uint64_t da = oz::desc(st + t * A_SLICE + kk * 2 * A_LBO, A_LBO);
-            const uint64_t db = oz::desc(st + B_OFF + u * B_SLICE + kk * 2 * B_LBO, B_LBO);
-            asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-                         :: "r"(tbase + BN * acc), "l"(da), "l"(db), "r"(idesc), "r"(en));
+            for (int t = 0; t < 2 * p + 2; ++t) {
+              // levels 2p, 2p + 1 from slice t of A and slices 2p - t, 2p - t + 1 of B (row 64 (u + 1); u = -1: zeros)
+              const uint64_t da = oz::desc(st + t * 2 * A_LBO, A_LBO);
+              const uint64_t db = oz::desc(st + A_STAGE + (2 * p - t + 1) * BN * 16, B_KG);
+              const uint32_t en = (first && t == 0) ? 0u : 1u;
+              asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
+                           :: "r"(tbase + 2 * BN * p), "l"(da), "l"(db), "r"(idesc), "r"(en));
+            }
+          }
+          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(tcg::saddr(&empty[slot])) : "memory");
+          if ((s + 1) % SPC == 0 || s + 1 == nst) {
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(tcg::saddr(&acc_full)) : "memory");
+            ++chunk;
           }
         }
       }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(tcg::saddr(&bars[s & 1])) : "memory");
-      if (chunk_end)
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(tcg::saddr(&bars[2])) : "memory");
-      if (chunk_end) fresh = (1u << NACC) - 1u;   // every level restarts after the drain
-    }
-    if (s + 1 < nst) {
-      if (s >= 1) {   // the other buffer was read by the MMAs of stage s - 1
-        const int b = (s + 1) & 1;
-        if (!tcg::wait_parity(tcg::saddr(&bars[b]), phase[b], timeout_ns)) ok = false;
-        phase[b] ^= 1u;
-      }
-      load_stage(s + 1);
-    }
-    if (chunk_end) {
-      if (!tcg::wait_parity(tcg::saddr(&bars[2]), cphase, timeout_ns)) ok = false;
-      cphase ^= 1u;
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      if (ok) {
-        uint32_t v[16];
-#pragma unroll
-        for (int acc = 0; acc < NACC; ++acc) {
-          OZ_LD16(v, 0, tl + BN * acc);
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-          for (int j = 0; j < 16; ++j) df_add(hi[j], lo[j], __uint_as_float(v[j]));
-        }
-      }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       if (!ok) s_fail = 1;
-      __syncthreads();
-      if (s_fail) break;
-    }
-  }
-  if (!s_fail) {
-    const int row = row0 + 32 * lg + lane;
-    const int er = row < M ? oz_ex(eA[row]) : 0;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int j = (rcol0 >> 1) + 8 * cg + q;     // complex column: real part 2q, imaginary 2q + 1
-      if (row >= M || j >= N) continue;
-      const int sc = er + oz_ex(eB[j]);
-      double re = (double)hi[2 * q] + (double)lo[2 * q];
-      double im = (double)hi[2 * q + 1] + (double)lo[2 * q + 1];
-      re = ldexp(re, sc) * alpha;
-      im = ldexp(im, sc) * alpha;
-      if (accumulate) { const double2 cv = C[(size_t)row * ldc + j]; re += cv.x; im += cv.y; }
-      C[(size_t)row * ldc + j] = make_double2(re, im);
+      // MMAs still in flight finish before TMEM is released
+      for (int j = max(0, it - NSTAGE); j < it; ++j)
+        (void)tcg::wait_parity(tcg::saddr(&empty[j % NSTAGE]), (uint32_t)(j / NSTAGE) & 1u, timeout_ns);
     }
   } else {
-    if (tid == 0) atomicExch(status, 1);
-    // let MMAs still in flight finish (bounded) before TMEM is released
-    (void)tcg::wait_parity(tcg::saddr(&bars[2]), cphase, timeout_ns);
+    // ---- drain and epilogue ------------------------------------------------
+    const int lg = warp & 3, half = warp >> 2;      // rows 32 lg .., real columns 32 half .. of each level
+    const uint32_t tl0 = tbase + ((uint32_t)(32 * lg) << 16) + 32 * half;
+    int chunk = 0;
+    bool ok = true;
+    for (int id = blockIdx.x; id < ntiles && ok; id += gridDim.x) {
+      int rb, cb;
+      tl.tile(id, rb, cb);
+      const int nch = (tl.stages(cb) + SPC - 1) / SPC;
+      float hi[32], lo[32];
+#pragma unroll
+      for (int j = 0; j < 32; ++j) { hi[j] = 0.f; lo[j] = 0.f; }
+      for (int q = 0; q < nch; ++q, ++chunk) {
+        ok = tcg::wait_parity(tcg::saddr(&acc_full), (uint32_t)chunk & 1u, timeout_ns) && !*fail;
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        uint32_t v[2][32];
+        OZ_LD32(v[0], tl0);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int l = 0; l < S; ++l) {
+          if (l + 1 < S) OZ_LD32(v[(l + 1) & 1], tl0 + BN * (l + 1));
+#pragma unroll
+          for (int j = 0; j < 32; ++j) df_add(hi[j], lo[j], __uint_as_float(v[l & 1][j]));
+          if (l + 1 < S) asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          if (l + 2 == S) {            // the last level is in registers: the accumulators are free
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(tcg::saddr(&acc_empty)) : "memory");
+          }
+        }
+      }
+      if (!ok) break;
+      const int row = rb * BM + 32 * lg + lane;
+      const int er = row < a.n ? oz_ex(a.raw[row]) : 0;
+#pragma unroll
+      for (int q = 0; q < 16; ++q) {
+        const int j = cb * (BN / 2) + 16 * half + q;   // complex column: real part 2q, imaginary 2q + 1
+        if (row >= a.n || j >= b.n) continue;
+        const int sc = er + oz_ex(b.raw[j]);
+        double re = ldexp((double)hi[2 * q] + (double)lo[2 * q], sc) * alpha;
+        double im = ldexp((double)hi[2 * q + 1] + (double)lo[2 * q + 1], sc) * alpha;
+        double2* dst = &C[(size_t)row * ldc + j];
+        if (accumulate) { const double2 cv = *dst; re += cv.x; im += cv.y; }
+        *dst = make_double2(re, im);
+      }
+    }
+    if (!ok) s_fail = 1;
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
+  if (tid == 0 && s_fail) atomicExch(status, 1);
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tbase), "n"(TCOLS));
 }
