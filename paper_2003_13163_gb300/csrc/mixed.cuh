@@ -56,98 +56,277 @@ __global__ void ns_multiplier_kernel(double2* __restrict__ G, int m) {
 }
 
 // ---------------------------------------------------------------------------
-// Cholesky factorisation G = L L^H of a Hermitian positive definite complex
-// matrix with the inverse L^{-1} alongside, by recursive halving (the host
-// issues the off-diagonal GEMMs): this kernel is the base case, a diagonal
-// block of at most NB rows factored in shared memory (Golub & Van Loan,
-// Matrix Computations, Sec. 4.2) whose triangular factor is then inverted by
-// forward substitution; L goes to the lower triangle of the block in G
-// (leading dimension ldg), L^{-1} to Linv (leading dimension ldl, zeros above
-// the diagonal). A non-positive pivot sets *status (the factorisation then
-// continues with a tiny pivot so that no NaN is produced). The precision
-// form instantiates it in FP32 with NB = 64.
-// ---------------------------------------------------------------------------
-template <typename T, int NB>
-constexpr int chol_smem_bytes() { return 2 * NB * (NB + 1) * (int)sizeof(cplx<T>); }
-constexpr int CHOL32_NB = 64;     // FP32 base block
-
-template <typename T, int NB>
-__global__ void __launch_bounds__(256) chol_diag_kernel(cplx<T>* __restrict__ G, int ldg, int k0, int b,
-                                                        cplx<T>* __restrict__ Linv, int ldl, int* __restrict__ status) {
-  constexpr int LD = NB + 1;
-  extern __shared__ __align__(16) unsigned char csm[];
-  cplx<T>* Ls = reinterpret_cast<cplx<T>*>(csm);            // [NB][LD]
-  cplx<T>* Xs = Ls + NB * LD;                                // [NB][LD]
-  __shared__ T s_inv;
-  const int tid = threadIdx.x;
-  for (int e = tid; e < b * b; e += blockDim.x) {
-    const int i = e / b, j = e % b;
-    Ls[i * LD + j] = i >= j ? G[(size_t)(k0 + i) * ldg + k0 + j] : czero<T>();
-  }
-  __syncthreads();
-  for (int j = 0; j < b; ++j) {
-    if (tid == 0) {
-      T d = Ls[j * LD + j].x;
-      if (!(d > T(0))) { atomicExch(status, 1); d = sizeof(T) == 8 ? T(1e-300) : T(1e-30); }
-      d = sqrt(d);
-      Ls[j * LD + j] = mk<T>(d, T(0));
-      s_inv = T(1) / d;
-    }
-    __syncthreads();
-    for (int i = j + 1 + tid; i < b; i += blockDim.x) Ls[i * LD + j] = cscale<T>(Ls[i * LD + j], s_inv);
-    __syncthreads();
-    const int t = b - j - 1;   // trailing block (j+1 .. b-1), lower triangle
-    for (int e = tid; e < t * t; e += blockDim.x) {
-      const int i = j + 1 + e / t, l = j + 1 + e % t;
-      if (l > i) continue;
-      Ls[i * LD + l] = csub<T>(Ls[i * LD + l], cmul<T>(Ls[i * LD + j], cconj<T>(Ls[l * LD + j])));
-    }
-    __syncthreads();
-  }
-  // X = L^{-1} by forward substitution, one column per thread
-  for (int c = tid; c < b; c += blockDim.x) {
-    for (int i = 0; i < b; ++i) {
-      if (i < c) { Xs[i * LD + c] = czero<T>(); continue; }
-      cplx<T> x = mk<T>(i == c ? T(1) : T(0), T(0));
-      for (int l = c; l < i; ++l) x = csub<T>(x, cmul<T>(Ls[i * LD + l], Xs[l * LD + c]));
-      Xs[i * LD + c] = cscale<T>(x, T(1) / Ls[i * LD + i].x);
-    }
-  }
-  __syncthreads();
-  for (int e = tid; e < b * b; e += blockDim.x) {
-    const int i = e / b, j = e % b;
-    if (i >= j) G[(size_t)(k0 + i) * ldg + k0 + j] = Ls[i * LD + j];
-    Linv[(size_t)i * ldl + j] = Xs[i * LD + j];
-  }
-}
-
-// Mixed-precision Cholesky QR, first half: A (m x m, FP32) = fl32(D G D) +
-// shift I with D = diag(G)^{-1/2} (a zero column gets d = 0), so that the
-// FP32 Cholesky factors a unit-diagonal matrix whatever the column scales;
-// d goes to dvec.
-__global__ void scale_gram_fp32_kernel(const double2* __restrict__ G, int m, float shift, float2* __restrict__ A,
-                                       double* __restrict__ dvec) {
-  const size_t total = (size_t)m * m;
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-    const int i = (int)(e / m), j = (int)(e % m);
-    const double gi = G[(size_t)i * m + i].x, gj = G[(size_t)j * m + j].x;
-    const double di = gi > 1e-300 ? rsqrt(gi) : 0.0, dj = gj > 1e-300 ? rsqrt(gj) : 0.0;
-    const double2 g = G[e];
-    A[e] = make_float2((float)(di * dj * g.x) + (i == j ? shift : 0.0f), (float)(di * dj * g.y));
-    if (i == j) dvec[i] = di;
-  }
-}
-
-// Second half: W (m x m, FP64) = D L^{-H} from the FP32 inverse factor
-// Linv = L^{-1} (lower triangular): W_ij = d_i conj(Linv_ji), upper triangle.
+// Mixed-precision Cholesky QR, the small factor: from the Gram G = Y^H Y (m x m,
+// complex128) to W = D L^{-H} (complex128, upper triangular), with
+// D = diag(G)^{-1/2} (0 for a zero column) and A = fl32(D G D) + shift I =
+// L L^H factored in FP32 (Golub & Van Loan, Matrix Computations, Sec. 4.2).
 // Y W then has Gram L^{-1} (D G D) L^{-H}, close to the identity.
-__global__ void form_w_kernel(const float2* __restrict__ Linv, const double* __restrict__ dvec, int m,
-                              double2* __restrict__ W) {
-  const size_t total = (size_t)m * m;
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-    const int i = (int)(e / m), j = (int)(e % m);
-    const float2 l = Linv[(size_t)j * m + i];
-    W[e] = j >= i ? make_double2(dvec[i] * (double)l.x, -dvec[i] * (double)l.y) : make_double2(0.0, 0.0);
+//
+// One cooperative launch, right-looking over 64 x 64 tiles on [A | I], which
+// turns into [L^H | L^{-1}]: step j multiplies the tiles below A_jj by L_jj^{-H}
+// and row j of the right half by L_jj^{-1} (barrier), then subtracts rank 64
+// from everything below; CTA 0 meanwhile updates A_{j+1,j+1} first and factors
+// it, so the serial 64 x 64 factorisation runs under the tile products
+// (barrier). The factorisation holds its tile and the tile of L^{-1} in
+// registers (4 x 4 of each per thread) and passes one barrier per column.
+// What bounds it: FP32 FMAs for m >= 1024 (m^3 / 3 tile flops), else the chain
+// of 2 m / 64 barriers and tile latencies. A pass at m = 2048 took 8.4 ms as 156
+// launches (recursive halving, a 64 x 64 base case of 130 us), 2.4 ms now; at
+// m = 512 1.5 -> 0.44 ms.
+// A non-positive pivot sets *status to 1 (the factorisation goes on with a tiny
+// one, so that no NaN is produced), a barrier that timed out to 2.
+// ---------------------------------------------------------------------------
+constexpr int CH = 64;                 // tile
+constexpr int CHP = CH + 2;            // padded row of a staged tile (16-byte rows)
+constexpr int CHOL_SMEM = 2 * CH * CHP * (int)sizeof(float2);
+
+// Stage the CH x CH tile at (r0, c0) of M (ld m, zero outside m x m) as
+// dst[k][i]: trans != 0 puts the tile's columns along k (dst[k][i] = M[r0 + i][c0 + k]),
+// 0 its rows (dst[k][i] = M[r0 + k][c0 + i]).
+__device__ __forceinline__ void chol_stage(float2* dst, const float2* M, int m, int r0, int c0, int trans) {
+#pragma unroll 4
+  for (int e = threadIdx.x; e < CH * CH; e += 256) {
+    const int r = e >> 6, c = e & 63;
+    const float2 v = r0 + r < m && c0 + c < m ? ldcg(&M[(size_t)(r0 + r) * m + c0 + c]) : make_float2(0.f, 0.f);
+    if (trans) dst[c * CHP + r] = v;
+    else dst[r * CHP + c] = v;
+  }
+}
+
+// acc[a][b] = sum_k As[k][4 ty + a] op(Bs[k][4 tx + b]), op = conjugate if conjb.
+__device__ __forceinline__ void chol_tile(float2 (&acc)[4][4], const float2* As, const float2* Bs, bool conjb) {
+  const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+  const float sg = conjb ? -1.0f : 1.0f;
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) acc[a][b] = make_float2(0.f, 0.f);
+#pragma unroll 8
+  for (int k = 0; k < CH; ++k) {
+    float2 av[4], bv[4];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float4 x = *reinterpret_cast<const float4*>(&As[k * CHP + 4 * ty + 2 * h]);
+      const float4 y = *reinterpret_cast<const float4*>(&Bs[k * CHP + 4 * tx + 2 * h]);
+      av[2 * h] = make_float2(x.x, x.y); av[2 * h + 1] = make_float2(x.z, x.w);
+      bv[2 * h] = make_float2(y.x, sg * y.y); bv[2 * h + 1] = make_float2(y.z, sg * y.w);
+    }
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) cfma<float>(acc[a][b], av[a], bv[b]);
+  }
+}
+
+// Factor the Hermitian tile a (this thread's 4 x 4 part; rows and columns from
+// m on read as identity) and leave the lower triangular L^{-1} in r.
+__device__ __forceinline__ void chol_factor(float2 (&a)[4][4], float2 (&r)[4][4], float2* buf, float* diag, int* status) {
+  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) r[i][k] = make_float2(ty == tx && i == k ? 1.f : 0.f, 0.f);
+  for (int jb = 0; jb < CH / 4; ++jb) {
+#pragma unroll
+    for (int jj = 0; jj < 4; ++jj) {
+      const int j = 4 * jb + jj;
+      float2* col = buf + (j & 1) * 2 * CH;    // column j of A, row j of the right half; two buffers in turn
+      float2* row = col + CH;
+      if (tx == jb) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) col[4 * ty + i] = a[i][jj];
+      }
+      if (ty == jb) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) row[4 * tx + k] = r[jj][k];
+      }
+      __syncthreads();
+      float d = col[j].x;
+      if (!(d > 0.f)) {
+        if (tid == 0) atomicMax(status, 1);
+        d = 1e-30f;
+      }
+      if (tid == 0) diag[j] = d;
+      const float inv = 1.0f / d;
+      float2 f[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float2 c = col[4 * ty + i];
+        f[i] = 4 * ty + i > j ? make_float2(c.x * inv, c.y * inv) : make_float2(0.f, 0.f);
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float2 c = col[4 * tx + k], w = row[4 * tx + k];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          // a_ik -= f_i conj(a_kj), r_ik -= f_i r_jk
+          a[i][k].x = fmaf(-f[i].x, c.x, fmaf(-f[i].y, c.y, a[i][k].x));
+          a[i][k].y = fmaf(-f[i].y, c.x, fmaf(f[i].x, c.y, a[i][k].y));
+          r[i][k].x = fmaf(-f[i].x, w.x, fmaf(f[i].y, w.y, r[i][k].x));
+          r[i][k].y = fmaf(-f[i].x, w.y, fmaf(-f[i].y, w.x, r[i][k].y));
+        }
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float s = rsqrtf(diag[4 * ty + i]);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) r[i][k] = 4 * tx + k <= 4 * ty + i ? make_float2(s * r[i][k].x, s * r[i][k].y) : make_float2(0.f, 0.f);
+  }
+}
+
+__global__ void __launch_bounds__(256) cholqr_factor_kernel(const double2* __restrict__ G, int m, float shift, float2* A,
+                                                            float2* Li, double2* __restrict__ W, int* status, GridCtl* ctl,
+                                                            long long timeout_ns) {
+  extern __shared__ __align__(16) unsigned char csm[];
+  float2* As = reinterpret_cast<float2*>(csm);
+  float2* Bs = As + CH * CHP;
+  __shared__ double s_d[2 * CH];
+  __shared__ float s_diag[CH];
+  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, nb = (m + CH - 1) / CH;
+  const int nblk = (int)gridDim.x, bid = (int)blockIdx.x;
+  auto barrier = [&]() -> bool {
+    if (grid_barrier(ctl, gridDim.x, timeout_ns)) return true;
+    if (tid == 0) atomicMax(status, 2);
+    return false;
+  };
+  // column scales of tiles ti and tk -> s_d
+  auto scales = [&](int ti, int tk) {
+    __syncthreads();
+    if (tid < 2 * CH) {
+      const int i = (tid < CH ? ti : tk) * CH + (tid & (CH - 1));
+      const double g = i < m ? G[(size_t)i * m + i].x : 0.0;
+      s_d[tid] = g > 1e-300 ? rsqrt(g) : 0.0;
+    }
+    __syncthreads();
+  };
+  // this thread's part of a finished tile of L^{-1}: to Li and, conjugate
+  // transposed and scaled, to W; the tile of W across the diagonal is zero
+  auto finish = [&](int j, int k, const float2 (&r)[4][4]) {
+    scales(k, k);
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const int gi = j * CH + 4 * ty + a, gk = k * CH + 4 * tx + b;
+        if (gi >= m || gk >= m) continue;
+        stcg(&Li[(size_t)gi * m + gk], r[a][b]);
+        if (gk <= gi) {
+          const double d = s_d[4 * tx + b];
+          W[(size_t)gk * m + gi] = make_double2(d * (double)r[a][b].x, -d * (double)r[a][b].y);
+        }
+        if (gk < gi) W[(size_t)gi * m + gk] = make_double2(0.0, 0.0);
+      }
+  };
+
+  // A = fl32(D G D) + shift I, lower tiles
+  for (int q = bid; q < nb * (nb + 1) / 2; q += nblk) {
+    int i = 0, k = q;
+    while (k > i) k -= ++i;
+    scales(i, k);
+    for (int e = tid; e < CH * CH; e += 256) {
+      const int r = e >> 6, c = e & 63, gr = i * CH + r, gc = k * CH + c;
+      if (gr >= m || gc >= m) continue;
+      const double2 g = G[(size_t)gr * m + gc];
+      const double dd = s_d[r] * s_d[CH + c];
+      stcg(&A[(size_t)gr * m + gc], make_float2((float)(dd * g.x) + (gr == gc ? shift : 0.0f), (float)(dd * g.y)));
+    }
+  }
+  if (!barrier()) return;
+
+  float2 acc[4][4];
+  // diagonal tile j, less the product in acc, factored by this CTA
+  auto diagonal = [&](int j) {
+    float2 a[4][4], r[4][4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x)
+#pragma unroll
+      for (int y = 0; y < 4; ++y) {
+        const int gi = j * CH + 4 * ty + x, gk = j * CH + 4 * tx + y;
+        // the upper triangle is not used (column j of the tile is read below the pivot)
+        float2 v = gi < m && gk < m ? ldcg(&A[(size_t)gi * m + gk]) : make_float2(gi == gk ? 1.f : 0.f, 0.f);
+        a[x][y] = csub<float>(v, acc[x][y]);
+      }
+    __syncthreads();
+    chol_factor(a, r, As, s_diag, status);
+    finish(j, j, r);
+  };
+  if (bid == 0) {
+#pragma unroll
+    for (int x = 0; x < 4; ++x)
+#pragma unroll
+      for (int y = 0; y < 4; ++y) acc[x][y] = make_float2(0.f, 0.f);
+    diagonal(0);
+  }
+  if (!barrier()) return;
+  for (int j = 0; j < nb; ++j) {
+    // panel: L_ij = A_ij L_jj^{-H} (i > j), (L^{-1})_jk = L_jj^{-1} R_jk (k < j)
+    for (int q = bid; q < nb; q += nblk) {
+      if (q == j) continue;
+      __syncthreads();
+      if (q > j) {
+        chol_stage(As, A, m, q * CH, j * CH, 1);
+        chol_stage(Bs, Li, m, j * CH, j * CH, 1);
+      } else {
+        chol_stage(As, Li, m, j * CH, j * CH, 1);
+        chol_stage(Bs, Li, m, j * CH, q * CH, 0);
+      }
+      __syncthreads();
+      chol_tile(acc, As, Bs, q > j);
+      if (q > j) {
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+#pragma unroll
+          for (int y = 0; y < 4; ++y) {
+            const int gi = q * CH + 4 * ty + x, gk = j * CH + 4 * tx + y;
+            if (gi < m && gk < m) stcg(&A[(size_t)gi * m + gk], acc[x][y]);
+          }
+      } else {
+        finish(j, q, acc);
+      }
+    }
+    if (j + 1 == nb) break;
+    if (!barrier()) return;
+    // rank-64 update of the rows below: A_ik -= L_ij L_kj^H (j < k <= i) and
+    // R_ik -= L_ij (L^{-1})_jk (k <= j; R_ij starts here); CTA 0 takes the next
+    // diagonal tile, the others the rest
+    const int lanes = nblk > 1 ? nblk - 1 : 1, me = nblk > 1 ? bid - 1 : 0;
+    if (bid == 0) {
+      __syncthreads();
+      chol_stage(As, A, m, (j + 1) * CH, j * CH, 1);
+      __syncthreads();
+      chol_tile(acc, As, As, true);
+      diagonal(j + 1);
+    }
+    if (me >= 0) {
+      int total = 0;
+      for (int i = j + 1; i < nb; ++i) total += i + 1;
+      for (int q = me; q < total; q += lanes) {
+        int i = j + 1, k = q;
+        while (k > i) k -= ++i;
+        if (i == j + 1 && k == i) continue;
+        const bool right = k <= j;
+        __syncthreads();
+        chol_stage(As, A, m, i * CH, j * CH, 1);
+        if (right) chol_stage(Bs, Li, m, j * CH, k * CH, 0);
+        else chol_stage(Bs, A, m, k * CH, j * CH, 1);
+        __syncthreads();
+        chol_tile(acc, As, Bs, !right);
+        float2* C = right ? Li : A;
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+#pragma unroll
+          for (int y = 0; y < 4; ++y) {
+            const int gi = i * CH + 4 * ty + x, gk = k * CH + 4 * tx + y;
+            if (gi >= m || gk >= m) continue;
+            const float2 c0 = k == j ? make_float2(0.f, 0.f) : ldcg(&C[(size_t)gi * m + gk]);
+            stcg(&C[(size_t)gi * m + gk], csub<float>(c0, acc[x][y]));
+          }
+      }
+    }
+    if (!barrier()) return;
   }
 }
 

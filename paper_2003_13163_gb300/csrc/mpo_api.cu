@@ -146,8 +146,7 @@ struct mpo_ctx {
   double* mx_w = nullptr;
   double2* mx_W = nullptr;         // D L^{-H} of a Cholesky QR pass; the FP32 Ritz vectors, promoted
   double2* mx_Q0 = nullptr;        // the stage-2 basis (FP32 Ritz directions in FP64)
-  float2 *mx_A32 = nullptr, *mx_Li32 = nullptr, *mx_t32 = nullptr;   // FP32 Cholesky: scaled Gram, L^{-1}, scratch
-  double* mx_d = nullptr;          // column scales of a Cholesky QR pass
+  float2 *mx_A32 = nullptr, *mx_Li32 = nullptr;   // FP32 Cholesky: scaled Gram, L^{-1}
   unsigned long long mx_seed = 0;  // start-basis counter
   int mx_last_steps = 0;           // subspace steps taken by the last factorisation
   int mx_cur_bond = -1;            // bond of the gate being factorised (-1: not a gate)
@@ -560,39 +559,23 @@ static int mx_newton_schulz(mpo_ctx* h, double2*& Y, double2*& spare, int rows, 
   return MPO_OK;
 }
 
-// FP32 Cholesky factorisation of the Hermitian block A[k0:k0+s, k0:k0+s]
-// (leading dimension m) into L (lower triangle, in place) and L^{-1} into the
-// same block of Li, by recursive halving: with A = [[A11, .], [A21, A22]],
-//   L11, L11^{-1} <- recursion on A11;  L21 = A21 L11^{-H};
-//   A22 -= L21 L21^H;  L22, L22^{-1} <- recursion on A22;
-//   (L^{-1})_21 = -L22^{-1} L21 L11^{-1}.
-// Blocks of at most CHOL32_NB rows are factored by chol_diag_kernel, the rest
-// by FP32 GEMMs. Li is zero above the diagonal blocks on entry.
-static int chol32_rec(mpo_ctx* h, float2* A, float2* Li, int m, int k0, int s) {
-  if (s <= CHOL32_NB) {
-    chol_diag_kernel<float, CHOL32_NB><<<1, 256, chol_smem_bytes<float, CHOL32_NB>(), h->st>>>(
-        A, m, k0, s, Li + (size_t)k0 * m + k0, m, h->mx_chst);
-    CK(h, cudaGetLastError());
-    return MPO_OK;
-  }
-  const int s1 = std::min(s - 1, (s / 2 + CHOL32_NB - 1) / CHOL32_NB * CHOL32_NB), s2 = s - s1;
-  int rc = chol32_rec(h, A, Li, m, k0, s1);
-  if (rc) return rc;
-  float2* A21 = A + (size_t)(k0 + s1) * m + k0;
-  float2* A22 = A21 + s1;
-  const float2* Li11 = Li + (size_t)k0 * m + k0;
-  float2* Li21 = Li + (size_t)(k0 + s1) * m + k0;
-  const float2* Li22 = Li21 + s1;
-  float2* T = h->mx_t32;                                                                // s2 x s1
-  CK(h, cgemm<float>(h->st, s2, s1, s1, A21, m, 0, Li11, m, 1, T, s1));                 // L21 = A21 L11^{-H}
-  CK(h, cudaMemcpy2DAsync(A21, (size_t)m * sizeof(float2), T, (size_t)s1 * sizeof(float2),
-                          (size_t)s1 * sizeof(float2), s2, cudaMemcpyDeviceToDevice, h->st));
-  CK(h, cgemm<float>(h->st, s2, s2, s1, A21, m, 0, A21, m, 1, A22, m, nullptr, -1.0, 1));   // A22 -= L21 L21^H
-  rc = chol32_rec(h, A, Li, m, k0 + s1, s2);
-  if (rc) return rc;
-  CK(h, cgemm<float>(h->st, s2, s1, s1, A21, m, 0, Li11, m, 0, T, s1));                 // L21 L11^{-1}
-  CK(h, cgemm<float>(h->st, s2, s1, s2, Li22, m, 0, T, s1, 0, Li21, m, nullptr, -1.0, 0));   // -L22^{-1} (.)
-  return MPO_OK;
+// The FP32 shift 8 m u_32 is explained at mx_cholqr_pass. ctl stays zeroed
+// between launches (a barrier leaves its word's low bits at zero).
+static cudaError_t launch_cholqr_factor(cudaStream_t st, const double2* G, int m, float2* A, float2* Li, double2* W,
+                                        int* status, GridCtl* ctl, double timeout_s, int num_sms) {
+  cudaError_t e = ensure_dynamic_smem((const void*)cholqr_factor_kernel, CHOL_SMEM);
+  if (e != cudaSuccess) return e;
+  int per_sm = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cholqr_factor_kernel, 256, CHOL_SMEM);
+  if (e != cudaSuccess) return e;
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  // the widest phase, the update after the first step, has nb (nb + 1) / 2 - 1 tiles
+  const int nb = (m + CH - 1) / CH;
+  const int blocks = std::max(1, std::min(std::min(per_sm, 2) * num_sms, nb * (nb + 1) / 2));
+  float shift = (float)(8.0 * m * 5.9604644775390625e-08);
+  long long timeout_ns = (long long)(timeout_s * 1e9);
+  void* args[] = {&G, &m, &shift, &A, &Li, &W, &status, &ctl, &timeout_ns};
+  return cudaLaunchCooperativeKernel((const void*)cholqr_factor_kernel, dim3(blocks), dim3(256), args, CHOL_SMEM, st);
 }
 
 // One mixed-precision Cholesky QR pass on Y (rows x m, leading dimension m):
@@ -609,15 +592,8 @@ static int mx_cholqr_pass(mpo_ctx* h, double2*& Y, double2*& spare, int rows, in
   CK(h, mx_gemm(h, m, m, rows, Y, m, 1, Y, m, 0, h->mx_G, m));
   {
     ProfScope ps(h, PK_REFINE, 16.0 * m * m * m / 3.0, 6.0 * m * m * sizeof(float2));
-    const float shift = (float)(8.0 * m * 5.9604644775390625e-08);
-    scale_gram_fp32_kernel<<<grid_for((size_t)m * m, h->num_sms), 256, 0, h->st>>>(h->mx_G, m, shift, h->mx_A32,
-                                                                                      h->mx_d);
-    CK(h, cudaGetLastError());
-    CK(h, cudaMemsetAsync(h->mx_Li32, 0, (size_t)m * m * sizeof(float2), h->st));
-    int rc = chol32_rec(h, h->mx_A32, h->mx_Li32, m, 0, m);
-    if (rc) return rc;
-    form_w_kernel<<<grid_for((size_t)m * m, h->num_sms), 256, 0, h->st>>>(h->mx_Li32, h->mx_d, m, h->mx_W);
-    CK(h, cudaGetLastError());
+    CK(h, launch_cholqr_factor(h->st, h->mx_G, m, h->mx_A32, h->mx_Li32, h->mx_W, h->mx_chst, h->ctl,
+                               h->opts.barrier_timeout_s, h->num_sms));
   }
   CK(h, mx_gemm(h, rows, m, m, Y, m, 0, h->mx_W, m, 0, spare, m));
   std::swap(Y, spare);
@@ -653,6 +629,7 @@ static int msvd_status(mpo_ctx* h) {
   if (h->hs->ctl.err) return fail(h, MPO_ERR_TIMEOUT, "grid barrier wait timed out in the FP32 Rayleigh-Ritz SVD");
   if (h->hs->ctl.status) return fail(h, MPO_ERR_NOCONV, "FP32 Rayleigh-Ritz SVD reached eig_max_sweeps");
   if (h->use_oz && h->hs->oz_err) return fail(h, MPO_ERR_TIMEOUT, "an mbarrier wait timed out in the tensor-core FP64 GEMM");
+  if (h->hs->chol_status == 2) return fail(h, MPO_ERR_TIMEOUT, "grid barrier wait timed out in the Cholesky QR factorisation");
   if (h->hs->chol_status) return fail(h, MPO_ERR_NOCONV, "Cholesky QR met a non-positive pivot");
   return MPO_OK;
 }
@@ -969,6 +946,7 @@ static int mx_isometry(mpo_ctx* h, double2*& Y, int rows, int r, bool* ok) {
   if (h->use_oz) CK(h, cudaMemcpyAsync(&h->hs->oz_err, h->oz.status, sizeof(int), cudaMemcpyDeviceToHost, h->st));
   CK(h, cudaStreamSynchronize(h->st));
   if (h->use_oz && h->hs->oz_err) return fail(h, MPO_ERR_TIMEOUT, "an mbarrier wait timed out in the tensor-core FP64 GEMM");
+  if (h->hs->chol_status == 2) return fail(h, MPO_ERR_TIMEOUT, "grid barrier wait timed out in the Cholesky QR factorisation");
   *ok = !h->hs->chol_status && defect <= 1e-5;
   return MPO_OK;
 }
@@ -1459,10 +1437,8 @@ static bool alloc_factor_ws(mpo_ctx* h, int m, int ccap, size_t bj_nch) {
     ok = ok && alloc((void**)&h->mx_Q0, (size_t)m * mm * sizeof(double2));
     ok = ok && alloc((void**)&h->mx_A32, mm * mm * sizeof(float2));
     ok = ok && alloc((void**)&h->mx_Li32, mm * mm * sizeof(float2));
-    ok = ok && alloc((void**)&h->mx_t32, mm * mm * sizeof(float2));
-    ok = ok && alloc((void**)&h->mx_d, mm * sizeof(double));
     ok = ok && alloc((void**)&h->mx_chst, sizeof(int));
-    if (ok) ok = ensure_dynamic_smem((const void*)chol_diag_kernel<float, CHOL32_NB>, chol_smem_bytes<float, CHOL32_NB>()) == cudaSuccess;
+    ok = ok && cudaMemsetAsync(h->ctl, 0, sizeof(GridCtl), h->st) == cudaSuccess;
   }
   return ok;
 }
@@ -1562,8 +1538,8 @@ int mpo_init(mpo_handle* out, int n, int chi_max, mpo_precision prec, void* stre
                                       2 * (size_t)mx_ccap * h->mx_mcap * sizeof(double2) +
                                       2 * (size_t)h->mx_mcap * h->mx_mcap * sizeof(double2) +
                                       2 * (size_t)h->mx_mcap * h->mx_mcap * sizeof(double2) +
-                                      3 * (size_t)h->mx_mcap * h->mx_mcap * sizeof(float2) +
-                                      (size_t)m * h->mx_mcap * sizeof(double2) + (size_t)h->mx_mcap * sizeof(double)
+                                      2 * (size_t)h->mx_mcap * h->mx_mcap * sizeof(float2) +
+                                      (size_t)m * h->mx_mcap * sizeof(double2)
                                 : 0) +
                       (h->use_oz ? (size_t)oz::S * 2 * 3 * (size_t)std::max(m, mx_ccap) * 2 *
                                        (size_t)((std::max(m, mx_ccap) + 127) / 128 * 128)
@@ -1638,7 +1614,7 @@ void mpo_free(mpo_handle h) {
                 h->dsup, h->dp, h->info, h->ctl, h->scal, h->dS, h->dschmidt, h->tv0, h->tv1,
                 h->mx_a32, h->mx_ut32, h->mx_w32, h->mx_perm32, h->mx_lam32, h->mx_info32, h->mx_Q, h->mx_Q2,
                 h->mx_B, h->mx_T, h->mx_V, h->mx_G, h->mx_w,
-                h->mx_W, h->mx_A32, h->mx_Li32, h->mx_t32, h->mx_d, h->mx_chst, h->mx_eosctl, h->mx_rot, h->mx_Q0};
+                h->mx_W, h->mx_A32, h->mx_Li32, h->mx_chst, h->mx_eosctl, h->mx_rot, h->mx_Q0};
   for (void* p : ps) if (p) cudaFree(p);
   if (h->hs) cudaFreeHost(h->hs);
   free_oz(h->oz);
