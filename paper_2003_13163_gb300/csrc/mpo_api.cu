@@ -464,20 +464,22 @@ constexpr int kMixedSteps = 4;        // steps before the first convergence chec
 // the MMA kernel. Returns cudaErrorInvalidValue if the scratch is too small.
 static cudaError_t oz_gemm(cudaStream_t st, int M, int N, int K, const double2* A, int lda, int opA, const double2* B,
                            int ldb, int opB, double2* C, int ldc, double alpha, int accumulate, const OzWork& w,
-                           double timeout_s, int num_sms) {
+                           double timeout_s, int num_sms, int mode = OzTiles::kGeneral) {
   if (M <= 0 || N <= 0) return cudaSuccess;
   const int nkb = (std::max(K, 1) + 15) / 16;
   const int Mp = (M + oz::BM - 1) / oz::BM * oz::BM, Nrp = (2 * N + oz::BN - 1) / oz::BN * oz::BN;
   const size_t Kp = 32 * (size_t)nkb;
   if ((size_t)oz::S * Mp * Kp > w.a_cap || (size_t)oz::S * Nrp * Kp > w.b_cap || Mp > w.e_cap || Nrp / 2 > w.e_cap)
     return cudaErrorInvalidValue;
-  const OzOp a{A, lda, opA, M, w.ea, w.a}, b{B, ldb, opB, N, w.eb, w.b};
+  // the rows and columns of a Hermitian product have the same exponents
+  const bool herm = mode == OzTiles::kHerm;
+  const OzOp a{A, lda, opA, M, w.ea, w.a}, b{B, ldb, opB, N, herm ? w.ea : w.eb, w.b};
   // scaling exponents (eb follows ea in one allocation), then the slices: one
   // launch each for both operands
   cudaError_t e = cudaMemsetAsync(w.ea, 0, sizeof(int) * ((size_t)w.e_cap + N), st);
   if (e != cudaSuccess) return e;
   auto scans = [&](int rows, int cols) { return ((cols + 31) / 32) * ((rows + 255) / 256); };
-  const int na = opA ? scans(K, M) : scans(M, K), nb = opB ? scans(N, K) : scans(K, N);
+  const int na = opA ? scans(K, M) : scans(M, K), nb = herm ? 0 : (opB ? scans(N, K) : scans(K, N));
   oz_exp_kernel<<<na + nb, dim3(32, 8), 0, st>>>(a, b, K, na);
   const int sa = nkb * (Mp / 32), sb = nkb * (Nrp / 32);
   oz_split_kernel<<<sa + sb, 128, 0, st>>>(a, b, K, nkb, sa);
@@ -485,8 +487,8 @@ static cudaError_t oz_gemm(cudaStream_t st, int M, int N, int K, const double2* 
   if (e != cudaSuccess) return e;
   e = ensure_dynamic_smem((const void*)oz_mma_kernel, oz::SMEM_BYTES);
   if (e != cudaSuccess) return e;
-  const OzTiles tl{Mp / oz::BM, Nrp / oz::BN, nkb};
-  oz_mma_kernel<<<std::min(num_sms, tl.nrb * tl.ncb), oz::NT, oz::SMEM_BYTES, st>>>(tl, a, b, C, ldc, alpha, accumulate,
+  const OzTiles tl{Mp / oz::BM, Nrp / oz::BN, nkb, mode};
+  oz_mma_kernel<<<std::min(num_sms, tl.count()), oz::NT, oz::SMEM_BYTES, st>>>(tl, a, b, C, ldc, alpha, accumulate,
                                                                                   w.status, (long long)(timeout_s * 1e9));
   return cudaGetLastError();
 }
@@ -524,14 +526,21 @@ static void free_oz(OzWork& w) {
 static bool oz_worth(int M, int N, int K) { return (double)M * N * K >= 2.6e5 && M >= 16 && N >= 8 && K >= 16; }
 
 static cudaError_t mx_gemm(mpo_ctx* h, int M, int N, int K, const double2* A, int lda, int opA, const double2* B,
-                           int ldb, int opB, double2* C, int ldc, double alpha = 1.0, int accumulate = 0) {
+                           int ldb, int opB, double2* C, int ldc, double alpha = 1.0, int accumulate = 0,
+                           int mode = OzTiles::kGeneral) {
   ProfScope ps(h, PK_REFINE, 8.0 * M * N * K, (double)((size_t)M * K + (size_t)K * N + (size_t)M * N) * sizeof(double2));
   if (h->use_oz && oz_worth(M, N, K)) {
     ps.cls = PK_OZ;
     return oz_gemm(h->st, M, N, K, A, lda, opA, B, ldb, opB, C, ldc, alpha, accumulate, h->oz,
-                   h->opts.barrier_timeout_s, h->num_sms);
+                   h->opts.barrier_timeout_s, h->num_sms, mode);
   }
   return cgemm<double>(h->st, M, N, K, A, lda, opA, B, ldb, opB, C, ldc, nullptr, alpha, accumulate);
+}
+
+// G (n x n) = op(Y) op(Y)^H: the Gram of the columns (op 1: Y^H Y, Y k x n) or of
+// the rows (op 0: Y Y^H, Y n x k).
+static cudaError_t mx_gram(mpo_ctx* h, int n, int k, const double2* Y, int ldy, int op, double2* G, int ldg) {
+  return mx_gemm(h, n, n, k, Y, ldy, op, Y, ldy, 1 - op, G, ldg, 1.0, 0, OzTiles::kHerm);
 }
 
 // Y (rows x m, leading dimension m) <- Y (3 I - Y^H Y) / 2, iters times
@@ -542,7 +551,7 @@ static cudaError_t mx_gemm(mpo_ctx* h, int M, int N, int K, const double2* A, in
 static int mx_newton_schulz(mpo_ctx* h, double2*& Y, double2*& spare, int rows, int m, int iters,
                             double* defect_dev = nullptr) {
   for (int it = 0; it < iters; ++it) {
-    CK(h, mx_gemm(h, m, m, rows, Y, m, 1, Y, m, 0, h->mx_G, m));
+    CK(h, mx_gram(h, m, rows, Y, m, 1, h->mx_G, m));
     if (defect_dev && it == iters - 1) {   // |Y^H Y - I| entering the last step
       CK(h, cudaMemsetAsync(defect_dev, 0, sizeof(double), h->st));
       defect_kernel<<<grid_for((size_t)m * m, h->num_sms), 256, 0, h->st>>>(h->mx_G, m, defect_dev);
@@ -589,13 +598,13 @@ static cudaError_t launch_cholqr_factor(cudaStream_t st, const double2* G, int m
 // Tomov & Dongarra, SIAM J. Sci. Comput. 37 (2015); the shift: Fukaya,
 // Kannan, Nakatsukasa, Yamamoto & Yanagisawa, SIAM J. Sci. Comput. 42 (2020).
 static int mx_cholqr_pass(mpo_ctx* h, double2*& Y, double2*& spare, int rows, int m) {
-  CK(h, mx_gemm(h, m, m, rows, Y, m, 1, Y, m, 0, h->mx_G, m));
+  CK(h, mx_gram(h, m, rows, Y, m, 1, h->mx_G, m));
   {
     ProfScope ps(h, PK_REFINE, 16.0 * m * m * m / 3.0, 6.0 * m * m * sizeof(float2));
     CK(h, launch_cholqr_factor(h->st, h->mx_G, m, h->mx_A32, h->mx_Li32, h->mx_W, h->mx_chst, h->ctl,
                                h->opts.barrier_timeout_s, h->num_sms));
   }
-  CK(h, mx_gemm(h, rows, m, m, Y, m, 0, h->mx_W, m, 0, spare, m));
+  CK(h, mx_gemm(h, rows, m, m, Y, m, 0, h->mx_W, m, 0, spare, m, 1.0, 0, OzTiles::kUpper));
   std::swap(Y, spare);
   return MPO_OK;
 }
@@ -746,8 +755,8 @@ static int msvd_select(mpo_ctx* h, double2* X, int r, int c, int ldx, int cap, b
     const double2* Bs = iterate ? h->mx_B : X;
     const int ldbs = iterate ? c : ldx;
     CK(h, mx_gemm(h, m, c, m, h->mx_W, m, 1, Bs, ldbs, 0, h->mx_T, c));        // V^H B (m x c)
-    CK(h, mx_gemm(h, m, m, c, h->mx_T, c, 0, h->mx_T, c, 1, h->mx_G, m));      // S = V^H H V
-    CK(h, mx_gemm(h, m, m, m, h->mx_W, m, 1, h->mx_W, m, 0, h->mx_V, m));      // G = V^H V
+    CK(h, mx_gram(h, m, c, h->mx_T, c, 0, h->mx_G, m));      // S = V^H H V
+    CK(h, mx_gram(h, m, m, h->mx_W, m, 1, h->mx_V, m));      // G = V^H V
     {
       ProfScope ps(h, PK_REFINE, 0.0, 3.0 * (double)m * mp * sizeof(double2));
       partition_correction_kernel<<<grid_for((size_t)(m - mp) * mp, h->num_sms), 256, 0, h->st>>>(
@@ -767,7 +776,7 @@ static int msvd_select(mpo_ctx* h, double2* X, int r, int c, int ldx, int cap, b
   // 4. FP64 Rayleigh-Ritz (stage 2): B' = Q'^H X, H' = B' B'^H, nearly
   // diagonal, and the FP64 Hermitian Jacobi eigen-solve H' = V diag(w) V^H
   CK(h, mx_gemm(h, mp, c, r, Qp, mp, 1, X, ldx, 0, h->mx_B, c));            // B' (mp x c)
-  CK(h, mx_gemm(h, mp, mp, c, h->mx_B, c, 0, h->mx_B, c, 1, h->mx_G, mp));  // H' (mp x mp)
+  CK(h, mx_gram(h, mp, c, h->mx_B, c, 0, h->mx_G, mp));  // H' (mp x mp)
   {
     ProfScope ps(h, PK_EIG64, 13.3 * (double)mp * mp * mp, 3.0 * (double)mp * mp * sizeof(double2));
     hermitise_kernel<<<grid_for((size_t)mp * mp, h->num_sms), 256, 0, h->st>>>(h->mx_G, mp);
@@ -934,7 +943,7 @@ static int mx_isometry(mpo_ctx* h, double2*& Y, int rows, int r, bool* ok) {
   if (rc) return rc;
   rc = mx_newton_schulz(h, Y, sp, rows, r, 2);
   if (rc) return rc;
-  CK(h, mx_gemm(h, r, r, rows, Y, r, 1, Y, r, 0, h->mx_G, r));
+  CK(h, mx_gram(h, r, rows, Y, r, 1, h->mx_G, r));
   CK(h, cudaMemsetAsync(h->scal + 3, 0, sizeof(double), h->st));
   defect_kernel<<<grid_for((size_t)r * r, h->num_sms), 256, 0, h->st>>>(h->mx_G, r, h->scal + 3);
   CK(h, cudaGetLastError());

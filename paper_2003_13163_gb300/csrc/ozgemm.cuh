@@ -243,18 +243,41 @@ __device__ __forceinline__ void df_add(float& hi, float& lo, float x) {
   lo = __fadd_rn(lo, err);
 }
 
-// The tile list of a product. Row blocks go in groups of 16 and the column
-// blocks of a group in turn, so the tiles in flight at one time share their
-// operands in L2.
+// The tile list of a product. General: row blocks in groups of 16 and the
+// column blocks of a group in turn, so the tiles in flight at one time share
+// their operands in L2.
+// kHerm (op(A) op(B) Hermitian, e.g. a Gram): only the tiles that reach the
+// diagonal or lie above it; the epilogue writes the mirror image too.
+// kUpper (op(B) upper triangular, zero below the diagonal): a tile's K loop ends
+// with its last column; column blocks from the longest down.
+// Both halve the work of a Cholesky QR pass (Y^H Y and Y W).
 struct OzTiles {
+  enum { kGeneral = 0, kHerm = 1, kUpper = 2 };
   int nrb, ncb, nkb;      // row blocks, column blocks, blocks of 16 complex k
-  __device__ __forceinline__ int count() const { return nrb * ncb; }
+  int mode;
+  __host__ __device__ __forceinline__ int count() const {
+    if (mode != kHerm) return nrb * ncb;
+    int n = 0;
+    for (int rb = 0; rb < nrb && 4 * rb < ncb; ++rb) n += ncb - 4 * rb;
+    return n;
+  }
   __device__ __forceinline__ void tile(int id, int& rb, int& cb) const {
+    if (mode == kHerm) {            // row 128 rb <= column 32 cb + 31
+      rb = 0;
+      while (id >= ncb - 4 * rb) id -= ncb - 4 * rb++;
+      cb = 4 * rb + id;
+      return;
+    }
+    if (mode == kUpper) {
+      cb = ncb - 1 - id / nrb;
+      rb = id % nrb;
+      return;
+    }
     const int per = 16 * ncb, g = id / per, h = min(16, nrb - 16 * g), w = id - g * per;
     rb = 16 * g + w % h;
     cb = w / h;
   }
-  __device__ __forceinline__ int stages(int) const { return 2 * nkb; }
+  __device__ __forceinline__ int stages(int cb) const { return 2 * (mode == kUpper ? min(nkb, 2 * cb + 2) : nkb); }
 };
 
 #define OZ_LD32(v, taddr)                                                                                      \
@@ -428,6 +451,10 @@ __global__ void __launch_bounds__(oz::NT, 1) oz_mma_kernel(OzTiles tl, OzOp a, O
         const int sc = er + oz_ex(b.raw[j]);
         double re = ldexp((double)hi[2 * q] + (double)lo[2 * q], sc) * alpha;
         double im = ldexp((double)hi[2 * q + 1] + (double)lo[2 * q + 1], sc) * alpha;
+        if (tl.mode == OzTiles::kHerm) {
+          if (row > j) continue;
+          if (row < j) C[(size_t)j * ldc + row] = make_double2(re, -im);
+        }
         double2* dst = &C[(size_t)row * ldc + j];
         if (accumulate) { const double2 cv = *dst; re += cv.x; im += cv.y; }
         *dst = make_double2(re, im);
