@@ -73,8 +73,10 @@ __global__ void ns_multiplier_kernel(double2* __restrict__ G, int m) {
 // of 2 m / 64 barriers and tile latencies. A pass at m = 2048 took 8.4 ms as 156
 // launches (recursive halving, a 64 x 64 base case of 130 us), 2.4 ms now; at
 // m = 512 1.5 -> 0.44 ms.
-// A non-positive pivot sets *status to 1 (the factorisation goes on with a tiny
-// one, so that no NaN is produced), a barrier that timed out to 2.
+// A non-positive pivot sets status[0] to 1 (the factorisation goes on with a tiny
+// one, so that no NaN is produced), a barrier that timed out to 2. status[1]
+// receives max |L^{-1}_ij|^2 (FP32 bits), the caller's measure of how far Y was
+// from orthogonal columns: 1 when they already were.
 // ---------------------------------------------------------------------------
 constexpr int CH = 64;                 // tile
 constexpr int CHP = CH + 2;            // padded row of a staged tile (16-byte rows)
@@ -206,6 +208,7 @@ __global__ void __launch_bounds__(256) cholqr_factor_kernel(const double2* __res
   // transposed and scaled, to W; the tile of W across the diagonal is zero
   auto finish = [&](int j, int k, const float2 (&r)[4][4]) {
     scales(k, k);
+    float mx = 0.0f;
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
@@ -213,14 +216,18 @@ __global__ void __launch_bounds__(256) cholqr_factor_kernel(const double2* __res
         const int gi = j * CH + 4 * ty + a, gk = k * CH + 4 * tx + b;
         if (gi >= m || gk >= m) continue;
         stcg(&Li[(size_t)gi * m + gk], r[a][b]);
+        mx = fmaxf(mx, r[a][b].x * r[a][b].x + r[a][b].y * r[a][b].y);
         if (gk <= gi) {
           const double d = s_d[4 * tx + b];
           W[(size_t)gk * m + gi] = make_double2(d * (double)r[a][b].x, -d * (double)r[a][b].y);
         }
         if (gk < gi) W[(size_t)gi * m + gk] = make_double2(0.0, 0.0);
       }
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if ((tid & 31) == 0) atomicMax(&status[1], __float_as_int(mx));
   };
 
+  if (bid == 0 && tid == 0) status[1] = 0;   // before the first barrier; written after it
   // A = fl32(D G D) + shift I, lower tiles
   for (int q = bid; q < nb * (nb + 1) / 2; q += nblk) {
     int i = 0, k = q;

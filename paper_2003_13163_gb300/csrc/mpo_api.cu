@@ -60,6 +60,7 @@ struct HostSync {   // pinned read-back of the last select + eigen-solve
   int tc_err;
   GridCtl eig[8];     // FP64 eigen-solves of the last mixed factorisation
   int chol_status;    // Cholesky QR pivot status of the last mixed factorisation
+  int chol_pass[2];   // status words after a Cholesky QR pass (cholqr_factor_kernel)
   int oz_err;         // the tensor-core FP64 GEMM's wait-limit flag
 };
 
@@ -609,26 +610,43 @@ static int mx_cholqr_pass(mpo_ctx* h, double2*& Y, double2*& spare, int rows, in
   return MPO_OK;
 }
 
-static int mx_cholqr(mpo_ctx* h, double2*& Y, double2*& spare, int rows, int m, int passes) {
+// Cholesky QR passes until Y's columns are orthogonal to the shift, at most
+// `passes`. A pass that found them nearly orthogonal already (max |L^{-1}_ij|^2 <=
+// 4 on the unit-diagonal Gram: every column keeps at least half of its length
+// beside the others) leaves a defect of a few shifts, 8 m u_32 each, and ends
+// the loop after `extra` more. In the subspace iteration the columns of X T are
+// close to the singular vectors after the first step, so most half steps need
+// one pass instead of three; the span, and so the result, does not depend on it.
+// The host waits for the two status words after each pass but the last (~20 us
+// against 0.15 ms (m = 128) .. 7 ms (m = 2048) for a pass saved).
+static int mx_cholqr(mpo_ctx* h, double2*& Y, double2*& spare, int rows, int m, int passes, int extra) {
   for (int p = 0; p < passes; ++p) {
     int rc = mx_cholqr_pass(h, Y, spare, rows, m);
     if (rc) return rc;
+    if (p + 1 + extra >= passes) continue;
+    CK(h, cudaMemcpyAsync(h->hs->chol_pass, h->mx_chst, 2 * sizeof(int), cudaMemcpyDeviceToHost, h->st));
+    CK(h, cudaStreamSynchronize(h->st));
+    float mu;
+    memcpy(&mu, &h->hs->chol_pass[1], sizeof mu);
+    if (mu <= 4.0f) passes = p + 1 + extra;
   }
   return MPO_OK;
 }
 
 // Subspace-iteration steps Q <- orth(X orth(X^H Q)) on Q (r x m). Each half
-// step is followed by three Cholesky QR passes, which hold the basis
+// step is followed by up to three Cholesky QR passes, which hold the basis
 // condition number near 1 although every product multiplies it by up to
-// sigma_1 / sigma_m (each pass divides it by about 30).
+// sigma_1 / sigma_m (each pass divides it by about 30); the last step's bases
+// take one pass more, because the FP32 Rayleigh-Ritz step needs them orthonormal.
+constexpr int kCholPasses = 3;
 static int mx_subspace_steps(mpo_ctx* h, const double2* X, int r, int c, int ldx, int m, int steps) {
-  const int passes = 3;
   for (int it = 0; it < steps; ++it) {
+    const int extra = it + 1 == steps ? 1 : 0;
     CK(h, mx_gemm(h, c, m, r, X, ldx, 1, h->mx_Q, m, 0, h->mx_T, m));     // T = X^H Q (c x m)
-    int rc = mx_cholqr(h, h->mx_T, h->mx_B, c, m, passes);
+    int rc = mx_cholqr(h, h->mx_T, h->mx_B, c, m, kCholPasses, extra);
     if (rc) return rc;
     CK(h, mx_gemm(h, r, m, c, X, ldx, 0, h->mx_T, m, 0, h->mx_Q, m));     // Q = X T (r x m)
-    rc = mx_cholqr(h, h->mx_Q, h->mx_Q2, r, m, passes);
+    rc = mx_cholqr(h, h->mx_Q, h->mx_Q2, r, m, kCholPasses, extra);
     if (rc) return rc;
   }
   return MPO_OK;
@@ -670,7 +688,7 @@ static int msvd_select(mpo_ctx* h, double2* X, int r, int c, int ldx, int cap, b
       CK(h, cudaGetLastError());
     }
     CK(h, mx_gemm(h, r, m, c, X, ldx, 0, h->mx_T, m, 0, h->mx_Q, m));     // Q = X Omega
-    rc = mx_cholqr(h, h->mx_Q, h->mx_Q2, r, m, 3);
+    rc = mx_cholqr(h, h->mx_Q, h->mx_Q2, r, m, kCholPasses, 0);
     if (rc) return rc;
     steps = std::max(std::max(1, h->mx_steps), remembered > 0 ? remembered + 1 : 0);
     rc = mx_subspace_steps(h, X, r, c, ldx, m, steps);
@@ -681,7 +699,7 @@ static int msvd_select(mpo_ctx* h, double2* X, int r, int c, int ldx, int cap, b
   // estimated from the FP32 Ritz values as (w_m / w_cap)^steps; above 1e-7
   // the iteration takes the steps that bring the estimate to 1e-8 and the
   // FP32 step is repeated (the kept-theta error is about 2e-2 of the estimate)
-  for (;;) {
+  for (bool reorth = false;;) {
     // the FP32 solve runs on M = Q^H X T (m x m; T the orthonormal basis of
     // the last half step, so M M^H = Q^H X X^H Q up to the iteration's
     // residual) rather than on B = Q^H X (m x c), and stops at relative
@@ -724,8 +742,14 @@ static int msvd_select(mpo_ctx* h, double2* X, int r, int c, int ldx, int cap, b
     CK(h, cudaStreamSynchronize(h->st));
     rc = msvd_status(h);
     if (rc) return rc;
-    if (!(std::max(rd[2], rd[3]) <= 1e-3))
-      return fail(h, MPO_ERR_NOCONV, "subspace basis not orthonormal after Cholesky QR");
+    if (!(std::max(rd[2], rd[3]) <= 1e-3)) {
+      if (reorth) return fail(h, MPO_ERR_NOCONV, "subspace basis not orthonormal after Cholesky QR");
+      reorth = true;               // every pass on both bases, then the FP32 step again
+      rc = mx_cholqr(h, h->mx_T, h->mx_B, c, m, kCholPasses, kCholPasses);
+      if (!rc) rc = mx_cholqr(h, h->mx_Q, h->mx_Q2, r, m, kCholPasses, kCholPasses);
+      if (rc) return rc;
+      continue;
+    }
     const double rho2 = rd[0] > 0.0 ? std::max(0.0, rd[1]) / rd[0] : 0.0;
     if (steps >= kMixedMaxSteps || rho2 <= 0.0 || std::pow(rho2, steps) <= 1e-7) break;
     const int need = rho2 < 1.0 ? (int)std::ceil(std::log(1e-8) / std::log(rho2)) : kMixedMaxSteps;
@@ -939,15 +963,9 @@ constexpr int kMovePasses = 5;
 static int mx_isometry(mpo_ctx* h, double2*& Y, int rows, int r, bool* ok) {
   double2* sp = h->mx_Q2;
   CK(h, cudaMemsetAsync(h->mx_chst, 0, sizeof(int), h->st));
-  int rc = mx_cholqr(h, Y, sp, rows, r, kMovePasses);
+  int rc = mx_cholqr(h, Y, sp, rows, r, kMovePasses, 1);
   if (rc) return rc;
-  rc = mx_newton_schulz(h, Y, sp, rows, r, 2);
-  if (rc) return rc;
-  CK(h, mx_gram(h, r, rows, Y, r, 1, h->mx_G, r));
-  CK(h, cudaMemsetAsync(h->scal + 3, 0, sizeof(double), h->st));
-  defect_kernel<<<grid_for((size_t)r * r, h->num_sms), 256, 0, h->st>>>(h->mx_G, r, h->scal + 3);
-  CK(h, cudaGetLastError());
-  rc = mx_newton_schulz(h, Y, sp, rows, r, 1);
+  rc = mx_newton_schulz(h, Y, sp, rows, r, 3, h->scal + 3);   // the defect entering the third step -> scal[3]
   if (rc) return rc;
   double defect = 1.0;
   CK(h, cudaMemcpyAsync(&defect, h->scal + 3, sizeof(double), cudaMemcpyDeviceToHost, h->st));
@@ -1446,7 +1464,7 @@ static bool alloc_factor_ws(mpo_ctx* h, int m, int ccap, size_t bj_nch) {
     ok = ok && alloc((void**)&h->mx_Q0, (size_t)m * mm * sizeof(double2));
     ok = ok && alloc((void**)&h->mx_A32, mm * mm * sizeof(float2));
     ok = ok && alloc((void**)&h->mx_Li32, mm * mm * sizeof(float2));
-    ok = ok && alloc((void**)&h->mx_chst, sizeof(int));
+    ok = ok && alloc((void**)&h->mx_chst, 2 * sizeof(int));
     ok = ok && cudaMemsetAsync(h->ctl, 0, sizeof(GridCtl), h->st) == cudaSuccess;
   }
   return ok;
