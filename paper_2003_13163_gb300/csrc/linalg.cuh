@@ -202,145 +202,25 @@ inline cudaError_t cgemm(cudaStream_t st, int M, int N, int K, const cplx<T>* A,
 // the rounding level of the input). The solve stops after a sweep without a
 // rotation; status = 1 if max_sweeps is reached first.
 //
-// Each round runs as three phases of one persistent cooperative launch:
+// Only the upper triangle is kept: entry (i, j) with i > j is read as the
+// conjugate of (j, i). A round runs as two phases of one persistent cooperative
+// launch:
 //   A: the round's rotation table, each pair by one thread of the grid, to
 //      the global table of this round's parity;                     barrier
-//   B (G <- G J, V <- V J): one warp per row, lanes over pairs;   barrier
-//   C (G <- J^H G): one warp per pair, lanes over columns;           barrier
+//   B: the round's pairs split G into 2 x 2 blocks G[p_a, q_a][p_b, q_b]; each
+//      block a <= b becomes J_a^H G_ab J_b, and V <- V J;              barrier
+// (work items of 32 blocks of one a, or 32 pairs of four rows of V, a warp each).
 // All G/V traffic uses L2-only loads/stores because other CTAs write it.
-// The FP64 unit (2 FMA per clock and SM) bounds all three phases (m = 1088,
-// nearly diagonal: 303 ms with tables built by every CTA, 173 ms now), so the work
-// is spread evenly over the SMs: a rotation costs ~200 FP64 instructions
-// (hypot, square roots, divisions), which every CTA repeated for all m / 2
-// pairs of a round when the table was built redundantly; and warp w of CTA b
-// takes items w gridDim + b, so that fewer items than warps still reach every
-// SM.
+// What bounds it: the FP64 unit (2 FMA per clock and SM) from m ~ 500, the two
+// barriers and the rotation parameters below. Updating both triangles by rows
+// and then by columns, with a third barrier, took 1.5 times the FP64 work; a
+// table built by every CTA, with ~200 FP64 instructions per rotation, 6 us per
+// round. Nearly diagonal m = 1088: 303 -> 111 ms, m = 320 18.6 -> 9.1, m = 128 5.0 -> 3.5.
 // ---------------------------------------------------------------------------
 template <typename T> struct JRot { T c, s, ur, ui; };
 
 __device__ __forceinline__ int rr_player(int pos, int r, int N) {
   return pos == 0 ? 0 : 1 + ((pos - 1 + r) % (N - 1));
-}
-
-template <typename T>
-__global__ void __launch_bounds__(256) jacobi_kernel(cplx<T>* G, int m, cplx<T>* V, T* w, JRot<T>* table, GridCtl* ctl,
-                                                      int max_sweeps, T tol_rel, T floor_rel, long long timeout_ns) {
-  extern __shared__ unsigned char jsmem[];
-  JRot<T>* rot = reinterpret_cast<JRot<T>*>(jsmem);
-  __shared__ T s_red[32];
-  const int N = m + (m & 1), npairs = N / 2;
-  const unsigned nblk = gridDim.x;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nwarp_blk = blockDim.x >> 5;
-  const long gwarp = (long)warp * nblk + blockIdx.x, nwarps = (long)nblk * nwarp_blk;
-  const size_t gtid = (size_t)blockIdx.x * blockDim.x + threadIdx.x, gthreads = (size_t)nblk * blockDim.x;
-
-  // V = I
-  for (size_t e = gtid; e < (size_t)m * m; e += gthreads) {
-    size_t r = e / m, c = e % m;
-    stcg(&V[e], mk<T>(r == c ? T(1) : T(0), T(0)));
-  }
-  // scale = max_i |G_ii| (each CTA redundantly)
-  T loc = T(0);
-  for (int i = threadIdx.x; i < m; i += blockDim.x) loc = fmax(loc, fabs(ldcg(&G[(size_t)i * m + i]).x));
-  for (int o = 16; o > 0; o >>= 1) loc = fmax(loc, __shfl_xor_sync(0xffffffffu, loc, o));
-  if (lane == 0) s_red[warp] = loc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    T mx = T(0);
-    for (int i = 0; i < nwarp_blk; ++i) mx = fmax(mx, s_red[i]);
-    s_red[0] = mx;
-  }
-  __syncthreads();
-  const T floor_abs = floor_rel * s_red[0];
-  if (!grid_barrier(ctl, nblk, timeout_ns)) return;
-
-  int sweep = 0;
-  bool converged = (m <= 1);
-  for (; sweep < max_sweeps && !converged; ++sweep) {
-    long sweep_active = 0;
-    for (int r = 0; r < N - 1; ++r) {
-      // ---- phase A: rotation table -------------------------------------
-      // two tables in turn: a CTA that is already in the next round writes
-      // the other one while slower CTAs still read this one
-      JRot<T>* tab = table + (size_t)((sweep * (N - 1) + r) & 1) * npairs;
-      for (long pi = blockIdx.x + (long)threadIdx.x * nblk; pi < npairs; pi += (long)nblk * blockDim.x) {
-        int p = rr_player((int)pi, r, N), q = rr_player(N - 1 - (int)pi, r, N);
-        if (p > q) { int t_ = p; p = q; q = t_; }
-        JRot<T> R; R.c = T(1); R.s = T(0); R.ur = T(1); R.ui = T(0);
-        if (q < m) {
-          const T a = ldcg(&G[(size_t)p * m + p]).x, b = ldcg(&G[(size_t)q * m + q]).x;
-          const cplx<T> g = ldcg(&G[(size_t)p * m + q]);
-          const T ag = hypot(g.x, g.y);
-          const T thr = fmax(tol_rel * sqrt(fabs(a * b)), floor_abs);
-          if (ag > thr && ag > T(0)) {
-            const T zeta = (b - a) / (T(2) * ag);
-            T t;
-            if (fabs(zeta) > T(1) / eps_of<T>::value) t = T(0.5) / zeta;
-            else t = (zeta >= T(0) ? T(1) : T(-1)) / (fabs(zeta) + sqrt(T(1) + zeta * zeta));
-            const T c = T(1) / sqrt(T(1) + t * t);
-            R.c = c; R.s = t * c; R.ur = g.x / ag; R.ui = g.y / ag;
-          }
-        }
-        __stcg(&tab[pi].c, R.c); __stcg(&tab[pi].s, R.s); __stcg(&tab[pi].ur, R.ur); __stcg(&tab[pi].ui, R.ui);
-      }
-      // phase B rewrites the pivots (G_pp, G_qq, G_pq) that phase A reads:
-      // no CTA rotates before the whole table has been built from the same G
-      if (!grid_barrier(ctl, nblk, timeout_ns)) return;
-      int my_active = 0;
-      for (int pi = threadIdx.x; pi < npairs; pi += blockDim.x) {
-        JRot<T> R;
-        R.c = __ldcg(&tab[pi].c); R.s = __ldcg(&tab[pi].s); R.ur = __ldcg(&tab[pi].ur); R.ui = __ldcg(&tab[pi].ui);
-        rot[pi] = R;
-        if (R.s != T(0)) my_active = 1;
-      }
-      const int act = __syncthreads_or(my_active);   // identical in every CTA: the same table
-      if (act == 0) continue;
-      ++sweep_active;
-      // ---- phase B: column rotations, G <- G J and V <- V J ---------------
-      for (long row = gwarp; row < 2L * m; row += nwarps) {
-        cplx<T>* Rw = row < m ? G + (size_t)row * m : V + (size_t)(row - m) * m;
-        for (int pi = lane; pi < npairs; pi += 32) {
-          const JRot<T> R = rot[pi];
-          if (R.s == T(0)) continue;
-          int p = rr_player(pi, r, N), q = rr_player(N - 1 - pi, r, N);
-          if (p > q) { int t_ = p; p = q; q = t_; }
-          const cplx<T> x = ldcg(&Rw[p]), y = ldcg(&Rw[q]);
-          const cplx<T> uy = cmul<T>(mk<T>(R.ur, -R.ui), y);   // conj(u) y
-          stcg(&Rw[p], mk<T>(R.c * x.x - R.s * uy.x, R.c * x.y - R.s * uy.y));
-          stcg(&Rw[q], mk<T>(R.s * x.x + R.c * uy.x, R.s * x.y + R.c * uy.y));
-        }
-      }
-      if (!grid_barrier(ctl, nblk, timeout_ns)) return;
-      // ---- phase C: row rotations, G <- J^H G ----------------------------
-      for (long pi = gwarp; pi < npairs; pi += nwarps) {
-        const JRot<T> R = rot[pi];
-        if (R.s == T(0)) continue;
-        int p = rr_player((int)pi, r, N), q = rr_player(N - 1 - (int)pi, r, N);
-        if (p > q) { int t_ = p; p = q; q = t_; }
-        cplx<T>* Rp = G + (size_t)p * m;
-        cplx<T>* Rq = G + (size_t)q * m;
-        for (int j = lane; j < m; j += 32) {
-          const cplx<T> x = ldcg(&Rp[j]), y = ldcg(&Rq[j]);
-          const cplx<T> uy = cmul<T>(mk<T>(R.ur, R.ui), y);    // u y
-          cplx<T> np_ = mk<T>(R.c * x.x - R.s * uy.x, R.c * x.y - R.s * uy.y);
-          cplx<T> nq_ = mk<T>(R.s * x.x + R.c * uy.x, R.s * x.y + R.c * uy.y);
-          if (j == q) np_ = czero<T>();
-          if (j == p) { nq_ = czero<T>(); np_.y = T(0); }
-          if (j == q) nq_.y = T(0);
-          stcg(&Rp[j], np_);
-          stcg(&Rq[j], nq_);
-        }
-      }
-      if (!grid_barrier(ctl, nblk, timeout_ns)) return;
-    }
-    if (sweep_active == 0) converged = true;
-  }
-  for (size_t i = gtid; i < (size_t)m; i += gthreads) w[i] = ldcg(&G[i * m + i]).x;
-  if (gtid == 0) {
-    ctl->sweeps = sweep;
-    ctl->status = converged ? 0 : 1;
-  }
 }
 
 // ---------------------------------------------------------------------------
@@ -663,7 +543,7 @@ __device__ __forceinline__ bool osj_rotation(double a, double b, double gr, doub
   const double sc = osj_pow2(-e);
   const double x = gr * sc, y = gi * sc;
   const double g2 = fma(x, x, y * y);             // in [1, 8)
-  if (!(g2 > tol2 * ((a * sc) * (b * sc)))) return false;
+  if (!(g2 > tol2 * fabs((a * sc) * (b * sc)))) return false;
   const double inv = osj_rsqrt(g2);
   if (!(g2 * inv * osj_pow2(e) > floor_abs)) return false;
   const double zeta = ((b - a) * sc) * (0.5 * inv);
@@ -716,6 +596,163 @@ __device__ __forceinline__ void osj_rotate(cplx<T>& x, cplx<T>& y, T c, T s, T s
   const cplx<T> xn = mk<T>(fma(sui, y.y, fma(-sur, y.x, c * x.x)), fma(-sui, y.x, fma(-sur, y.y, c * x.y)));
   y = mk<T>(fma(-cui, y.y, fma(cur, y.x, s * x.x)), fma(cui, y.x, fma(cur, y.y, s * x.y)));
   x = xn;
+}
+
+// The two-sided solver (described at JRot).
+template <typename T>
+__global__ void __launch_bounds__(256) jacobi_kernel(cplx<T>* G, int m, cplx<T>* V, T* w, JRot<T>* table, GridCtl* ctl,
+                                                      int max_sweeps, T tol_rel, T floor_rel, long long timeout_ns) {
+  extern __shared__ unsigned char jsmem[];
+  JRot<T>* rot = reinterpret_cast<JRot<T>*>(jsmem);
+  __shared__ T s_red[32];
+  const int N = m + (m & 1), npairs = N / 2;
+  const unsigned nblk = gridDim.x;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nwarp_blk = blockDim.x >> 5;
+  const long gwarp = (long)warp * nblk + blockIdx.x, nwarps = (long)nblk * nwarp_blk;
+  const size_t gtid = (size_t)blockIdx.x * blockDim.x + threadIdx.x, gthreads = (size_t)nblk * blockDim.x;
+
+  // V = I
+  for (size_t e = gtid; e < (size_t)m * m; e += gthreads) {
+    size_t r = e / m, c = e % m;
+    stcg(&V[e], mk<T>(r == c ? T(1) : T(0), T(0)));
+  }
+  // scale = max_i |G_ii| (each CTA redundantly)
+  T loc = T(0);
+  for (int i = threadIdx.x; i < m; i += blockDim.x) loc = fmax(loc, fabs(ldcg(&G[(size_t)i * m + i]).x));
+  for (int o = 16; o > 0; o >>= 1) loc = fmax(loc, __shfl_xor_sync(0xffffffffu, loc, o));
+  if (lane == 0) s_red[warp] = loc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    T mx = T(0);
+    for (int i = 0; i < nwarp_blk; ++i) mx = fmax(mx, s_red[i]);
+    s_red[0] = mx;
+  }
+  __syncthreads();
+  const T floor_abs = floor_rel * s_red[0];
+  if (!grid_barrier(ctl, nblk, timeout_ns)) return;
+
+  auto ld = [&](int i, int j) -> cplx<T> {
+    return i < j ? ldcg(&G[(size_t)i * m + j]) : cconj<T>(ldcg(&G[(size_t)j * m + i]));
+  };
+  auto st = [&](int i, int j, cplx<T> v) {
+    if (i < j) stcg(&G[(size_t)i * m + j], v);
+    else stcg(&G[(size_t)j * m + i], cconj<T>(v));
+  };
+  // the work items of phase B: blocks (a, b) with b in chunk k and a <= b, then
+  // four rows of V by one chunk of pairs
+  const int nch = (npairs + 31) / 32;
+  long nblocks = 0;
+  for (int k = 0; k < nch; ++k) nblocks += min(npairs, 32 * (k + 1));
+  const long nitems = nblocks + (long)((m + 3) / 4) * nch;
+  const double tol2 = (double)tol_rel * (double)tol_rel;
+
+  int sweep = 0;
+  bool converged = (m <= 1);
+  for (; sweep < max_sweeps && !converged; ++sweep) {
+    long sweep_active = 0;
+    for (int r = 0; r < N - 1; ++r) {
+      // ---- phase A: rotation table -------------------------------------
+      // two tables in turn: a CTA that is already in the next round writes
+      // the other one while slower CTAs still read this one
+      JRot<T>* tab = table + (size_t)((sweep * (N - 1) + r) & 1) * npairs;
+      for (long pi = blockIdx.x + (long)threadIdx.x * nblk; pi < npairs; pi += (long)nblk * blockDim.x) {
+        int p = rr_player((int)pi, r, N), q = rr_player(N - 1 - (int)pi, r, N);
+        if (p > q) { int t_ = p; p = q; q = t_; }
+        JRot<T> R; R.c = T(1); R.s = T(0); R.ur = T(1); R.ui = T(0);
+        if (q < m) {
+          const T a = ldcg(&G[(size_t)p * m + p]).x, b = ldcg(&G[(size_t)q * m + q]).x;
+          const cplx<T> g = ldcg(&G[(size_t)p * m + q]);
+          double cs, sn, ur, ui;
+          if (osj_rotation((double)a, (double)b, (double)g.x, (double)g.y, tol2, (double)floor_abs, cs, sn, ur, ui)) {
+            R.c = (T)cs; R.s = (T)sn; R.ur = (T)ur; R.ui = (T)ui;
+          }
+        }
+        __stcg(&tab[pi].c, R.c); __stcg(&tab[pi].s, R.s); __stcg(&tab[pi].ur, R.ur); __stcg(&tab[pi].ui, R.ui);
+      }
+      // phase B rewrites the pivots (G_pp, G_qq, G_pq) that phase A reads:
+      // no CTA rotates before the whole table has been built from the same G
+      if (!grid_barrier(ctl, nblk, timeout_ns)) return;
+      int my_active = 0;
+      for (int pi = threadIdx.x; pi < npairs; pi += blockDim.x) {
+        JRot<T> R;
+        R.c = __ldcg(&tab[pi].c); R.s = __ldcg(&tab[pi].s); R.ur = __ldcg(&tab[pi].ur); R.ui = __ldcg(&tab[pi].ui);
+        rot[pi] = R;
+        if (R.s != T(0)) my_active = 1;
+      }
+      const int act = __syncthreads_or(my_active);   // identical in every CTA: the same table
+      if (act == 0) continue;
+      ++sweep_active;
+      // ---- phase B -------------------------------------------------------
+      for (long it = gwarp; it < nitems; it += nwarps) {
+        if (it < nblocks) {
+          int k = 0;
+          long a_ = it;
+          while (a_ >= min(npairs, 32 * (k + 1))) a_ -= min(npairs, 32 * ++k);
+          const int a = (int)a_, b = 32 * k + lane;
+          if (b >= npairs || a > b) continue;
+          const JRot<T> Ra = rot[a], Rb = rot[b];
+          if (Ra.s == T(0) && Rb.s == T(0)) continue;
+          int p = rr_player(a, r, N), q = rr_player(N - 1 - a, r, N);
+          if (p > q) { int t_ = p; p = q; q = t_; }
+          if (a == b) {              // the rotated pair itself: G_pq becomes an exact zero
+            const cplx<T> g = ldcg(&G[(size_t)p * m + q]);
+            const T d = Ra.s / Ra.c * (g.x * Ra.ur + g.y * Ra.ui);     // t |g|
+            stcg(&G[(size_t)p * m + p], mk<T>(ldcg(&G[(size_t)p * m + p]).x - d, T(0)));
+            stcg(&G[(size_t)q * m + q], mk<T>(ldcg(&G[(size_t)q * m + q]).x + d, T(0)));
+            stcg(&G[(size_t)p * m + q], czero<T>());
+            continue;
+          }
+          int x = rr_player(b, r, N), y = rr_player(N - 1 - b, r, N);
+          if (x > y) { int t_ = x; x = y; y = t_; }
+          const bool hq = q < m, hy = y < m;      // false for the index that sits out (odd m)
+          cplx<T> b00 = ld(p, x), b01 = hy ? ld(p, y) : czero<T>();
+          cplx<T> b10 = hq ? ld(q, x) : czero<T>(), b11 = hq && hy ? ld(q, y) : czero<T>();
+          if (Rb.s != T(0)) {        // columns: [x y] <- [c x - s conj(u) y, s x + c conj(u) y]
+            const T sur = Rb.s * Rb.ur, sui = -Rb.s * Rb.ui, cur = Rb.c * Rb.ur, cui = -Rb.c * Rb.ui;
+            osj_rotate<T>(b00, b01, Rb.c, Rb.s, sur, sui, cur, cui);
+            osj_rotate<T>(b10, b11, Rb.c, Rb.s, sur, sui, cur, cui);
+          }
+          if (Ra.s != T(0)) {        // rows: [x; y] <- [c x - s u y; s x + c u y]
+            const T sur = Ra.s * Ra.ur, sui = Ra.s * Ra.ui, cur = Ra.c * Ra.ur, cui = Ra.c * Ra.ui;
+            osj_rotate<T>(b00, b10, Ra.c, Ra.s, sur, sui, cur, cui);
+            osj_rotate<T>(b01, b11, Ra.c, Ra.s, sur, sui, cur, cui);
+          }
+          st(p, x, b00);
+          if (hy) st(p, y, b01);
+          if (hq) st(q, x, b10);
+          if (hq && hy) st(q, y, b11);
+        } else {
+          const long v = it - nblocks;
+          const int b = 32 * (int)(v % nch) + lane, row0 = 4 * (int)(v / nch);
+          if (b >= npairs) continue;
+          const JRot<T> R = rot[b];
+          if (R.s == T(0)) continue;
+          int p = rr_player(b, r, N), q = rr_player(N - 1 - b, r, N);
+          if (p > q) { int t_ = p; p = q; q = t_; }
+          const T sur = R.s * R.ur, sui = -R.s * R.ui, cur = R.c * R.ur, cui = -R.c * R.ui;
+          cplx<T> xs[4], ys[4];
+#pragma unroll
+          for (int h = 0; h < 4; ++h)
+            if (row0 + h < m) { xs[h] = ldcg(&V[(size_t)(row0 + h) * m + p]); ys[h] = ldcg(&V[(size_t)(row0 + h) * m + q]); }
+#pragma unroll
+          for (int h = 0; h < 4; ++h)
+            if (row0 + h < m) {
+              osj_rotate<T>(xs[h], ys[h], R.c, R.s, sur, sui, cur, cui);
+              stcg(&V[(size_t)(row0 + h) * m + p], xs[h]);
+              stcg(&V[(size_t)(row0 + h) * m + q], ys[h]);
+            }
+        }
+      }
+      if (!grid_barrier(ctl, nblk, timeout_ns)) return;
+    }
+    if (sweep_active == 0) converged = true;
+  }
+  for (size_t i = gtid; i < (size_t)m; i += gthreads) w[i] = ldcg(&G[i * m + i]).x;
+  if (gtid == 0) {
+    ctl->sweeps = sweep;
+    ctl->status = converged ? 0 : 1;
+  }
 }
 
 template <typename T, int E>

@@ -398,34 +398,36 @@ __global__ void hermitise_kernel(double2* __restrict__ H, int m) {
   }
 }
 
-// First-order correction of a partition of approximate eigenvectors
-// (one refinement step of Ogita & Aishima, Japan J. Indust. Appl. Math. 35
-// (2018), restricted to the coupling between the leading mp directions P and
-// the remaining ones R): with the approximate eigenvector matrix V (m x m),
-// S = V^H H V and G = V^H V (both FP64-accurate), R = I - G and
-// lambda_i = S_ii / (1 - R_ii), the columns i in P gain the components
-//   E_ji = (S_ji + lambda_i R_ji) / (lambda_i - lambda_j),   j in R,
-// which removes their error along R to first order; pairs whose relative gap
-// is below 1e-2 (P and R meet inside a cluster, only in the margin beyond the
-// kept directions) get the orthogonality term R_ji / 2 alone.
-// Output E ((m - mp) x mp, row j - mp, column i).
+// First-order correction of the leading approximate eigenvectors (one
+// refinement step of Ogita & Aishima, Japan J. Indust. Appl. Math. 35 (2018)):
+// with the approximate eigenvector matrix V (m x m), S = V^H H V and G = V^H V
+// (both FP64-accurate), R = I - G and lambda_i = S_ii / (1 - R_ii), the leading
+// columns i < mp gain
+//   E_ji = (S_ji + lambda_i R_ji) / (lambda_i - lambda_j)
+// of column j, which removes their error along it to first order. Towards the
+// remaining columns (j >= mp) that is what keeps the FP32 solve's couplings out
+// of the kept subspace; pairs with a relative gap below 1e-2 (inside a cluster
+// at the edge, only in the margin beyond the kept directions) get the
+// orthogonality term R_ji / 2 alone. Among the leading columns it saves the FP64
+// eigen-solve that follows a sweep; there a pair is taken where |E_ji| <= 1e-3, so
+// that V_P (I + E_PP) stays within reach of the Newton-Schulz steps, else R_ji / 2.
+// Output (m x mp): rows j < mp are I + E_PP, the others E_RP.
 __global__ void partition_correction_kernel(const double2* __restrict__ S, const double2* __restrict__ G, int m, int mp,
                                             double2* __restrict__ E) {
-  const size_t total = (size_t)(m - mp) * mp;
+  const size_t total = (size_t)m * mp;
   for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-    const int j = mp + (int)(e / mp), i = (int)(e % mp);
+    const int j = (int)(e / mp), i = (int)(e % mp);
+    if (i == j) { E[e] = make_double2(1.0, 0.0); continue; }
     const double li = S[(size_t)i * m + i].x / G[(size_t)i * m + i].x;
     const double lj = S[(size_t)j * m + j].x / G[(size_t)j * m + j].x;
     const double2 s = S[(size_t)j * m + i];
     const double2 g = G[(size_t)j * m + i];
     const double2 rji = make_double2(-g.x, -g.y);      // (I - G)_ji, j != i
     const double gap = li - lj;
-    double2 v;
-    if (fabs(gap) > 1e-2 * fmax(fabs(li), fabs(lj)))
-      v = make_double2((s.x + li * rji.x) / gap, (s.y + li * rji.y) / gap);
-    else
-      v = make_double2(0.5 * rji.x, 0.5 * rji.y);
-    E[e] = v;
+    const double2 num = make_double2(s.x + li * rji.x, s.y + li * rji.y);
+    const bool far = j < mp ? fmax(fabs(num.x), fabs(num.y)) <= 1e-3 * fabs(gap)
+                            : fabs(gap) > 1e-2 * fmax(fabs(li), fabs(lj));
+    E[e] = far ? make_double2(num.x / gap, num.y / gap) : make_double2(0.5 * rji.x, 0.5 * rji.y);
   }
 }
 

@@ -261,7 +261,7 @@ static cudaError_t ensure_dynamic_smem(const void* fn, int bytes) {
 
 template <typename T>
 static cudaError_t launch_jacobi(cudaStream_t st, cplx<T>* G, int m, cplx<T>* V, T* w, JRot<T>* table, GridCtl* ctl,
-                                 int max_sweeps, double timeout_s, int num_sms) {
+                                 int max_sweeps, double timeout_s, int num_sms, double floor = eps_of<T>::value) {
   const int N = m + (m & 1);
   const size_t smem = sizeof(JRot<T>) * (size_t)std::max(1, N / 2);
   cudaError_t e = ensure_dynamic_smem((const void*)jacobi_kernel<T>, (int)smem);
@@ -271,15 +271,14 @@ static cudaError_t launch_jacobi(cudaStream_t st, cplx<T>* G, int m, cplx<T>* V,
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const int coresident = per_sm * num_sms;
-  // one warp per row of G and V in phase B; small matrices spread their rows
-  // over as many SMs as there are pairs, large ones keep two CTAs per SM (one: 178.6 ms, two:
-  // 172.6 ms at m = 1088; more lengthen the barriers, the FP64 unit is busy)
-  const int want = std::max((2 * m + 7) / 8, N / 2);
+  // one CTA per work item of phase B while they are few, two CTAs per SM
+  // beyond (more lengthen the barriers and add nothing: the FP64 unit is busy)
+  const int nch = (N / 2 + 31) / 32, want = nch * (N / 2 + (m + 3) / 4);
   const int blocks = std::max(1, std::min(std::min(coresident, 2 * num_sms), want));
   e = cudaMemsetAsync(ctl, 0, sizeof(GridCtl), st);
   if (e != cudaSuccess) return e;
   const T tol_rel = std::is_same<T, double>::value ? (T)1e-14 : (T)2e-6;
-  const T floor_rel = eps_of<T>::value;
+  const T floor_rel = (T)floor;
   long long timeout_ns = (long long)(timeout_s * 1e9);
   void* args[] = {&G, &m, &V, &w, &table, &ctl, &max_sweeps, (void*)&tol_rel, (void*)&floor_rel, &timeout_ns};
   return cudaLaunchCooperativeKernel((const void*)jacobi_kernel<T>, dim3(blocks), dim3(256), args, smem, st);
@@ -457,6 +456,7 @@ static cudaError_t launch_block_jacobi(cudaStream_t st, cplx<T>* X, int r, int c
 // squared Frobenius norm of X (the Ritz values cover span(Q) only).
 // ---------------------------------------------------------------------------
 constexpr int kMixedMargin = 64;      // Ritz directions carried into the FP64 step beyond cap
+constexpr int kCorrectMin = 32;       // basis size from which an untruncated solve corrects its FP32 vectors too
 constexpr int kMixedMaxSteps = 24;    // cap on subspace-iteration steps of one factorisation
 constexpr int kMixedSteps = 4;        // steps before the first convergence check
 
@@ -775,24 +775,33 @@ static int msvd_select(mpo_ctx* h, double2* X, int r, int c, int ldx, int cap, b
                                                                                       h->mx_W);
     CK(h, cudaGetLastError());
   }
-  if (mp < m) {
+  const double2* Vp = h->mx_W;     // the mp leading columns, leading dimension ldv
+  int ldv = m;
+  if (mp < m || m >= kCorrectMin) {
     const double2* Bs = iterate ? h->mx_B : X;
     const int ldbs = iterate ? c : ldx;
     CK(h, mx_gemm(h, m, c, m, h->mx_W, m, 1, Bs, ldbs, 0, h->mx_T, c));        // V^H B (m x c)
-    CK(h, mx_gram(h, m, c, h->mx_T, c, 0, h->mx_G, m));      // S = V^H H V
-    CK(h, mx_gram(h, m, m, h->mx_W, m, 1, h->mx_V, m));      // G = V^H V
+    CK(h, mx_gram(h, m, c, h->mx_T, c, 0, h->mx_G, m));                         // S = V^H H V
+    CK(h, mx_gram(h, m, m, h->mx_W, m, 1, h->mx_V, m));                         // G = V^H V
     {
       ProfScope ps(h, PK_REFINE, 0.0, 3.0 * (double)m * mp * sizeof(double2));
-      partition_correction_kernel<<<grid_for((size_t)(m - mp) * mp, h->num_sms), 256, 0, h->st>>>(
-          h->mx_G, h->mx_V, m, mp, h->mx_B);
+      partition_correction_kernel<<<grid_for((size_t)m * mp, h->num_sms), 256, 0, h->st>>>(h->mx_G, h->mx_V, m, mp,
+                                                                                          h->mx_B);
       CK(h, cudaGetLastError());
     }
-    CK(h, mx_gemm(h, m, mp, m - mp, h->mx_W + mp, m, 0, h->mx_B, mp, 0, h->mx_W, m, 1.0, 1));   // V_P += V_R E
+    // V_P += V_R E_RP, which fixes the span of P, then V_P (I + E_PP) within it
+    // (I + E in one product would leave E_RP E_PP in the span)
+    if (mp < m)
+      CK(h, mx_gemm(h, m, mp, m - mp, h->mx_W + mp, m, 0, h->mx_B + (size_t)mp * mp, mp, 0, h->mx_W, m, 1.0, 1));
+    double2* out = iterate ? h->mx_V : Qp;
+    CK(h, mx_gemm(h, m, mp, mp, h->mx_W, m, 0, h->mx_B, mp, 0, out, mp));
+    Vp = out;
+    ldv = mp;
   }
   if (iterate) {
-    CK(h, mx_gemm(h, r, mp, m, h->mx_Q, m, 0, h->mx_W, m, 0, Qp, mp));
-  } else {
-    CK(h, cudaMemcpy2DAsync(Qp, (size_t)mp * sizeof(double2), h->mx_W, (size_t)m * sizeof(double2),
+    CK(h, mx_gemm(h, r, mp, m, h->mx_Q, m, 0, Vp, ldv, 0, Qp, mp));
+  } else if (Vp != Qp) {
+    CK(h, cudaMemcpy2DAsync(Qp, (size_t)mp * sizeof(double2), Vp, (size_t)ldv * sizeof(double2),
                             (size_t)mp * sizeof(double2), r, cudaMemcpyDeviceToDevice, h->st));
   }
   rc = mx_newton_schulz(h, Qp, Qsp, r, mp, 3);
@@ -805,8 +814,12 @@ static int msvd_select(mpo_ctx* h, double2* X, int r, int c, int ldx, int cap, b
     ProfScope ps(h, PK_EIG64, 13.3 * (double)mp * mp * mp, 3.0 * (double)mp * mp * sizeof(double2));
     hermitise_kernel<<<grid_for((size_t)mp * mp, h->num_sms), 256, 0, h->st>>>(h->mx_G, mp);
     CK(h, cudaGetLastError());
+    // couplings are rotated down to 1e-14 of their own pair's size as far as the
+    // kept values reach (cutoff 1e-7: lambda^2 >= 1e-14 of the largest): a floor
+    // of eps would leave those that the correction above has already brought
+    // below it
     CK(h, launch_jacobi<double>(h->st, h->mx_G, mp, h->mx_V, h->mx_w, h->mx_rot, &h->mx_eosctl->g, h->opts.eig_max_sweeps,
-                                h->opts.barrier_timeout_s, h->num_sms));
+                                h->opts.barrier_timeout_s, h->num_sms, 1e-24));
   }
   // left factor Q' V, stored as rows conj(column j) = V^H Q'^H; the rows
   // V^H B' = Lambda W^H go to X
