@@ -899,6 +899,237 @@ __global__ void __launch_bounds__(OSJ_NT) pair_jacobi_kernel(cplx<T>* X, int r, 
 }
 
 // ---------------------------------------------------------------------------
+// Row Jacobi in FP32 on blocks of RB rows, the precision form's Rayleigh-Ritz
+// solve: the same rotations as above, row pair by row pair (no Gram of the block,
+// so the relative accuracy of the row method stays), but a CTA holds two blocks
+// in registers and rotates all RB^2 pairs between them (at the first round of a
+// sweep the pairs inside each block too) before it writes them back.
+// Why: at 2048 rows the pair form reads and writes X and U once per round,
+// 128 MB at 13 TB/s of L2, and passes a grid barrier for each; blocks of four
+// divide both by four. RB pairs are rotated at a time: their 4 RB sums are
+// reduced together and one lane each forms the rotations, in FP32 (c and 1 / |g|
+// by one Newton step, so c^2 + s^2 and |u| are 1 to FP32 rounding; the solve's
+// vectors are orthonormalised in FP64 afterwards). U takes the recorded
+// rotations in one pass. Rows of up to 256 E columns.
+// Measured in the precision form, pair kernel -> this one: 2048 rows 166 -> 82 ms,
+// 512 rows 18.5 -> 5.3 ms.
+// ---------------------------------------------------------------------------
+constexpr int QJ_NT = 256;
+
+__device__ __forceinline__ float qj_rsqrt(float x) {
+  const float y = rsqrtf(x);
+  return fmaf(0.5f * y, fmaf(-x * y, y, 1.0f), y);
+}
+
+// osj_rotation in FP32.
+__device__ __forceinline__ bool qj_rotation(float a, float b, float gr, float gi, float tol2, float floor_abs, float& c,
+                                            float& s, float& ur, float& ui) {
+  const int er = (__float_as_int(gr) >> 23) & 0xFF, ei = (__float_as_int(gi) >> 23) & 0xFF;
+  const int e = max(er, ei) - 127;
+  if (e <= -126 || e >= 126) return false;
+  const float sc = __int_as_float((127 - e) << 23);
+  const float x = gr * sc, y = gi * sc;
+  const float g2 = fmaf(x, x, y * y);
+  if (!(g2 > tol2 * ((a * sc) * (b * sc)))) return false;
+  const float inv = qj_rsqrt(g2);
+  if (!(g2 * inv * __int_as_float((127 + e) << 23) > floor_abs)) return false;
+  const float z = ((b - a) * sc) * (0.5f * inv), az = fabsf(z);
+  if (!(az < 3e38f)) return false;
+  float t = az > 1e18f ? 0.5f / az : 1.0f / (az + sqrtf(fmaf(az, az, 1.0f)));
+  if (z < 0.0f) t = -t;
+  c = qj_rsqrt(fmaf(t, t, 1.0f));
+  s = t * c;
+  ur = x * inv;
+  ui = y * inv;
+  return s != 0.0f;
+}
+
+template <int RB, int E>
+__global__ void __launch_bounds__(QJ_NT) quad_jacobi_kernel(float2* X, int r, int c, int ldx, float2* Ut, float* w, OSCtl* ctl,
+                                                            int max_sweeps, float tol_rel, float floor_rel,
+                                                            long long timeout_ns) {
+  constexpr int NV = 4 * RB;                       // sums of one step
+  constexpr int NSTEP = 2 * RB - 1;                // steps of a round: RB - 1 inside the blocks, RB across
+  __shared__ float part[QJ_NT / 32][NV];
+  __shared__ float4 s_rot[NSTEP][RB];              // c, s, u; s = 0: no rotation
+  __shared__ int s_any;
+  const int nb = (r + RB - 1) / RB, N = nb + (nb & 1), npairs = N / 2;
+  const unsigned nblk = gridDim.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const size_t gtid = (size_t)blockIdx.x * QJ_NT + tid, gthreads = (size_t)nblk * QJ_NT;
+  if (max_sweeps > 64) max_sweeps = 64;
+
+  for (size_t e = gtid; e < (size_t)r * r; e += gthreads) {
+    const size_t i = e / r, j = e % r;
+    stcg(&Ut[e], make_float2(i == j ? 1.0f : 0.0f, 0.0f));
+  }
+  auto norms = [&]() {
+    for (long i = gtid >> 5; i < r; i += (long)(gthreads >> 5)) {
+      float s = 0.0f;
+      for (int j = lane; j < c; j += 32) {
+        const float2 x = ldcg(&X[(size_t)i * ldx + j]);
+        s = fmaf(x.x, x.x, fmaf(x.y, x.y, s));
+      }
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == 0) __stcg(&w[i], s);
+    }
+  };
+  norms();
+  if (!grid_barrier(&ctl->g, nblk, timeout_ns)) return;
+  const float floor_abs = floor_rel * block_max<float>(w, r);
+  const float tol2 = tol_rel * tol_rel;
+
+  int sweep = 0;
+  bool converged = (r <= 1);
+  for (; sweep < max_sweeps && !converged; ++sweep) {
+    const int nround = N > 1 ? N - 1 : 1;
+    for (int rd = 0; rd < nround; ++rd) {
+      for (int pi = blockIdx.x; pi < npairs; pi += nblk) {
+        const int P = rr_player(pi, rd, N), Q = rr_player(N - 1 - pi, rd, N);
+        if ((P >= nb || Q >= nb) && rd > 0) continue;      // sits out (its own rows are rotated at the first round)
+        auto row_of = [&](int i) -> int {                  // block row i of the CTA; r if there is none
+          const int g = i < RB ? P * RB + i : Q * RB + (i - RB);
+          return g < r ? g : r;
+        };
+        float2 x[2 * RB][E];
+        auto load = [&](const float2* M, int ld, int n) {
+#pragma unroll
+          for (int i = 0; i < 2 * RB; ++i) {
+            const int g = row_of(i);
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+              const int j = tid + QJ_NT * e;
+              x[i][e] = g < r && j < n ? ldcg(&M[(size_t)g * ld + j]) : make_float2(0.f, 0.f);
+            }
+          }
+        };
+        auto store = [&](float2* M, int ld, int n) {
+#pragma unroll
+          for (int i = 0; i < 2 * RB; ++i) {
+            const int g = row_of(i);
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+              const int j = tid + QJ_NT * e;
+              if (g < r && j < n) stcg(&M[(size_t)g * ld + j], x[i][e]);
+            }
+          }
+        };
+        load(X, ldx, c);
+        if (tid == 0) s_any = 0;
+        // step k < RB - 1: pairs (i, i ^ (k + 1)) inside both blocks; then
+        // (i, RB + (i ^ (k - RB + 1))) across. Pair q's rows: first, second
+#pragma unroll
+        for (int k = 0; k < NSTEP; ++k) {
+          constexpr int H = RB / 2;
+          if (k < RB - 1 && rd > 0) continue;
+          auto first = [&](int q) -> int {
+            if (k >= RB - 1) return q;
+            const int blk = q / H, n = q % H, m = k + 1;   // the n-th i with i < i ^ m
+            int cnt = 0, f = 0;
+#pragma unroll
+            for (int i = 0; i < RB; ++i)
+              if (i < (i ^ m)) { if (cnt == n) f = i; ++cnt; }
+            return blk * RB + f;
+          };
+          auto second = [&](int q) -> int { return k >= RB - 1 ? RB + (q ^ (k - RB + 1)) : first(q) ^ (k + 1); };
+          float v[NV];
+#pragma unroll
+          for (int q = 0; q < RB; ++q) {
+            float a = 0.f, b = 0.f, gr = 0.f, gi = 0.f;
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+              const float2 p0 = x[first(q)][e], p1 = x[second(q)][e];
+              a = fmaf(p0.x, p0.x, fmaf(p0.y, p0.y, a));
+              b = fmaf(p1.x, p1.x, fmaf(p1.y, p1.y, b));
+              gr = fmaf(p0.x, p1.x, fmaf(p0.y, p1.y, gr));
+              gi = fmaf(p0.y, p1.x, fmaf(-p0.x, p1.y, gi));
+            }
+            v[4 * q] = a; v[4 * q + 1] = b; v[4 * q + 2] = gr; v[4 * q + 3] = gi;
+          }
+          // halves: after the step of width h a lane keeps the values whose bit agrees with its own
+          int o = 16;
+#pragma unroll
+          for (int h = NV / 2; h >= 1; h >>= 1, o >>= 1) {
+            const bool up = lane & o;
+#pragma unroll
+            for (int i = 0; i < h; ++i) {
+              const float keep = up ? v[i + h] : v[i], send = up ? v[i] : v[i + h];
+              v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+          }
+          constexpr int LPV = 32 / NV;      // lanes that share a value now
+#pragma unroll
+          for (int h = LPV / 2; h >= 1; h >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], h);
+          if ((lane % LPV) == 0) part[warp][lane / LPV] = v[0];
+          __syncthreads();
+          if (warp == 0) {
+            float t = 0.f;
+#pragma unroll
+            for (int u = 0; u < QJ_NT / 32; ++u) t += part[u][lane % NV];
+            const int q = lane % RB;
+            const float a = __shfl_sync(0xffffffffu, t, 4 * q), b = __shfl_sync(0xffffffffu, t, 4 * q + 1);
+            const float gr = __shfl_sync(0xffffffffu, t, 4 * q + 2), gi = __shfl_sync(0xffffffffu, t, 4 * q + 3);
+            float cs = 1.f, sn = 0.f, ur = 1.f, ui = 0.f;
+            const bool on = qj_rotation(a, b, gr, gi, tol2, floor_abs, cs, sn, ur, ui);
+            if (lane < RB) s_rot[k][q] = on ? make_float4(cs, sn, ur, ui) : make_float4(1.f, 0.f, 1.f, 0.f);
+            const unsigned any = __ballot_sync(0xffffffffu, on && lane < RB);
+            if (lane == 0 && any) {
+              s_any = 1;
+              atomicAdd(&ctl->active[sweep], __popc(any));
+            }
+          }
+          __syncthreads();
+#pragma unroll
+          for (int q = 0; q < RB; ++q) {
+            const float4 R = s_rot[k][q];
+            if (R.y == 0.f) continue;
+            const float sur = R.y * R.z, sui = R.y * R.w, cur = R.x * R.z, cui = R.x * R.w;
+#pragma unroll
+            for (int e = 0; e < E; ++e) osj_rotate<float>(x[first(q)][e], x[second(q)][e], R.x, R.y, sur, sui, cur, cui);
+          }
+        }
+        if (s_any) {
+          store(X, ldx, c);
+          load(Ut, r, r);
+#pragma unroll
+          for (int k = 0; k < NSTEP; ++k) {
+            constexpr int H = RB / 2;
+            if (k < RB - 1 && rd > 0) continue;
+            auto first = [&](int q) -> int {
+              if (k >= RB - 1) return q;
+              const int blk = q / H, n = q % H, m = k + 1;
+              int cnt = 0, f = 0;
+#pragma unroll
+              for (int i = 0; i < RB; ++i)
+                if (i < (i ^ m)) { if (cnt == n) f = i; ++cnt; }
+              return blk * RB + f;
+            };
+            auto second = [&](int q) -> int { return k >= RB - 1 ? RB + (q ^ (k - RB + 1)) : first(q) ^ (k + 1); };
+#pragma unroll
+            for (int q = 0; q < RB; ++q) {
+              const float4 R = s_rot[k][q];
+              if (R.y == 0.f) continue;
+              const float sur = R.y * R.z, sui = -R.y * R.w, cur = R.x * R.z, cui = -R.x * R.w;   // U <- U J: the conjugate phase
+#pragma unroll
+              for (int e = 0; e < E; ++e) osj_rotate<float>(x[first(q)][e], x[second(q)][e], R.x, R.y, sur, sui, cur, cui);
+            }
+          }
+          store(Ut, r, r);
+        }
+        __syncthreads();            // s_any and s_rot are free for the next pair
+      }
+      if (!grid_barrier(&ctl->g, nblk, timeout_ns)) return;
+    }
+    if (atomicAdd(&ctl->active[sweep], 0) == 0) converged = true;
+  }
+  norms();
+  if (gtid == 0) {
+    ctl->g.sweeps = sweep;
+    ctl->g.status = converged ? 0 : 1;
+  }
+}
+
+// ---------------------------------------------------------------------------
 // LQ preconditioning of the complex128 SVD (Drmac & Veselic, SIAM J. Matrix
 // Anal. Appl. 29 (2008), without pivoting): with A = L Q (L r x r lower
 // triangular, Q with orthonormal rows) the row Jacobi runs on R = L^H instead

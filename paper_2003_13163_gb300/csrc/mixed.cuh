@@ -42,14 +42,14 @@ __global__ void promote_columns_kernel(const float2* __restrict__ Ut, int r, con
   }
 }
 
-// G (m x m) <- (3 I - G) / 2 in place: the Newton-Schulz multiplier
+// G (m x m) <- (I - G) / 2 in place: the Newton-Schulz correction
 // (Higham, Functions of Matrices, Sec. 8.3).
 __global__ void ns_multiplier_kernel(double2* __restrict__ G, int m) {
   const size_t total = (size_t)m * m;
   for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
     const int i = (int)(e / m), j = (int)(e % m);
     double2 g = G[e];
-    g.x = (i == j ? 1.5 : 0.0) - 0.5 * g.x;
+    g.x = 0.5 * ((i == j ? 1.0 : 0.0) - g.x);
     g.y = -0.5 * g.y;
     G[e] = g;
   }

@@ -352,6 +352,37 @@ static cudaError_t launch_pair_jacobi(cudaStream_t st, cplx<T>* X, int r, int c,
   return cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(OSJ_NT), args, 0, st);
 }
 
+// Rows from which the FP32 solve works on blocks of rows.
+constexpr int kQuadMinRows = 32;
+
+// The precision form's FP32 row Jacobi: blocks of four rows while two of them fit
+// a CTA's registers (up to 2048 columns), of two up to 4096, else row pairs.
+static cudaError_t launch_fp32_jacobi(cudaStream_t st, float2* X, int r, int c, int ldx, float2* Ut, float* w, OSCtl* ctl,
+                                      int max_sweeps, double timeout_s, int num_sms, double tol_min) {
+  const int n = std::max(r, c);
+  if (n > 16 * QJ_NT || r < kQuadMinRows)
+    return launch_pair_jacobi<float>(st, X, r, c, ldx, Ut, w, ctl, max_sweeps, timeout_s, num_sms, tol_min);
+  const int rb = n > 8 * QJ_NT ? 2 : 4;
+  const void* fn = n <= QJ_NT ? (const void*)quad_jacobi_kernel<4, 1>
+                   : n <= 2 * QJ_NT ? (const void*)quad_jacobi_kernel<4, 2>
+                   : n <= 4 * QJ_NT ? (const void*)quad_jacobi_kernel<4, 4>
+                   : n <= 8 * QJ_NT ? (const void*)quad_jacobi_kernel<4, 8>
+                                    : (const void*)quad_jacobi_kernel<2, 16>;
+  int per_sm = 0;
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, QJ_NT, 0);
+  if (e != cudaSuccess) return e;
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  const int nb = (r + rb - 1) / rb;
+  const int blocks = std::max(1, std::min(per_sm * num_sms, (nb + 1) / 2));
+  e = cudaMemsetAsync(ctl, 0, sizeof(OSCtl), st);
+  if (e != cudaSuccess) return e;
+  float tol_rel = (float)std::max(tol_min, 2.0 * eps_of<float>::value * std::sqrt((double)std::max(c, 1)));
+  float floor_rel = eps_of<float>::value * eps_of<float>::value;
+  long long timeout_ns = (long long)(timeout_s * 1e9);
+  void* args[] = {&X, &r, &c, &ldx, &Ut, &w, &ctl, &max_sweeps, &tol_rel, &floor_rel, &timeout_ns};
+  return cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(QJ_NT), args, 0, st);
+}
+
 // Rows below which the LQ step costs more than the sweeps it saves.
 constexpr int kLqMinRows = 8;
 
@@ -548,7 +579,11 @@ static cudaError_t mx_gram(mpo_ctx* h, int n, int k, const double2* Y, int ldy, 
 // (Newton-Schulz iteration for the orthonormal polar factor, Higham,
 // Functions of Matrices, Sec. 8.3): each step squares the defect
 // |Y^H Y - I|, so a basis orthonormal to ~1e-3 reaches FP64 rounding in four
-// steps. The result is left in Y (spare is scratch; the two are swapped).
+// steps. A step adds Y E, E = (I - Y^H Y) / 2, to Y: the split product's error
+// of 2^-42 then scales with the small E instead of with Y (an isometry defect
+// of 2e-12 came from forming Y (3 I - Y^H Y) / 2 in one product). That product
+// splits Y before it writes C, so it adds to Y in place; the SIMT one adds to
+// a copy (the two buffers are then swapped).
 static int mx_newton_schulz(mpo_ctx* h, double2*& Y, double2*& spare, int rows, int m, int iters,
                             double* defect_dev = nullptr) {
   for (int it = 0; it < iters; ++it) {
@@ -563,8 +598,13 @@ static int mx_newton_schulz(mpo_ctx* h, double2*& Y, double2*& spare, int rows, 
       ns_multiplier_kernel<<<grid_for((size_t)m * m, h->num_sms), 256, 0, h->st>>>(h->mx_G, m);
       CK(h, cudaGetLastError());
     }
-    CK(h, mx_gemm(h, rows, m, m, Y, m, 0, h->mx_G, m, 0, spare, m));
-    std::swap(Y, spare);
+    if (h->use_oz && oz_worth(rows, m, m)) {
+      CK(h, mx_gemm(h, rows, m, m, Y, m, 0, h->mx_G, m, 0, Y, m, 1.0, 1));
+    } else {
+      CK(h, cudaMemcpyAsync(spare, Y, (size_t)rows * m * sizeof(double2), cudaMemcpyDeviceToDevice, h->st));
+      CK(h, mx_gemm(h, rows, m, m, Y, m, 0, h->mx_G, m, 0, spare, m, 1.0, 1));
+      std::swap(Y, spare);
+    }
   }
   return MPO_OK;
 }
@@ -723,7 +763,7 @@ static int msvd_select(mpo_ctx* h, double2* X, int r, int c, int ldx, int cap, b
     {
       const double fm = m, fc = c1;
       ProfScope ps(h, disc ? PK_SVD : PK_SVD_SWEEP, 4.0 * fm * fm * fc, (2.0 * fm * fc + fm * fm) * sizeof(float2));
-      CK(h, launch_pair_jacobi<float>(h->st, h->mx_a32, m, c1, c1, h->mx_ut32, h->mx_w32, h->osctl,
+      CK(h, launch_fp32_jacobi(h->st, h->mx_a32, m, c1, c1, h->mx_ut32, h->mx_w32, h->osctl,
                                    h->opts.eig_max_sweeps, h->opts.barrier_timeout_s, h->num_sms, 3e-5));
     }
     {
