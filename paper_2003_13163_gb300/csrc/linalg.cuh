@@ -758,7 +758,7 @@ __global__ void __launch_bounds__(256) jacobi_kernel(cplx<T>* G, int m, cplx<T>*
 template <typename T, int E>
 __global__ void __launch_bounds__(OSJ_NT) pair_jacobi_kernel(cplx<T>* X, int r, int c, int ldx, cplx<T>* Ut, T* w,
                                                              OSCtl* ctl, int max_sweeps, T tol_rel, T floor_rel,
-                                                             long long timeout_ns) {
+                                                             int given_u, long long timeout_ns) {
   __shared__ T part[4][4];
   __shared__ OsjRot<T> s_rot;
   const int N = r + (r & 1), npairs = N / 2;
@@ -768,7 +768,7 @@ __global__ void __launch_bounds__(OSJ_NT) pair_jacobi_kernel(cplx<T>* X, int r, 
   const bool regs = c <= OSJ_NT * E, uregs = r <= OSJ_NT * E;   // the rows fit the registers
   if (max_sweeps > 64) max_sweeps = 64;
 
-  for (size_t e = gtid; e < (size_t)r * r; e += gthreads) {
+  for (size_t e = gtid; e < (size_t)r * r && !given_u; e += gthreads) {   // else Ut already holds a U to rotate on
     const size_t i = e / r, j = e % r;
     stcg(&Ut[e], mk<T>(i == j ? T(1) : T(0), T(0)));
   }
@@ -1144,7 +1144,58 @@ __global__ void __launch_bounds__(QJ_NT) quad_jacobi_kernel(float2* X, int r, in
 // (one reduction for both), so nothing waits for a broadcast.
 // Truncated SVD, row Jacobi on A -> with the LQ step: 128 x 128 13.7 -> 8.5 ms,
 // 256 x 256 52 -> 21 ms, 577 x 600 260 -> 119 ms, 1024 x 1024 1244 -> 539 ms.
+//
+// FP32 start. From kPreMinRows rows on, the FP32 solver first runs on fl32(R)
+// (scaled to a largest entry near 1), and the FP64 solve starts from W^H R and W,
+// W the FP32 left factor made orthonormal to FP64 rounding: with E = (I - W^H W)
+// / 2, W (I + E + 3/2 E^2 + 5/2 E^3) is off by 35/8 E^4 (E is at most ~5e-5, the
+// drift of the FP32 rotations). The FP64
+// unit runs at 1/64 of the FP32 rate, so its sweeps are what the solve costs, and
+// five (the last of them quiet) remain of eleven; it stops by the same test as
+// without the start. Truncated SVD, LQ only -> with the start: 64 x 64 4.1 -> 2.8 ms,
+// 256 x 256 21.5 -> 17.5 ms, 577 x 600 116 -> 88 ms, 1024 x 1024 542 -> 350 ms;
+// 768 x 1024 with a spectrum over three decades 253 -> 115 ms (FP64 solve 57, FP32
+// 21, products 16, LQ step and rows 21).
 // ---------------------------------------------------------------------------
+// *out = the largest biased exponent among the real and imaginary parts of a
+// matrix of n entries (zeroed before the launch).
+__global__ void __launch_bounds__(256) max_exp_kernel(const double2* __restrict__ R, size_t n, int* __restrict__ out) {
+  int v = 0;
+  for (size_t e = (size_t)blockIdx.x * 256 + threadIdx.x; e < n; e += (size_t)gridDim.x * 256) {
+    const double2 x = R[e];
+    v = max(v, max((int)((__double_as_longlong(x.x) >> 52) & 0x7FF), (int)((__double_as_longlong(x.y) >> 52) & 0x7FF)));
+  }
+  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+  if ((threadIdx.x & 31) == 0 && v > 0) atomicMax(out, v);
+}
+
+// out = fl32(R 2^-e), e the exponent found above (an all-zero R stays zero).
+__global__ void __launch_bounds__(256) scale_fp32_kernel(const double2* __restrict__ R, size_t n, const int* __restrict__ ex,
+                                                         float2* __restrict__ out) {
+  const int be = *ex;
+  const double sc = be > 0 && be < 2046 ? __longlong_as_double((long long)(2046 - be) << 52) : 1.0;   // 2^(1023 - be)
+  for (size_t e = (size_t)blockIdx.x * 256 + threadIdx.x; e < n; e += (size_t)gridDim.x * 256) {
+    const double2 x = R[e];
+    out[e] = make_float2((float)(x.x * sc), (float)(x.y * sc));
+  }
+}
+
+// out (c x r) = in (r x c)^T in FP64, 32 x 32 tiles through shared memory.
+template <typename S>
+__global__ void transpose_kernel(const S* __restrict__ in, int r, int c, double2* __restrict__ out) {
+  __shared__ double2 tile[32][33];
+  const int bx = blockIdx.x * 32, by = blockIdx.y * 32;
+  for (int yy = threadIdx.y; yy < 32; yy += blockDim.y) {
+    const int i = by + yy, j = bx + threadIdx.x;
+    if (i < r && j < c) { const S v = in[(size_t)i * c + j]; tile[yy][threadIdx.x] = make_double2((double)v.x, (double)v.y); }
+  }
+  __syncthreads();
+  for (int yy = threadIdx.y; yy < 32; yy += blockDim.y) {
+    const int j = bx + yy, i = by + threadIdx.x;
+    if (j < c && i < r) out[(size_t)j * r + i] = tile[threadIdx.x][yy];
+  }
+}
+
 // 1 / sqrt(x) for a normal positive x.
 __device__ __forceinline__ double lq_rsqrt(double x) {
   const int e = ((int)(__double_as_longlong(x) >> 52) - 1023) & ~1;
@@ -1288,13 +1339,13 @@ __global__ void __launch_bounds__(OSJ_NT) lq_kernel(const double2* __restrict__ 
 
 // Row j of the factorisation from the Jacobi result (Y rows Sigma U^H, Wt row j
 // = column j of W, w = sigma^2): X row j = sigma_j w_j^H Q = sigma_j [w_j^H 0]
-// H_{r-1} .. H_0, and Y row j <- conj(column j of U). One CTA per row; the row
+// H_{r-1} .. H_0, and Uc row j = conj(column j of U) (may be Y). One CTA per row; the row
 // stays in registers while the reflectors stream past (each is read ahead
 // while the previous one's dot product is reduced).
 template <int E>
 __global__ void __launch_bounds__(OSJ_NT) lq_apply_kernel(const double2* __restrict__ Z, int r, int c,
                                                           const double* __restrict__ f, const double2* __restrict__ zd,
-                                                          const double2* __restrict__ Wt, double2* __restrict__ Y,
+                                                          const double2* __restrict__ Wt, const double2* Y, double2* Uc,
                                                           const double* __restrict__ w, double2* __restrict__ X, int ldx) {
   __shared__ double part[2][2][4];
   const int j = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1386,7 +1437,7 @@ __global__ void __launch_bounds__(OSJ_NT) lq_apply_kernel(const double2* __restr
   for (int l = tid; l < r; l += OSJ_NT) {
     double2 v = cscale<double>(Y[(size_t)j * r + l], inv);
     if (!(sig > 0.0)) v = make_double2(l == j ? 1.0 : 0.0, 0.0);
-    Y[(size_t)j * r + l] = v;
+    Uc[(size_t)j * r + l] = v;
   }
 }
 

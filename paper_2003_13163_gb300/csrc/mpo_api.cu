@@ -58,6 +58,7 @@ struct HostSync {   // pinned read-back of the last select + eigen-solve
   GridCtl ctl;
   unsigned long long phase_ns[4];
   int tc_err;
+  GridCtl lq;         // control block of the FP64 form's LQ and FP32 solves
   GridCtl eig[8];     // FP64 eigen-solves of the last mixed factorisation
   int chol_status;    // Cholesky QR pivot status of the last mixed factorisation
   int chol_pass[2];   // status words after a Cholesky QR pass (cholqr_factor_kernel)
@@ -78,11 +79,14 @@ struct OzWork {
   int e_cap = 0;
 };
 
-// Workspace of the LQ-preconditioned SVD: the reflectors (m x ccap), the
-// accumulated W (m x m), the reflectors' factors and first entries.
+// Workspace of the LQ-preconditioned SVD: the reflectors (z, m x ccap) with their
+// factors and first entries (f, zd), three m x m matrices, the control block of
+// the LQ and FP32 solves.
 struct LqWork {
-  double2 *z = nullptr, *w = nullptr, *zd = nullptr;
+  double2 *z = nullptr, *w = nullptr, *s = nullptr, *v = nullptr, *zd = nullptr;
   double* f = nullptr;
+  OSCtl* ctl = nullptr;
+  int* ex = nullptr;
 };
 
 struct mpo_ctx {
@@ -332,8 +336,7 @@ static cudaError_t launch_onesided(cudaStream_t st, cplx<T>* X, int r, int c, in
 template <typename T>
 static cudaError_t launch_pair_jacobi(cudaStream_t st, cplx<T>* X, int r, int c, int ldx, cplx<T>* Ut, T* w, OSCtl* ctl,
                                       int max_sweeps, double timeout_s, int num_sms, double tol_min = 0.0,
-                                      bool clear = true,
-                                      double floor = eps_of<T>::value * eps_of<T>::value) {
+                                      double floor = eps_of<T>::value * eps_of<T>::value, int given_u = 0) {
   constexpr int EL = sizeof(T) == 8 ? 8 : 16;
   const void* fn = std::max(r, c) <= 2 * OSJ_NT ? (const void*)pair_jacobi_kernel<T, 2> : (const void*)pair_jacobi_kernel<T, EL>;
   int per_sm = 0;
@@ -341,14 +344,14 @@ static cudaError_t launch_pair_jacobi(cudaStream_t st, cplx<T>* X, int r, int c,
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const int blocks = std::max(1, std::min(per_sm * num_sms, (r + 1) / 2));
-  if (clear) e = cudaMemsetAsync(ctl, 0, sizeof(OSCtl), st);
+  e = cudaMemsetAsync(ctl, 0, sizeof(OSCtl), st);
   if (e != cudaSuccess) return e;
   // rows count as orthogonal once |<x_p, x_q>| <= 2 eps sqrt(c) ||x_p|| ||x_q||,
   // the rounding level of the length-c dot product itself
   const T tol_rel = (T)std::max(tol_min, 2.0 * eps_of<T>::value * std::sqrt((double)std::max(c, 1)));
   const T floor_rel = (T)floor;
   long long timeout_ns = (long long)(timeout_s * 1e9);
-  void* args[] = {&X, &r, &c, &ldx, &Ut, &w, &ctl, &max_sweeps, (void*)&tol_rel, (void*)&floor_rel, &timeout_ns};
+  void* args[] = {&X, &r, &c, &ldx, &Ut, &w, &ctl, &max_sweeps, (void*)&tol_rel, (void*)&floor_rel, &given_u, &timeout_ns};
   return cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(OSJ_NT), args, 0, st);
 }
 
@@ -386,9 +389,12 @@ static cudaError_t launch_fp32_jacobi(cudaStream_t st, float2* X, int r, int c, 
 // Rows below which the LQ step costs more than the sweeps it saves.
 constexpr int kLqMinRows = 8;
 
+// Rows from which the FP32 start pays.
+constexpr int kPreMinRows = 32;
+
 // X (r x c, r <= c) <- the rows Sigma V^H, vecs (r x r) <- rows conj(column of
-// U), w <- sigma^2 (lq_kernel). A barrier that timed out in the first kernel
-// leaves its error in ctl, which the Jacobi launch does not clear.
+// U), w <- sigma^2 (lq_kernel). q.ctl and ctl receive the barrier errors of the
+// first two kernels and of the FP64 solve.
 static cudaError_t launch_lq_jacobi(cudaStream_t st, double2* X, int r, int c, int ldx, double2* vecs, double* w,
                                     const LqWork& q, OSCtl* ctl, int max_sweeps, double timeout_s, int num_sms) {
   const bool small = c <= 2 * OSJ_NT;
@@ -398,20 +404,48 @@ static cudaError_t launch_lq_jacobi(cudaStream_t st, double2* X, int r, int c, i
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const int blocks = std::max(1, std::min(std::min(per_sm, 4) * num_sms, r));
-  e = cudaMemsetAsync(ctl, 0, sizeof(OSCtl), st);
+  e = cudaMemsetAsync(q.ctl, 0, sizeof(OSCtl), st);
   if (e != cudaSuccess) return e;
   long long timeout_ns = (long long)(timeout_s * 1e9);
   LqWork k = q;
-  void* args[] = {&X, &ldx, &r, &c, &k.z, &vecs, &k.f, &k.zd, &ctl, &timeout_ns};
+  void* args[] = {&X, &ldx, &r, &c, &k.z, &vecs, &k.f, &k.zd, &k.ctl, &timeout_ns};
   e = cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(OSJ_NT), args, 0, st);
   if (e != cudaSuccess) return e;
+  const double2* Y = vecs;       // what the FP64 solve works on, and its accumulated left factor
+  double2* Wt = q.w;
+  const bool pre = r >= kPreMinRows;
+  if (pre) {
+    const size_t n = (size_t)r * r;
+    const dim3 tg((r + 31) / 32, (r + 31) / 32), tb(32, 8);
+    float2 *a32 = (float2*)q.s, *u32 = a32 + n;
+    e = cudaMemsetAsync(q.ex, 0, sizeof(int), st);
+    if (e != cudaSuccess) return e;
+    max_exp_kernel<<<grid_for(n, num_sms), 256, 0, st>>>(vecs, n, q.ex);
+    scale_fp32_kernel<<<grid_for(n, num_sms), 256, 0, st>>>(vecs, n, q.ex, a32);
+    // a start only: sixteen sweeps at most, and no failure if they run out
+    e = launch_fp32_jacobi(st, a32, r, r, r, u32, (float*)w, q.ctl, 16, timeout_s, num_sms, 0.0);
+    if (e != cudaSuccess) return e;
+    transpose_kernel<float2><<<tg, tb, 0, st>>>(u32, r, r, q.v);                       // W, row-major
+    if ((e = cgemm<double>(st, r, r, r, q.v, r, 1, q.v, r, 0, X, r)) != cudaSuccess) return e;   // W^H W (X is free: Z holds the matrix)
+    ns_multiplier_kernel<<<grid_for(n, num_sms), 256, 0, st>>>(X, r);                  // E
+    if ((e = cudaMemcpyAsync(q.s, X, n * sizeof(double2), cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
+    if ((e = cgemm<double>(st, r, r, r, X, r, 0, X, r, 0, q.s, r, nullptr, 5.0 / 3.0, 1)) != cudaSuccess) return e;   // T = E + 5/3 E^2
+    if ((e = cudaMemcpyAsync(Wt, X, n * sizeof(double2), cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
+    if ((e = cgemm<double>(st, r, r, r, X, r, 0, q.s, r, 0, Wt, r, nullptr, 1.5, 1)) != cudaSuccess) return e;   // E + 3/2 E T
+    if ((e = cudaMemcpyAsync(X, q.v, n * sizeof(double2), cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
+    if ((e = cgemm<double>(st, r, r, r, q.v, r, 0, Wt, r, 0, X, r, nullptr, 1.0, 1)) != cudaSuccess) return e;   // W
+    if ((e = cgemm<double>(st, r, r, r, X, r, 1, vecs, r, 0, q.v, r)) != cudaSuccess) return e;                  // W^H R
+    transpose_kernel<double2><<<tg, tb, 0, st>>>(X, r, r, Wt);
+    Y = q.v;
+  }
   // the columns of U come from the rows of the result, so these are made
   // orthogonal relative to their own size down to 1e-14 of the largest each
   // (a floor of eps^2 would leave pairs at 1e-11 coupled by 1e-10)
-  e = launch_pair_jacobi<double>(st, vecs, r, r, r, k.w, w, ctl, max_sweeps, timeout_s, num_sms, 0.0, false, 1e-44);
+  e = launch_pair_jacobi<double>(st, const_cast<double2*>(Y), r, r, r, Wt, w, ctl, max_sweeps, timeout_s, num_sms, 0.0, 1e-44,
+                                 pre ? 1 : 0);
   if (e != cudaSuccess) return e;
-  if (small) lq_apply_kernel<2><<<r, OSJ_NT, 0, st>>>(k.z, r, c, k.f, k.zd, k.w, vecs, w, X, ldx);
-  else lq_apply_kernel<8><<<r, OSJ_NT, 0, st>>>(k.z, r, c, k.f, k.zd, k.w, vecs, w, X, ldx);
+  if (small) lq_apply_kernel<2><<<r, OSJ_NT, 0, st>>>(k.z, r, c, k.f, k.zd, Wt, Y, vecs, w, X, ldx);
+  else lq_apply_kernel<8><<<r, OSJ_NT, 0, st>>>(k.z, r, c, k.f, k.zd, Wt, Y, vecs, w, X, ldx);
   return cudaGetLastError();
 }
 
@@ -929,7 +963,10 @@ static int svd_select(mpo_ctx* h, cplx<T>* X, int r, int c, int ldx, int cap, bo
   CK(h, cudaMemcpyAsync(&h->hs->ctl, &h->osctl->g, sizeof(GridCtl), cudaMemcpyDeviceToHost, h->st));
   if (h->prof) CK(h, cudaMemcpyAsync(h->hs->phase_ns, h->osctl->phase_ns, sizeof(h->hs->phase_ns), cudaMemcpyDeviceToHost, h->st));
   CK(h, cudaMemcpyAsync(&h->hs->tc_err, h->tc_status, sizeof(int), cudaMemcpyDeviceToHost, h->st));
+  h->hs->lq.err = 0;
+  if (h->vecs_conj) CK(h, cudaMemcpyAsync(&h->hs->lq, &h->lq.ctl->g, sizeof(GridCtl), cudaMemcpyDeviceToHost, h->st));
   CK(h, cudaStreamSynchronize(h->st));
+  if (h->hs->lq.err) return fail(h, MPO_ERR_TIMEOUT, "grid barrier wait timed out in the SVD");
   if (h->hs->tc_err) return fail(h, MPO_ERR_TIMEOUT, "an mbarrier wait timed out in the tensor-core GEMM");
   if (h->prof) for (int i = 0; i < 3; ++i) h->prof_phase_ns[i] += h->hs->phase_ns[i];
   if (h->hs->ctl.err) return fail(h, MPO_ERR_TIMEOUT, "grid barrier wait timed out in the SVD");
@@ -1529,17 +1566,18 @@ static bool alloc_factor_ws(mpo_ctx* h, int m, int ccap, size_t bj_nch) {
 static void alloc_lq(mpo_ctx* h, int m, int ccap, size_t room) {
   if (h->prec != MPO_FP64) return;
   const size_t z = (size_t)m * ccap * sizeof(double2), w = (size_t)m * m * sizeof(double2);
-  const size_t sum = z + w + (size_t)m * (sizeof(double2) + sizeof(double));
+  const size_t sum = z + 3 * w + (size_t)m * (sizeof(double2) + sizeof(double)) + sizeof(OSCtl) + sizeof(int);
   size_t freeb = 0, totb = 0;
   if (sum > room || cudaMemGetInfo(&freeb, &totb) != cudaSuccess || sum > freeb) { cudaGetLastError(); return; }
   LqWork q;
   const size_t before = h->bytes;
-  if (ws_alloc(h, (void**)&q.z, z) && ws_alloc(h, (void**)&q.w, w) && ws_alloc(h, (void**)&q.zd, (size_t)m * sizeof(double2)) &&
-      ws_alloc(h, (void**)&q.f, (size_t)m * sizeof(double))) {
+  if (ws_alloc(h, (void**)&q.z, z) && ws_alloc(h, (void**)&q.w, w) && ws_alloc(h, (void**)&q.s, w) && ws_alloc(h, (void**)&q.v, w) &&
+      ws_alloc(h, (void**)&q.zd, (size_t)m * sizeof(double2)) && ws_alloc(h, (void**)&q.f, (size_t)m * sizeof(double)) &&
+      ws_alloc(h, (void**)&q.ctl, sizeof(OSCtl)) && ws_alloc(h, (void**)&q.ex, sizeof(int))) {
     h->lq = q;
     return;
   }
-  cudaFree(q.z); cudaFree(q.w); cudaFree(q.zd); cudaFree(q.f);
+  for (void* p : {(void*)q.z, (void*)q.w, (void*)q.s, (void*)q.v, (void*)q.zd, (void*)q.f, (void*)q.ctl, (void*)q.ex}) cudaFree(p);
   h->bytes = before;
 }
 
@@ -1690,7 +1728,7 @@ void mpo_free(mpo_handle h) {
   if (h->batch) { batch_free(h); return; }
   for (void* p : h->site) if (p) cudaFree(p);
   void* ps[] = {h->spare, h->theta, h->theta2, h->osctl, h->tc_status, h->bj_gpart, h->bj_j, h->bj_act, h->vecs, h->tmp, h->wv, h->perm, h->lam2, h->Ms, h->dgates,
-                h->lq.z, h->lq.w, h->lq.zd, h->lq.f,
+                h->lq.z, h->lq.w, h->lq.s, h->lq.v, h->lq.zd, h->lq.f, h->lq.ctl, h->lq.ex,
                 h->dsup, h->dp, h->info, h->ctl, h->scal, h->dS, h->dschmidt, h->tv0, h->tv1,
                 h->mx_a32, h->mx_ut32, h->mx_w32, h->mx_perm32, h->mx_lam32, h->mx_info32, h->mx_Q, h->mx_Q2,
                 h->mx_B, h->mx_T, h->mx_V, h->mx_G, h->mx_w,
