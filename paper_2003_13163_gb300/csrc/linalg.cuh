@@ -1795,7 +1795,6 @@ __global__ void __launch_bounds__(256) block_jacobi_kernel(cplx<T>* X, int r, in
   cplx<T>* Gs = reinterpret_cast<cplx<T>*>(smraw);     // phase E: the pair Gram; phase A: J^H or J^T
   cplx<T>* Vs = Gs + JP * LD;
 
-  __shared__ T s_gmax;
   cplx<T>* Js = reinterpret_cast<cplx<T>*>(red);        // phase A: J^H or J^T (ld JP+1)
   const int nb = (r + JB - 1) / JB, N = nb + (nb & 1), npairs = N / 2;
   const int nch = (c + JCW - 1) / JCW, nchu = (r + JCW - 1) / JCW;
@@ -2008,15 +2007,24 @@ __global__ void __launch_bounds__(256) block_jacobi_kernel(cplx<T>* X, int r, in
         if (P > Q) { int t_ = P; P = Q; Q = t_; }
         const bool full_e = Q < nb && pair_full(P, Q);
         if (Q >= nb || (!full_e && !pair_dirty(P, Q))) { if (tid == 0) act_flag[pi] = 0; continue; }
+        // FP64 only where its rounding matters (an FP64 warp instruction holds
+        // its SM partition for 64 clocks): sums of zero-padded loads and maxima
+        // taken in FP64 cost 18 of the 56 us of a pair solve
         for (int e = tid; e < JP * JP; e += blockDim.x) {
-          double sr = 0.0, si = 0.0;
           const cplx<T>* src = Gpart + (size_t)pi * nch * JP * JP + e;
+          if (nch == 1) {
+            const cplx<T> v = ldcg(src);
+            Gs[(e / JP) * LD + (e % JP)] = mk<T>(v.x + T(0), v.y + T(0));
+            continue;
+          }
+          double sr = 0.0, si = 0.0;
           for (int ch0 = 0; ch0 < nch; ch0 += 8) {   // up to eight loads in flight
             cplx<T> v[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) v[u] = ch0 + u < nch ? ldcg(src + (size_t)(ch0 + u) * JP * JP) : czero<T>();
 #pragma unroll
-            for (int u = 0; u < 8; ++u) { sr += (double)v[u].x; si += (double)v[u].y; }
+            for (int u = 0; u < 8; ++u)
+              if (ch0 + u < nch) { sr += (double)v[u].x; si += (double)v[u].y; }
           }
           Gs[(e / JP) * LD + (e % JP)] = mk<T>((T)sr, (T)si);
         }
@@ -2029,9 +2037,11 @@ __global__ void __launch_bounds__(256) block_jacobi_kernel(cplx<T>* X, int r, in
         // derived from this pair's Gram resolves its entries (rows gain norm
         // as the sweeps concentrate it, so the initial scale alone can sit
         // below what the pair solve can reach and the sweeps never end)
-        double gpmax = 0.0;
-        for (int i = 0; i < JP; ++i) gpmax = fmax(gpmax, (double)Gs[i * LD + i].x);
-        const double pfloor = fmax((double)floor_abs, (double)floor_rel * gpmax);
+        static_assert(JP == 32, "one diagonal entry per lane");
+        const T dl = Gs[lane * LD + lane].x;
+        T gpm = fmax(T(0), dl);
+        for (int o = 16; o > 0; o >>= 1) gpm = fmax(gpm, __shfl_xor_sync(0xffffffffu, gpm, o));
+        const double pfloor = fmax((double)floor_abs, (double)floor_rel * (double)gpm);
         for (int e = tid; e < (full_e ? JP * JP : JB * JB); e += blockDim.x) {
           const int i = full_e ? e / JP : e / JB, j = full_e ? e % JP : JB + e % JB;
           if (i >= j) continue;
@@ -2056,12 +2066,9 @@ __global__ void __launch_bounds__(256) block_jacobi_kernel(cplx<T>* X, int r, in
           // inner solve.
           int first_order = 0, exact = 1;
           if (!full_e) {
-            double gmin = 1e300, gmax = 0.0;
-            for (int i = 0; i < JP; ++i) {
-              const double d = (double)Gs[i * LD + i].x;
-              gmin = fmin(gmin, d);
-              gmax = fmax(gmax, d);
-            }
+            T gmn = dl;
+            for (int o = 16; o > 0; o >>= 1) gmn = fmin(gmn, __shfl_xor_sync(0xffffffffu, gmn, o));
+            const double gmin = (double)gmn, gmax = (double)gpm;
             const double e2lim = gmax > 0.0 ? fmax((double)tol_rel * gmin, pfloor) / (JB * gmax) : 0.0;
             int ok = 1;
             for (int e = tid; e < JB * JB; e += blockDim.x) {
@@ -2089,14 +2096,8 @@ __global__ void __launch_bounds__(256) block_jacobi_kernel(cplx<T>* X, int r, in
             __syncthreads();
             bj_polish_unitary_to<T>(Vs, Gs, Vs + JP * LD, T(8.0 * eps_of<T>::value * 5.66), 6);
           } else {
-            if (tid == 0) {
-              T gm = T(0);
-              for (int i = 0; i < JP; ++i) gm = fmax(gm, Gs[i * LD + i].x);
-              s_gmax = gm;
-            }
-            __syncthreads();
             exact = bj_inner_eig<T>(Gs, Vs + JP * LD, Vs, 4.0 * (double)eps_of<T>::value * sqrt((double)JP),
-                                    32.0 * (double)eps_of<T>::value * (double)s_gmax, 3);
+                                    32.0 * (double)eps_of<T>::value * (double)gpm, 3);
             // FP32: remove the rounding drift of J (FP64 rotations keep it at 1e-16)
             if constexpr (sizeof(T) == 4) bj_polish_unitary<T>(Vs, Gs, Vs + JP * LD);
           }
