@@ -35,6 +35,7 @@
 #include <algorithm>
 #include <type_traits>
 #include <atomic>
+#include <functional>
 #include <map>
 #include <mutex>
 #include <thread>
@@ -132,6 +133,9 @@ struct mpo_ctx {
   std::vector<char> s_valid;
   int centre = 0;
   size_t bytes = 0;
+  char* ws_base = nullptr;         // one device allocation holds every buffer of the handle (ws_build)
+  size_t ws_off = 0, ws_cap = 0;
+  bool ws_plan = false;
   int last_sweeps = 0;
   // kernel-class timing (mpo_profile): CUDA events recorded on h->st around
   // each launch, resolved lazily
@@ -559,31 +563,25 @@ static cudaError_t oz_gemm(cudaStream_t st, int M, int N, int K, const double2* 
   return cudaGetLastError();
 }
 
-// Allocate the scratch for products whose operands have at most dmax rows,
-// columns and inner dimension.
-static bool alloc_oz(OzWork& w, int dmax, size_t* bytes) {
-  const size_t Mp = (size_t)(dmax + oz::BM - 1) / oz::BM * oz::BM;
-  const size_t Nrp = (size_t)(2 * dmax + oz::BN - 1) / oz::BN * oz::BN;
-  const size_t Kp = 2 * (size_t)((dmax + 31) / 32 * 32);
+// Scratch of products with at most M rows, N columns and inner dimension K, from
+// `alloc` (void**, bytes): the slices of both operands, and one block of
+// exponents of A, of B and the status word.
+template <typename F>
+static bool alloc_oz(OzWork& w, int M, int N, int K, F alloc) {
+  const size_t Mp = (size_t)(M + oz::BM - 1) / oz::BM * oz::BM;
+  const size_t Nrp = (size_t)(2 * (size_t)N + oz::BN - 1) / oz::BN * oz::BN;
+  const size_t Kp = 32 * (size_t)((K + 15) / 16);
   w.a_cap = (size_t)oz::S * Mp * Kp;
   w.b_cap = (size_t)oz::S * Nrp * Kp;
   w.e_cap = (int)std::max(Mp, Nrp);
-  bool ok = cudaMalloc((void**)&w.a, w.a_cap * sizeof(__nv_bfloat16)) == cudaSuccess &&
-            cudaMalloc((void**)&w.b, w.b_cap * sizeof(__nv_bfloat16)) == cudaSuccess &&
-            cudaMalloc((void**)&w.ea, (2 * (size_t)w.e_cap + 1) * sizeof(int)) == cudaSuccess &&
-            cudaMemset(w.ea + 2 * (size_t)w.e_cap, 0, sizeof(int)) == cudaSuccess;
-  if (!ok) cudaGetLastError();
-  if (w.ea) {                      // one allocation: exponents of A, of B, status
+  if (!alloc((void**)&w.a, w.a_cap * sizeof(__nv_bfloat16)) || !alloc((void**)&w.b, w.b_cap * sizeof(__nv_bfloat16)) ||
+      !alloc((void**)&w.ea, (2 * (size_t)w.e_cap + 1) * sizeof(int)))
+    return false;
+  if (w.ea) {
     w.eb = w.ea + w.e_cap;
     w.status = w.ea + 2 * (size_t)w.e_cap;
   }
-  if (bytes) *bytes += (w.a_cap + w.b_cap) * sizeof(__nv_bfloat16) + 2 * w.e_cap * sizeof(int);
-  return ok;
-}
-
-static void free_oz(OzWork& w) {
-  cudaFree(w.a); cudaFree(w.b); cudaFree(w.ea);
-  w = OzWork();
+  return true;
 }
 
 // Products large enough to fill 128 x 128 real tiles go to the tensor cores.
@@ -1502,11 +1500,52 @@ static int init_fail(mpo_ctx* h, int code, const std::string& m) {
   return code;
 }
 
-// Device allocation that counts towards the handle's bytes.
+// A handle's device buffers are carved out of one allocation: about sixty
+// cudaMalloc / cudaFree pairs (each free waits for the device) cost 3 ms per
+// handle or truncated-SVD call. ws_build runs the list of ws_alloc calls twice,
+// first only adding up their sizes.
 static bool ws_alloc(mpo_ctx* h, void** p, size_t bytes) {
-  if (cudaMalloc(p, std::max<size_t>(bytes, 256)) != cudaSuccess) { cudaGetLastError(); *p = nullptr; return false; }
+  const size_t sz = (std::max<size_t>(bytes, 256) + 255) & ~(size_t)255;
+  if (h->ws_plan) { h->ws_cap += sz; return true; }
+  if (h->ws_off + sz > h->ws_cap) return false;
+  *p = h->ws_base + h->ws_off;
+  h->ws_off += sz;
   h->bytes += bytes;
   return true;
+}
+
+static bool ws_build(mpo_ctx* h, const std::function<bool()>& list) {
+  h->ws_cap = h->ws_off = 0;
+  h->ws_plan = true;
+  list();
+  h->ws_plan = false;
+  if (cudaMalloc((void**)&h->ws_base, h->ws_cap) != cudaSuccess) { cudaGetLastError(); h->ws_base = nullptr; return false; }
+  return list();
+}
+
+// Pinned read-back blocks, kept for the next handle (at most kHostSyncKeep of
+// them; a pinned allocation and its free cost ~0.2 ms and a device wait).
+constexpr size_t kHostSyncKeep = 16;
+static std::mutex g_hs_mu;
+static std::vector<HostSync*> g_hs_free;
+
+static HostSync* hostsync_get() {
+  {
+    std::lock_guard<std::mutex> lk(g_hs_mu);
+    if (!g_hs_free.empty()) { HostSync* p = g_hs_free.back(); g_hs_free.pop_back(); return p; }
+  }
+  HostSync* p = nullptr;
+  if (cudaHostAlloc((void**)&p, sizeof(HostSync), cudaHostAllocPortable) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+  return p;
+}
+
+static void hostsync_put(HostSync* p) {
+  if (!p) return;
+  {
+    std::lock_guard<std::mutex> lk(g_hs_mu);
+    if (g_hs_free.size() < kHostSyncKeep) { g_hs_free.push_back(p); return; }
+  }
+  cudaFreeHost(p);
 }
 
 // Workspace of the factorisations (svd_select / msvd_select) for matrices of
@@ -1555,30 +1594,40 @@ static bool alloc_factor_ws(mpo_ctx* h, int m, int ccap, size_t bj_nch) {
     ok = ok && alloc((void**)&h->mx_A32, mm * mm * sizeof(float2));
     ok = ok && alloc((void**)&h->mx_Li32, mm * mm * sizeof(float2));
     ok = ok && alloc((void**)&h->mx_chst, 2 * sizeof(int));
-    ok = ok && cudaMemsetAsync(h->ctl, 0, sizeof(GridCtl), h->st) == cudaSuccess;
+    if (!h->ws_plan) ok = ok && cudaMemsetAsync(h->ctl, 0, sizeof(GridCtl), h->st) == cudaSuccess;
   }
   return ok;
 }
 
-// Workspace of the FP64 form's LQ step. It only saves time, so a handle whose
-// memory limit (arena_cap_bytes: `room` bytes left) or device has no room for
-// it goes without.
-static void alloc_lq(mpo_ctx* h, int m, int ccap, size_t room) {
-  if (h->prec != MPO_FP64) return;
-  const size_t z = (size_t)m * ccap * sizeof(double2), w = (size_t)m * m * sizeof(double2);
-  const size_t sum = z + 3 * w + (size_t)m * (sizeof(double2) + sizeof(double)) + sizeof(OSCtl) + sizeof(int);
+// Workspace of the FP64 form's LQ step.
+static size_t lq_bytes(int m, int ccap) {
+  return ((size_t)m * ccap + 3 * (size_t)m * m) * sizeof(double2) + (size_t)m * (sizeof(double2) + sizeof(double)) +
+         sizeof(OSCtl) + sizeof(int) + 8 * 256;
+}
+
+static bool alloc_lq(mpo_ctx* h, int m, int ccap) {
+  LqWork& q = h->lq;
+  const size_t w = (size_t)m * m * sizeof(double2);
+  return ws_alloc(h, (void**)&q.z, (size_t)m * ccap * sizeof(double2)) && ws_alloc(h, (void**)&q.w, w) &&
+         ws_alloc(h, (void**)&q.s, w) && ws_alloc(h, (void**)&q.v, w) &&
+         ws_alloc(h, (void**)&q.zd, (size_t)m * sizeof(double2)) && ws_alloc(h, (void**)&q.f, (size_t)m * sizeof(double)) &&
+         ws_alloc(h, (void**)&q.ctl, sizeof(OSCtl)) && ws_alloc(h, (void**)&q.ex, sizeof(int));
+}
+
+// All buffers of a handle: `list(lq)` allocates them, with the LQ workspace if lq
+// is set. That one only saves time, so a handle whose memory limit (`room` bytes
+// left) or device has no room for it goes without.
+static bool ws_build_lq(mpo_ctx* h, int m, int ccap, size_t need, size_t room, const std::function<bool(bool)>& list) {
   size_t freeb = 0, totb = 0;
-  if (sum > room || cudaMemGetInfo(&freeb, &totb) != cudaSuccess || sum > freeb) { cudaGetLastError(); return; }
-  LqWork q;
-  const size_t before = h->bytes;
-  if (ws_alloc(h, (void**)&q.z, z) && ws_alloc(h, (void**)&q.w, w) && ws_alloc(h, (void**)&q.s, w) && ws_alloc(h, (void**)&q.v, w) &&
-      ws_alloc(h, (void**)&q.zd, (size_t)m * sizeof(double2)) && ws_alloc(h, (void**)&q.f, (size_t)m * sizeof(double)) &&
-      ws_alloc(h, (void**)&q.ctl, sizeof(OSCtl)) && ws_alloc(h, (void**)&q.ex, sizeof(int))) {
-    h->lq = q;
-    return;
+  const size_t lq = lq_bytes(m, ccap);
+  if (h->prec == MPO_FP64 && lq <= room && cudaMemGetInfo(&freeb, &totb) == cudaSuccess && need + lq <= freeb) {
+    if (ws_build(h, [&]() { return list(true); })) return true;
+    cudaFree(h->ws_base);
+    h->ws_base = nullptr;
+    h->lq = LqWork();
+    h->bytes = 0;
   }
-  for (void* p : {(void*)q.z, (void*)q.w, (void*)q.s, (void*)q.v, (void*)q.zd, (void*)q.f, (void*)q.ctl, (void*)q.ex}) cudaFree(p);
-  h->bytes = before;
+  return ws_build(h, [&]() { return list(false); });
 }
 
 int mpo_init(mpo_handle* out, int n, int chi_max, mpo_precision prec, void* stream, const mpo_opts* opts) {
@@ -1670,30 +1719,34 @@ int mpo_init(mpo_handle* out, int n, int chi_max, mpo_precision prec, void* stre
 
   auto alloc = [&](void** p, size_t bytes) -> bool { return ws_alloc(h, p, bytes); };
   h->site.assign(n, nullptr);
-  bool ok = true;
-  for (int k = 0; k < n && ok; ++k) ok = alloc(&h->site[k], h->site_cap * h->esz);
-  ok = ok && alloc(&h->spare, h->site_cap * h->esz);
-  ok = ok && alloc(&h->theta, th * h->esz);
-  ok = ok && alloc(&h->theta2, th * h->esz);
-  ok = ok && alloc(&h->tmp, h->tmp_cap * h->esz);
-  ok = ok && alloc(&h->Ms, (size_t)std::max(1, ngmax) * 256 * h->esz);
-  ok = ok && alloc((void**)&h->dgates, (size_t)std::max(1, ngmax) * 16 * sizeof(double2));
-  ok = ok && alloc((void**)&h->dp, (size_t)std::max(1, ngmax) * sizeof(double));
-  ok = ok && alloc((void**)&h->dsup, 256 * sizeof(double2));
-  ok = ok && alloc_factor_ws(h, m, mx_ccap, bj_nch);
-  if (ok && h->use_oz) ok = alloc_oz(h->oz, std::max(m, mx_ccap), &h->bytes);
-  ok = ok && alloc((void**)&h->scal, 8 * sizeof(double));
-  ok = ok && alloc((void**)&h->dS, (size_t)(n - 1) * sizeof(double));
-  ok = ok && alloc((void**)&h->dschmidt, (size_t)(n - 1) * chi_max * sizeof(double));
-  ok = ok && alloc((void**)&h->tv0, (size_t)(chi_max + 1) * sizeof(double2));
-  ok = ok && alloc((void**)&h->tv1, (size_t)(chi_max + 1) * sizeof(double2));
-  if (!ok) return init_fail(h, MPO_ERR_OOM, "cudaMalloc failed");
-  alloc_lq(h, m, mx_ccap, h->opts.arena_cap_bytes > 0 ? h->opts.arena_cap_bytes - need : ~(size_t)0);
-  if (cudaMallocHost((void**)&h->hs, sizeof(HostSync)) != cudaSuccess) {
-    cudaGetLastError();
-    h->hs = nullptr;
-    return init_fail(h, MPO_ERR_CUDA, "cudaMallocHost failed");
-  }
+  auto list = [&](bool lq) -> bool {
+    bool ok = true;
+    for (int k = 0; k < n && ok; ++k) ok = alloc(&h->site[k], h->site_cap * h->esz);
+    ok = ok && alloc(&h->spare, h->site_cap * h->esz);
+    ok = ok && alloc(&h->theta, th * h->esz);
+    ok = ok && alloc(&h->theta2, th * h->esz);
+    ok = ok && alloc(&h->tmp, h->tmp_cap * h->esz);
+    ok = ok && alloc(&h->Ms, (size_t)std::max(1, ngmax) * 256 * h->esz);
+    ok = ok && alloc((void**)&h->dgates, (size_t)std::max(1, ngmax) * 16 * sizeof(double2));
+    ok = ok && alloc((void**)&h->dp, (size_t)std::max(1, ngmax) * sizeof(double));
+    ok = ok && alloc((void**)&h->dsup, 256 * sizeof(double2));
+    ok = ok && alloc_factor_ws(h, m, mx_ccap, bj_nch);
+    const int d = std::max(m, mx_ccap);
+    if (ok && h->use_oz) ok = alloc_oz(h->oz, d, d, d, alloc);
+    ok = ok && alloc((void**)&h->scal, 8 * sizeof(double));
+    ok = ok && alloc((void**)&h->dS, (size_t)(n - 1) * sizeof(double));
+    ok = ok && alloc((void**)&h->dschmidt, (size_t)(n - 1) * chi_max * sizeof(double));
+    ok = ok && alloc((void**)&h->tv0, (size_t)(chi_max + 1) * sizeof(double2));
+    ok = ok && alloc((void**)&h->tv1, (size_t)(chi_max + 1) * sizeof(double2));
+    if (ok && lq) ok = alloc_lq(h, m, mx_ccap);
+    return ok;
+  };
+  const size_t room = h->opts.arena_cap_bytes > 0 ? h->opts.arena_cap_bytes - need : ~(size_t)0;
+  if (!ws_build_lq(h, m, mx_ccap, need, room, list)) return init_fail(h, MPO_ERR_OOM, "cudaMalloc failed");
+  h->hs = hostsync_get();
+  if (!h->hs) return init_fail(h, MPO_ERR_CUDA, "cudaHostAlloc failed");
+  if (h->use_oz && cudaMemsetAsync(h->oz.status, 0, sizeof(int), h->st) != cudaSuccess)
+    return init_fail(h, MPO_ERR_CUDA, "initial state upload failed");
   // product state |0..0><0..0|: every site 1 x 4 x 1 with A[0][0][0] = 1 (Sec. 4.1)
   std::vector<unsigned char> one(h->esz, 0);
   if (prec != MPO_FP32) { double v = 1.0; memcpy(one.data(), &v, sizeof v); }
@@ -1726,16 +1779,11 @@ static void batch_free(mpo_ctx* h);
 void mpo_free(mpo_handle h) {
   if (!h) return;
   if (h->batch) { batch_free(h); return; }
-  for (void* p : h->site) if (p) cudaFree(p);
-  void* ps[] = {h->spare, h->theta, h->theta2, h->osctl, h->tc_status, h->bj_gpart, h->bj_j, h->bj_act, h->vecs, h->tmp, h->wv, h->perm, h->lam2, h->Ms, h->dgates,
-                h->lq.z, h->lq.w, h->lq.s, h->lq.v, h->lq.zd, h->lq.f, h->lq.ctl, h->lq.ex,
-                h->dsup, h->dp, h->info, h->ctl, h->scal, h->dS, h->dschmidt, h->tv0, h->tv1,
-                h->mx_a32, h->mx_ut32, h->mx_w32, h->mx_perm32, h->mx_lam32, h->mx_info32, h->mx_Q, h->mx_Q2,
-                h->mx_B, h->mx_T, h->mx_V, h->mx_G, h->mx_w,
-                h->mx_W, h->mx_A32, h->mx_Li32, h->mx_chst, h->mx_eosctl, h->mx_rot, h->mx_Q0};
-  for (void* p : ps) if (p) cudaFree(p);
-  if (h->hs) cudaFreeHost(h->hs);
-  free_oz(h->oz);
+  // a handle's buffers and its read-back block may still be in use on its stream
+  // after an error or a call that did not wait; cudaFree waits for the device
+  if (h->ws_base) cudaFree(h->ws_base);
+  else if (h->hs) cudaStreamSynchronize(h->st);
+  hostsync_put(h->hs);
   for (auto& q : h->pend) { cudaEventDestroy(q.a); cudaEventDestroy(q.b); }
   for (auto e : h->evpool) cudaEventDestroy(e);
   delete h;
@@ -2065,17 +2113,21 @@ int mpo_svd_truncated(int r, int c, const void* A, int cap, mpo_precision prec, 
   h->mx_mcap = std::min(r, cap + h->mx_over);
   h->use_oz = h->mixed && h->opts.tensor_cores >= 0;
   const size_t nch = (size_t)(c + JCW - 1) / JCW + 1;
-  bool ok = ws_alloc(h, &h->theta, (size_t)r * c * h->esz) && alloc_factor_ws(h, r, c, nch) &&
-            ws_alloc(h, (void**)&h->scal, 8 * sizeof(double));
-  if (ok && h->use_oz) ok = alloc_oz(h->oz, c, &h->bytes);
-  if (ok && cudaMallocHost((void**)&h->hs, sizeof(HostSync)) != cudaSuccess) { cudaGetLastError(); h->hs = nullptr; ok = false; }
+  auto alloc = [&](void** p, size_t bytes) -> bool { return ws_alloc(h, p, bytes); };
+  auto list = [&](bool lq) -> bool {
+    return alloc(&h->theta, (size_t)r * c * h->esz) && alloc_factor_ws(h, r, c, nch) &&
+           alloc((void**)&h->scal, 8 * sizeof(double)) && (!h->use_oz || alloc_oz(h->oz, c, c, c, alloc)) &&
+           (!lq || alloc_lq(h, r, c));
+  };
+  bool ok = ws_build_lq(h, r, c, 0, h->opts.arena_cap_bytes > 0 ? 0 : ~(size_t)0, list);
+  if (ok && !(h->hs = hostsync_get())) ok = false;
   if (!ok) { mpo_free(h); g_last_init_error = "mpo_svd_truncated: allocation failed"; return MPO_ERR_OOM; }
-  alloc_lq(h, r, c, h->opts.arena_cap_bytes > 0 ? 0 : ~(size_t)0);
   int rc = MPO_OK, kk = 0;
   auto ck = [&](cudaError_t e) { if (rc == MPO_OK && e != cudaSuccess) { rc = MPO_ERR_CUDA; g_last_init_error = cudaGetErrorString(e); } };
   ck(cudaMemcpyAsync(h->theta, A, (size_t)r * c * h->esz, cudaMemcpyDeviceToDevice, h->st));
   ck(cudaMemsetAsync(h->scal, 0, 8 * sizeof(double), h->st));
   ck(cudaMemsetAsync(h->tc_status, 0, sizeof(int), h->st));
+  if (h->use_oz) ck(cudaMemsetAsync(h->oz.status, 0, sizeof(int), h->st));
   if (rc == MPO_OK) {
     rc = prec != MPO_FP32 ? svd_select<double>(h, (double2*)h->theta, r, c, c, cap, true, nullptr, nullptr, &kk)
                           : svd_select<float>(h, (float2*)h->theta, r, c, c, cap, true, nullptr, nullptr, &kk);
@@ -2225,13 +2277,26 @@ int mpo_gemm_ex(int M, int N, int K, const void* A, int lda, int opA, const void
   cudaError_t e = cudaSuccess;
   int hs = 0;
   if (prec == MPO_FP64 && engine == 1) {
+    // one allocation, sized for this product
     OzWork w;
-    if (!alloc_oz(w, std::max(M, std::max(N, K)), nullptr)) { free_oz(w); return MPO_ERR_OOM; }
-    e = oz_gemm(st, M, N, K, (const double2*)A, lda, opA, (const double2*)B, ldb, opB, (double2*)C, ldc, 1.0, 0, w,
-                5.0, sms);
+    size_t off = 0;
+    char* base = nullptr;
+    auto carve = [&](void** p, size_t bytes) -> bool {
+      if (base) *p = base + off;
+      off += (bytes + 255) & ~(size_t)255;
+      return true;
+    };
+    alloc_oz(w, M, N, K, carve);
+    if (cudaMalloc((void**)&base, off) != cudaSuccess) { cudaGetLastError(); return MPO_ERR_OOM; }
+    off = 0;
+    alloc_oz(w, M, N, K, carve);
+    e = cudaMemsetAsync(w.status, 0, sizeof(int), st);
+    if (e == cudaSuccess)
+      e = oz_gemm(st, M, N, K, (const double2*)A, lda, opA, (const double2*)B, ldb, opB, (double2*)C, ldc, 1.0, 0, w,
+                  5.0, sms);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&hs, w.status, sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    free_oz(w);
+    cudaFree(base);
   } else if (engine == 1) {
     return mpo_gemm(M, N, K, A, B, C, prec, 1, stream);
   } else {
