@@ -1588,10 +1588,20 @@ __device__ __forceinline__ void bj_rot_params(const cplx<TI>* G, int p, int q, T
 // accumulated rotations is removed afterwards by bj_polish_unitary. G0 holds
 // the input; G1 is scratch of the same shape; both are overwritten. Returns
 // 1 when a sweep found nothing left to rotate (the result is diagonal to the
-// tolerance), 0 when max_sweeps ran out first.
+// tolerance), 0 when max_sweeps ran out first. order[rd * NR + a] holds pair a of
+// round rd (bj_fill_order): six player indices modulo JP - 1 were a third of a
+// round's instructions.
+__device__ __forceinline__ void bj_fill_order(uchar2* order) {
+  for (int e = threadIdx.x; e < (JP - 1) * (JP / 2); e += blockDim.x) {
+    const int rd = e / (JP / 2), a = e % (JP / 2);
+    const int p = rr_player(a, rd, JP), q = rr_player(JP - 1 - a, rd, JP);
+    order[e] = make_uchar2((unsigned char)min(p, q), (unsigned char)max(p, q));
+  }
+}
+
 template <typename TI>
 __device__ int bj_inner_eig(cplx<TI>* G0, cplx<TI>* G1, cplx<TI>* Vs /*JP x JP, ld JP+1*/, double tol,
-                             double floor_abs, int max_sweeps) {
+                             double floor_abs, int max_sweeps, const uchar2* order) {
   constexpr int LD = JP + 1, NR = JP / 2;
   static_assert(NR * NR == 256, "one thread per 2 x 2 block");
   const int tid = threadIdx.x, ia = tid / NR, ib = tid % NR;
@@ -1606,18 +1616,15 @@ __device__ int bj_inner_eig(cplx<TI>* G0, cplx<TI>* G1, cplx<TI>* Vs /*JP x JP, 
   for (int sw = 0; sw < max_sweeps; ++sw) {
     int any = 0;
     for (int rd = 0; rd < JP - 1; ++rd) {
-      int pa = rr_player(ia, rd, JP), qa = rr_player(JP - 1 - ia, rd, JP);
-      if (pa > qa) { const int t_ = pa; pa = qa; qa = t_; }
-      int pb = rr_player(ib, rd, JP), qb = rr_player(JP - 1 - ib, rd, JP);
-      if (pb > qb) { const int t_ = pb; pb = qb; qb = t_; }
+      const uchar2 oa = order[rd * NR + ia], ob = order[rd * NR + ib];
+      const int pa = oa.x, qa = oa.y, pb = ob.x, qb = ob.y;
       // lane l of every warp derives rotation l % NR; threads fetch the two
       // they need by shuffle (no block barrier for a shared table)
       TI cl, sl, url, uil;
       {
         const int lr = (tid & 31) % NR;
-        int pl = rr_player(lr, rd, JP), ql = rr_player(JP - 1 - lr, rd, JP);
-        if (pl > ql) { const int t_ = pl; pl = ql; ql = t_; }
-        bj_rot_params<TI>(Gc, pl, ql, tol2, flo2, cl, sl, url, uil);
+        const uchar2 ol = order[rd * NR + lr];
+        bj_rot_params<TI>(Gc, ol.x, ol.y, tol2, flo2, cl, sl, url, uil);
       }
       // every warp derives the same table from the same matrix, so a round
       // with nothing to rotate is skipped by all threads alike (no writes,
@@ -1796,6 +1803,8 @@ __global__ void __launch_bounds__(256) block_jacobi_kernel(cplx<T>* X, int r, in
   cplx<T>* Vs = Gs + JP * LD;
 
   cplx<T>* Js = reinterpret_cast<cplx<T>*>(red);        // phase A: J^H or J^T (ld JP+1)
+  __shared__ uchar2 s_order[(JP - 1) * (JP / 2)];
+  bj_fill_order(s_order);                               // read after the first grid barrier
   const int nb = (r + JB - 1) / JB, N = nb + (nb & 1), npairs = N / 2;
   const int nch = (c + JCW - 1) / JCW, nchu = (r + JCW - 1) / JCW;
   const unsigned nblk = gridDim.x;
@@ -2097,7 +2106,7 @@ __global__ void __launch_bounds__(256) block_jacobi_kernel(cplx<T>* X, int r, in
             bj_polish_unitary_to<T>(Vs, Gs, Vs + JP * LD, T(8.0 * eps_of<T>::value * 5.66), 6);
           } else {
             exact = bj_inner_eig<T>(Gs, Vs + JP * LD, Vs, 4.0 * (double)eps_of<T>::value * sqrt((double)JP),
-                                    32.0 * (double)eps_of<T>::value * (double)gpm, 3);
+                                    32.0 * (double)eps_of<T>::value * (double)gpm, 3, s_order);
             // FP32: remove the rounding drift of J (FP64 rotations keep it at 1e-16)
             if constexpr (sizeof(T) == 4) bj_polish_unitary<T>(Vs, Gs, Vs + JP * LD);
           }
