@@ -806,7 +806,21 @@ __global__ void __launch_bounds__(OSJ_NT) pair_jacobi_kernel(cplx<T>* X, int r, 
           gr = fma(x.x, y.x, fma(x.y, y.y, gr));     // x conj(y)
           gi = fma(x.y, y.x, fma(-x.x, y.y, gi));
         };
+        cplx<T>* tp = Ut + (size_t)p * r;
+        cplx<T>* tq = Ut + (size_t)q * r;
         cplx<T> rx[E], ry[E];
+        // short rows: U's two rows are fetched together with X's, so that their
+        // L2 round trip runs under the reduction and the rotation parameters
+        constexpr int EU = E <= 2 ? E : 1;
+        cplx<T> ux[EU], uy[EU];
+        if (E <= 2 && uregs) {
+#pragma unroll
+          for (int e = 0; e < EU; ++e) {
+            const int j = tid + OSJ_NT * e;
+            ux[e] = j < r ? ldcg(&tp[j]) : czero<T>();
+            uy[e] = j < r ? ldcg(&tq[j]) : czero<T>();
+          }
+        }
         if (regs) {
 #pragma unroll
           for (int e = 0; e < E; ++e) {
@@ -839,8 +853,6 @@ __global__ void __launch_bounds__(OSJ_NT) pair_jacobi_kernel(cplx<T>* X, int r, 
         __syncthreads();
         if (!s_rot.on) continue;
         const T cs = s_rot.c, sn = s_rot.s, sur = s_rot.sur, sui = s_rot.sui, cur = s_rot.cur, cui = s_rot.cui;
-        cplx<T>* tp = Ut + (size_t)p * r;
-        cplx<T>* tq = Ut + (size_t)q * r;
         if (regs) {
 #pragma unroll
           for (int e = 0; e < E; ++e) {
@@ -861,7 +873,17 @@ __global__ void __launch_bounds__(OSJ_NT) pair_jacobi_kernel(cplx<T>* X, int r, 
           }
         }
         // U <- U J: the conjugate phase
-        if (uregs) {
+        if (E <= 2 && uregs) {
+#pragma unroll
+          for (int e = 0; e < EU; ++e) {
+            const int j = tid + OSJ_NT * e;
+            if (j < r) {
+              osj_rotate<T>(ux[e], uy[e], cs, sn, sur, -sui, cur, -cui);
+              stcg(&tp[j], ux[e]);
+              stcg(&tq[j], uy[e]);
+            }
+          }
+        } else if (uregs) {
 #pragma unroll
           for (int e = 0; e < E; ++e) {
             const int j = tid + OSJ_NT * e;
