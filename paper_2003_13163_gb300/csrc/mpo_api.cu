@@ -75,7 +75,8 @@ struct BatchState;
 // the handle issues).
 struct OzWork {
   __nv_bfloat16 *a = nullptr, *b = nullptr;
-  int *ea = nullptr, *eb = nullptr, *status = nullptr;
+  int *ea = nullptr, *eb = nullptr, *status = nullptr, *counters = nullptr;
+  double2* part = nullptr;         // sums of the K parts of small products; NULL: never split
   size_t a_cap = 0, b_cap = 0;     // elements
   int e_cap = 0;
 };
@@ -557,17 +558,30 @@ static cudaError_t oz_gemm(cudaStream_t st, int M, int N, int K, const double2* 
   if (e != cudaSuccess) return e;
   e = ensure_dynamic_smem((const void*)oz_mma_kernel, oz::SMEM_BYTES);
   if (e != cudaSuccess) return e;
-  const OzTiles tl{Mp / oz::BM, Nrp / oz::BN, nkb, mode};
-  oz_mma_kernel<<<std::min(num_sms, tl.count()), oz::NT, oz::SMEM_BYTES, st>>>(tl, a, b, C, ldc, alpha, accumulate,
+  // a tile takes ~0.7 us per stage: split K while tiles leave SMs idle, into parts
+  // of at least twenty stages (parts of eight made the K = 256 products of a short
+  // chain's circuit slower: 222 -> 226 ms; 513 x 300 x 1100: 405 us whole, 349 in three)
+  OzTiles tl{Mp / oz::BM, Nrp / oz::BN, nkb, mode, 1};
+  if (w.part && 2 * tl.count() <= num_sms && num_sms <= oz::MAXITEMS)
+    tl.splits = std::max(1, std::min(std::min(oz::MAXSPLIT, num_sms / tl.count()), 2 * nkb / 20));
+  oz_mma_kernel<<<std::min(num_sms, tl.count() * tl.splits), oz::NT, oz::SMEM_BYTES, st>>>(tl, a, b, C, ldc, alpha, accumulate, w.part, w.counters,
                                                                                   w.status, (long long)(timeout_s * 1e9));
   return cudaGetLastError();
 }
 
+// Bytes for the K parts of every product of at most M x N that oz_gemm may split.
+static size_t oz_part_bytes(int M, int N, int num_sms) {
+  const size_t tiles = (size_t)((M + oz::BM - 1) / oz::BM) * (size_t)((2 * (size_t)N + oz::BN - 1) / oz::BN);
+  return std::min((size_t)num_sms, tiles * oz::MAXSPLIT) * oz::PART_BYTES;
+}
+
 // Scratch of products with at most M rows, N columns and inner dimension K, from
 // `alloc` (void**, bytes): the slices of both operands, and one block of
-// exponents of A, of B and the status word.
+// exponents of A, of B, the status word and the counters of split tiles (the last
+// two zeroed by the caller); `part` bytes for the parts of split products (oz_part_bytes; 0:
+// products are not split).
 template <typename F>
-static bool alloc_oz(OzWork& w, int M, int N, int K, F alloc) {
+static bool alloc_oz(OzWork& w, int M, int N, int K, size_t part, F alloc) {
   const size_t Mp = (size_t)(M + oz::BM - 1) / oz::BM * oz::BM;
   const size_t Nrp = (size_t)(2 * (size_t)N + oz::BN - 1) / oz::BN * oz::BN;
   const size_t Kp = 32 * (size_t)((K + 15) / 16);
@@ -575,13 +589,14 @@ static bool alloc_oz(OzWork& w, int M, int N, int K, F alloc) {
   w.b_cap = (size_t)oz::S * Nrp * Kp;
   w.e_cap = (int)std::max(Mp, Nrp);
   if (!alloc((void**)&w.a, w.a_cap * sizeof(__nv_bfloat16)) || !alloc((void**)&w.b, w.b_cap * sizeof(__nv_bfloat16)) ||
-      !alloc((void**)&w.ea, (2 * (size_t)w.e_cap + 1) * sizeof(int)))
+      !alloc((void**)&w.ea, (2 * (size_t)w.e_cap + 1 + oz::MAXITEMS) * sizeof(int)))
     return false;
   if (w.ea) {
     w.eb = w.ea + w.e_cap;
     w.status = w.ea + 2 * (size_t)w.e_cap;
+    w.counters = w.status + 1;
   }
-  return true;
+  return part == 0 || alloc((void**)&w.part, part);
 }
 
 // Products large enough to fill 128 x 128 real tiles go to the tensor cores.
@@ -1719,6 +1734,10 @@ int mpo_init(mpo_handle* out, int n, int chi_max, mpo_precision prec, void* stre
 
   auto alloc = [&](void** p, size_t bytes) -> bool { return ws_alloc(h, p, bytes); };
   h->site.assign(n, nullptr);
+  const size_t room = h->opts.arena_cap_bytes > 0 ? h->opts.arena_cap_bytes - need : ~(size_t)0;
+  // only saves time, so a handle whose memory limit has no room goes without
+  const size_t oz_want = oz_part_bytes(std::max(m, mx_ccap), std::max(m, mx_ccap), h->num_sms);
+  const size_t oz_part = oz_want <= room ? oz_want : 0;
   auto list = [&](bool lq) -> bool {
     bool ok = true;
     for (int k = 0; k < n && ok; ++k) ok = alloc(&h->site[k], h->site_cap * h->esz);
@@ -1732,7 +1751,7 @@ int mpo_init(mpo_handle* out, int n, int chi_max, mpo_precision prec, void* stre
     ok = ok && alloc((void**)&h->dsup, 256 * sizeof(double2));
     ok = ok && alloc_factor_ws(h, m, mx_ccap, bj_nch);
     const int d = std::max(m, mx_ccap);
-    if (ok && h->use_oz) ok = alloc_oz(h->oz, d, d, d, alloc);
+    if (ok && h->use_oz) ok = alloc_oz(h->oz, d, d, d, oz_part, alloc);
     ok = ok && alloc((void**)&h->scal, 8 * sizeof(double));
     ok = ok && alloc((void**)&h->dS, (size_t)(n - 1) * sizeof(double));
     ok = ok && alloc((void**)&h->dschmidt, (size_t)(n - 1) * chi_max * sizeof(double));
@@ -1741,11 +1760,10 @@ int mpo_init(mpo_handle* out, int n, int chi_max, mpo_precision prec, void* stre
     if (ok && lq) ok = alloc_lq(h, m, mx_ccap);
     return ok;
   };
-  const size_t room = h->opts.arena_cap_bytes > 0 ? h->opts.arena_cap_bytes - need : ~(size_t)0;
   if (!ws_build_lq(h, m, mx_ccap, need, room, list)) return init_fail(h, MPO_ERR_OOM, "cudaMalloc failed");
   h->hs = hostsync_get();
   if (!h->hs) return init_fail(h, MPO_ERR_CUDA, "cudaHostAlloc failed");
-  if (h->use_oz && cudaMemsetAsync(h->oz.status, 0, sizeof(int), h->st) != cudaSuccess)
+  if (h->use_oz && cudaMemsetAsync(h->oz.status, 0, (1 + oz::MAXITEMS) * sizeof(int), h->st) != cudaSuccess)
     return init_fail(h, MPO_ERR_CUDA, "initial state upload failed");
   // product state |0..0><0..0|: every site 1 x 4 x 1 with A[0][0][0] = 1 (Sec. 4.1)
   std::vector<unsigned char> one(h->esz, 0);
@@ -2116,7 +2134,7 @@ int mpo_svd_truncated(int r, int c, const void* A, int cap, mpo_precision prec, 
   auto alloc = [&](void** p, size_t bytes) -> bool { return ws_alloc(h, p, bytes); };
   auto list = [&](bool lq) -> bool {
     return alloc(&h->theta, (size_t)r * c * h->esz) && alloc_factor_ws(h, r, c, nch) &&
-           alloc((void**)&h->scal, 8 * sizeof(double)) && (!h->use_oz || alloc_oz(h->oz, c, c, c, alloc)) &&
+           alloc((void**)&h->scal, 8 * sizeof(double)) && (!h->use_oz || alloc_oz(h->oz, c, c, c, h->opts.arena_cap_bytes > 0 ? 0 : oz_part_bytes(c, c, h->num_sms), alloc)) &&
            (!lq || alloc_lq(h, r, c));
   };
   bool ok = ws_build_lq(h, r, c, 0, h->opts.arena_cap_bytes > 0 ? 0 : ~(size_t)0, list);
@@ -2127,7 +2145,7 @@ int mpo_svd_truncated(int r, int c, const void* A, int cap, mpo_precision prec, 
   ck(cudaMemcpyAsync(h->theta, A, (size_t)r * c * h->esz, cudaMemcpyDeviceToDevice, h->st));
   ck(cudaMemsetAsync(h->scal, 0, 8 * sizeof(double), h->st));
   ck(cudaMemsetAsync(h->tc_status, 0, sizeof(int), h->st));
-  if (h->use_oz) ck(cudaMemsetAsync(h->oz.status, 0, sizeof(int), h->st));
+  if (h->use_oz) ck(cudaMemsetAsync(h->oz.status, 0, (1 + oz::MAXITEMS) * sizeof(int), h->st));
   if (rc == MPO_OK) {
     rc = prec != MPO_FP32 ? svd_select<double>(h, (double2*)h->theta, r, c, c, cap, true, nullptr, nullptr, &kk)
                           : svd_select<float>(h, (float2*)h->theta, r, c, c, cap, true, nullptr, nullptr, &kk);
@@ -2286,11 +2304,11 @@ int mpo_gemm_ex(int M, int N, int K, const void* A, int lda, int opA, const void
       off += (bytes + 255) & ~(size_t)255;
       return true;
     };
-    alloc_oz(w, M, N, K, carve);
+    alloc_oz(w, M, N, K, oz_part_bytes(M, N, sms), carve);
     if (cudaMalloc((void**)&base, off) != cudaSuccess) { cudaGetLastError(); return MPO_ERR_OOM; }
     off = 0;
-    alloc_oz(w, M, N, K, carve);
-    e = cudaMemsetAsync(w.status, 0, sizeof(int), st);
+    alloc_oz(w, M, N, K, oz_part_bytes(M, N, sms), carve);
+    e = cudaMemsetAsync(w.status, 0, (1 + oz::MAXITEMS) * sizeof(int), st);
     if (e == cudaSuccess)
       e = oz_gemm(st, M, N, K, (const double2*)A, lda, opA, (const double2*)B, ldb, opB, (double2*)C, ldc, 1.0, 0, w,
                   5.0, sms);

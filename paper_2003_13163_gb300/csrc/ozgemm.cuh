@@ -79,6 +79,9 @@ constexpr int NDRAIN = 8;                    // drain warps: 4 TMEM lane groups 
 constexpr int NT = 32 * (NDRAIN + 2);
 constexpr int TCOLS = 512;                   // TMEM allocation (power of two >= S * BN)
 static_assert(S * BN <= TCOLS, "accumulators exceed the TMEM allocation");
+constexpr int MAXSPLIT = 8;                  // parts of a tile's K range
+constexpr int MAXITEMS = 256;                // (tile, part) items of a split product, at most the SMs
+constexpr size_t PART_BYTES = (size_t)BM * BN * sizeof(double);   // a part's sums
 
 // Shared-memory matrix descriptor, K-major, no swizzle: start address, LBO
 // (byte step between the core matrices of consecutive K groups), SBO = 128 B
@@ -255,6 +258,10 @@ struct OzTiles {
   enum { kGeneral = 0, kHerm = 1, kUpper = 2 };
   int nrb, ncb, nkb;      // row blocks, column blocks, blocks of 16 complex k
   int mode;
+  // K parts per tile. A product with fewer tiles than SMs splits K between CTAs,
+  // one item each: the parts' sums go to global memory and the CTA that finishes a
+  // tile last adds them in order of k, so the result does not depend on the timing.
+  int splits;
   __host__ __device__ __forceinline__ int count() const {
     if (mode != kHerm) return nrb * ncb;
     int n = 0;
@@ -278,6 +285,13 @@ struct OzTiles {
     cb = w / h;
   }
   __device__ __forceinline__ int stages(int cb) const { return 2 * (mode == kUpper ? min(nkb, 2 * cb + 2) : nkb); }
+  // the item's tile, its part and its range of stages
+  __device__ __forceinline__ void item(int id, int& rb, int& cb, int& s0, int& s1) const {
+    tile(id / splits, rb, cb);
+    const int n = stages(cb), q = id % splits;
+    s0 = n * q / splits;
+    s1 = n * (q + 1) / splits;
+  }
 };
 
 #define OZ_LD32(v, taddr)                                                                                      \
@@ -294,14 +308,14 @@ struct OzTiles {
 // an mbarrier wait ran past timeout_ns (the CTA's remaining tiles are then left
 // unwritten).
 __global__ void __launch_bounds__(oz::NT, 1) oz_mma_kernel(OzTiles tl, OzOp a, OzOp b, double2* __restrict__ C, int ldc,
-                                                           double alpha, int accumulate, int* status,
-                                                           long long timeout_ns) {
+                                                           double alpha, int accumulate, double2* part, int* counters,
+                                                           int* status, long long timeout_ns) {
   using namespace oz;
   extern __shared__ __align__(1024) unsigned char oz_raw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>(((uintptr_t)oz_raw + 1023) & ~(uintptr_t)1023);
-  __shared__ __align__(8) uint64_t full[NSTAGE], empty[NSTAGE], acc_full, acc_empty;
+  __shared__ __align__(8) uint64_t full[NSTAGE], empty[NSTAGE], acc_full, acc_empty, part_done, last_known;
   __shared__ uint32_t tmem_base;
-  __shared__ int s_fail;
+  __shared__ int s_fail, s_last;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
   if (warp == 0) {
@@ -315,6 +329,8 @@ __global__ void __launch_bounds__(oz::NT, 1) oz_mma_kernel(OzTiles tl, OzOp a, O
     }
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(tcg::saddr(&acc_full)));
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(tcg::saddr(&acc_empty)), "n"(NDRAIN));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(tcg::saddr(&part_done)), "n"(NDRAIN));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(tcg::saddr(&last_known)));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     s_fail = 0;
   }
@@ -328,7 +344,7 @@ __global__ void __launch_bounds__(oz::NT, 1) oz_mma_kernel(OzTiles tl, OzOp a, O
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tbase = tmem_base;
-  const int ntiles = tl.count();
+  const int ntiles = tl.count() * tl.splits;
   volatile int* fail = &s_fail;
 
   if (warp == NDRAIN) {
@@ -337,12 +353,11 @@ __global__ void __launch_bounds__(oz::NT, 1) oz_mma_kernel(OzTiles tl, OzOp a, O
       int it = 0;
       bool ok = true;
       for (int id = blockIdx.x; id < ntiles && ok; id += gridDim.x) {
-        int rb, cb;
-        tl.tile(id, rb, cb);
-        const int nst = tl.stages(cb);
+        int rb, cb, s0, s1;
+        tl.item(id, rb, cb, s0, s1);
         const unsigned char* pa = reinterpret_cast<const unsigned char*>(a.sl) + (size_t)rb * 2 * tl.nkb * A_STAGE;
         const unsigned char* pb = reinterpret_cast<const unsigned char*>(b.sl) + (size_t)cb * 2 * tl.nkb * B_STAGE;
-        for (int s = 0; s < nst; ++s, ++it) {
+        for (int s = s0; s < s1; ++s, ++it) {
           const int slot = it % NSTAGE;
           if (it >= NSTAGE && !tcg::wait_parity(tcg::saddr(&empty[slot]), (uint32_t)(it / NSTAGE - 1) & 1u, timeout_ns)) ok = false;
           if (!ok || *fail) { ok = false; break; }
@@ -370,9 +385,9 @@ __global__ void __launch_bounds__(oz::NT, 1) oz_mma_kernel(OzTiles tl, OzOp a, O
       int it = 0, chunk = 0;
       bool ok = true;
       for (int id = blockIdx.x; id < ntiles && ok; id += gridDim.x) {
-        int rb, cb;
-        tl.tile(id, rb, cb);
-        const int nst = tl.stages(cb);
+        int rb, cb, s0, s1;
+        tl.item(id, rb, cb, s0, s1);
+        const int nst = s1 - s0;
         for (int s = 0; s < nst; ++s, ++it) {
           const int slot = it % NSTAGE;
           const bool first = s % SPC == 0;
@@ -411,12 +426,13 @@ __global__ void __launch_bounds__(oz::NT, 1) oz_mma_kernel(OzTiles tl, OzOp a, O
     // ---- drain and epilogue ------------------------------------------------
     const int lg = warp & 3, half = warp >> 2;      // rows 32 lg .., real columns 32 half .. of each level
     const uint32_t tl0 = tbase + ((uint32_t)(32 * lg) << 16) + 32 * half;
+    uint32_t pphase = 0;
     int chunk = 0;
     bool ok = true;
     for (int id = blockIdx.x; id < ntiles && ok; id += gridDim.x) {
-      int rb, cb;
-      tl.tile(id, rb, cb);
-      const int nch = (tl.stages(cb) + SPC - 1) / SPC;
+      int rb, cb, s0, s1;
+      tl.item(id, rb, cb, s0, s1);
+      const int nch = (s1 - s0 + SPC - 1) / SPC;
       float hi[32], lo[32];
 #pragma unroll
       for (int j = 0; j < 32; ++j) { hi[j] = 0.f; lo[j] = 0.f; }
@@ -442,6 +458,40 @@ __global__ void __launch_bounds__(oz::NT, 1) oz_mma_kernel(OzTiles tl, OzOp a, O
         }
       }
       if (!ok) break;
+      double2 sum[16];
+#pragma unroll
+      for (int q = 0; q < 16; ++q)
+        sum[q] = make_double2((double)hi[2 * q] + (double)lo[2 * q], (double)hi[2 * q + 1] + (double)lo[2 * q + 1]);
+      if (tl.splits > 1) {
+        // item's block of part: [complex column][128 rows], so a warp writes 512
+        // consecutive bytes; the drain warps meet on mbarriers (bounded waits)
+        double2* mine = part + (size_t)id * (BM * BN / 2) + (size_t)(16 * half) * BM + 32 * lg + lane;
+#pragma unroll
+        for (int q = 0; q < 16; ++q) stcg(&mine[(size_t)q * BM], sum[q]);
+        __threadfence();
+        const int tile = id / tl.splits;
+        __syncwarp();
+        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(tcg::saddr(&part_done)) : "memory");
+        ok = __all_sync(0xffffffffu, tcg::wait_parity(tcg::saddr(&part_done), pphase, timeout_ns));
+        if (!ok) break;
+        if (tid == 0) {
+          s_last = atomicAdd(&counters[tile], 1) == tl.splits - 1;
+          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(tcg::saddr(&last_known)) : "memory");
+        }
+        ok = __all_sync(0xffffffffu, tcg::wait_parity(tcg::saddr(&last_known), pphase, timeout_ns));
+        if (!ok) break;
+        pphase ^= 1u;
+        if (!s_last) continue;
+        __threadfence();
+        if (tid == 0) counters[tile] = 0;            // for the next launch
+        const double2* all = part + (size_t)tile * tl.splits * (BM * BN / 2) + (size_t)(16 * half) * BM + 32 * lg + lane;
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+          double2 v = ldcg(&all[(size_t)q * BM]);
+          for (int p = 1; p < tl.splits; ++p) v = cadd<double>(v, ldcg(&all[(size_t)p * (BM * BN / 2) + (size_t)q * BM]));
+          sum[q] = v;
+        }
+      }
       const int row = rb * BM + 32 * lg + lane;
       const int er = row < a.n ? oz_ex(a.raw[row]) : 0;
 #pragma unroll
@@ -449,8 +499,8 @@ __global__ void __launch_bounds__(oz::NT, 1) oz_mma_kernel(OzTiles tl, OzOp a, O
         const int j = cb * (BN / 2) + 16 * half + q;   // complex column: real part 2q, imaginary 2q + 1
         if (row >= a.n || j >= b.n) continue;
         const int sc = er + oz_ex(b.raw[j]);
-        double re = ldexp((double)hi[2 * q] + (double)lo[2 * q], sc) * alpha;
-        double im = ldexp((double)hi[2 * q + 1] + (double)lo[2 * q + 1], sc) * alpha;
+        double re = ldexp(sum[q].x, sc) * alpha;
+        double im = ldexp(sum[q].y, sc) * alpha;
         if (tl.mode == OzTiles::kHerm) {
           if (row > j) continue;
           if (row < j) C[(size_t)j * ldc + row] = make_double2(re, -im);
