@@ -57,9 +57,9 @@ FP64_PROBE_TFLOPS = 1.20
 FP32_PROBE_TFLOPS = 74.6
 # DRAM bytes (read + written) per algorithmic flop of the split-BF16 GEMM,
 # from an ncu capture of one 4096 x 2048 x 4096 complex product
-# (dram__bytes_read.sum + dram__bytes_write.sum = 6.418e9 B for 2.749e11 flop);
+# (dram__bytes_read.sum + dram__bytes_write.sum = 4.007e9 B for 2.749e11 flop);
 # the traffic of an average launch scales with its flops
-OZ_DRAM_BYTES_PER_FLOP = 6.418e9 / 2.749e11
+OZ_DRAM_BYTES_PER_FLOP = 4.007e9 / 2.749e11
 
 
 def load_peaks() -> dict:

@@ -17,14 +17,15 @@
 //   1. move the centre to i or i+1 (QR-type moves, below);
 //   2. theta = L(A_i) R(A_{i+1})                       (complex GEMM)
 //   3. theta' = M theta on (I, J)                      (superoperator kernel)
-//   4. Gram of the smaller side, Hermitian eigen-solve (Jacobi), select the
-//      chi_max largest lambda'^2 (App. A truncation), discarded weight;
+//   4. SVD of theta' (of its conjugate transpose when that has fewer rows) in
+//      the form's arithmetic, select the chi_max largest lambda'^2 (App. A
+//      truncation), discarded weight;
 //   5. write back: left isometry -> site i, Lambda W^H / ||kept|| -> site i+1.
-// Centre moves and the sweep use the same Gram/eigen route: for the centre C,
-// G = C^H C (or C C^H) = V diag(sigma^2) V^H, the isometry is C V Sigma^-1 (or
-// Sigma^-1 V^H C) and Sigma V^H (or V Sigma) is pushed into the neighbour;
-// sigma <= cutoff * sigma_max are dropped (they are below the rounding floor
-// of the Gram). The sweep's sigma at bond b are the Schmidt values lambda^[b].
+// Centre moves and the sweep use the same SVD: for the centre C = U Sigma V^H the
+// isometry U (or V^H) stays and Sigma V^H (or U Sigma) is pushed into the
+// neighbour; sigma <= cutoff * sigma_max are dropped. The sweep's sigma at bond b
+// are the Schmidt values lambda^[b]. The precision form's moves that record
+// nothing use a Cholesky QR isometry instead.
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -607,7 +608,8 @@ static bool oz_worth(int M, int N, int K) { return (double)M * N * K >= 2.6e5 &&
 static cudaError_t mx_gemm(mpo_ctx* h, int M, int N, int K, const double2* A, int lda, int opA, const double2* B,
                            int ldb, int opB, double2* C, int ldc, double alpha = 1.0, int accumulate = 0,
                            int mode = OzTiles::kGeneral) {
-  ProfScope ps(h, PK_REFINE, 8.0 * M * N * K, (double)((size_t)M * K + (size_t)K * N + (size_t)M * N) * sizeof(double2));
+  // a Hermitian product and one with a triangular factor are half the work
+  ProfScope ps(h, PK_REFINE, (mode == OzTiles::kGeneral ? 8.0 : 4.0) * M * N * K, (double)((size_t)M * K + (size_t)K * N + (size_t)M * N) * sizeof(double2));
   if (h->use_oz && oz_worth(M, N, K)) {
     ps.cls = PK_OZ;
     return oz_gemm(h->st, M, N, K, A, lda, opA, B, ldb, opB, C, ldc, alpha, accumulate, h->oz,
