@@ -411,6 +411,9 @@ __global__ void hermitise_kernel(double2* __restrict__ H, int m) {
 // orthogonality term R_ji / 2 alone. Among the leading columns it saves the FP64
 // eigen-solve that follows a sweep; there a pair is taken where |E_ji| <= 1e-3, so
 // that V_P (I + E_PP) stays within reach of the Newton-Schulz steps, else R_ji / 2.
+// A pair without a gap is never taken: exactly equal values with no coupling
+// (zero rows, equal rows, a multiple of the identity) have 0 / 0 there, and any
+// basis of their span is one of eigenvectors.
 // Output (m x mp): rows j < mp are I + E_PP, the others E_RP.
 __global__ void partition_correction_kernel(const double2* __restrict__ S, const double2* __restrict__ G, int m, int mp,
                                             double2* __restrict__ E) {
@@ -425,7 +428,7 @@ __global__ void partition_correction_kernel(const double2* __restrict__ S, const
     const double2 rji = make_double2(-g.x, -g.y);      // (I - G)_ji, j != i
     const double gap = li - lj;
     const double2 num = make_double2(s.x + li * rji.x, s.y + li * rji.y);
-    const bool far = j < mp ? fmax(fabs(num.x), fabs(num.y)) <= 1e-3 * fabs(gap)
+    const bool far = j < mp ? fabs(gap) > 0.0 && fmax(fabs(num.x), fabs(num.y)) <= 1e-3 * fabs(gap)
                             : fabs(gap) > 1e-2 * fmax(fabs(li), fabs(lj));
     E[e] = far ? make_double2(num.x / gap, num.y / gap) : make_double2(0.5 * rji.x, 0.5 * rji.y);
   }
