@@ -60,7 +60,7 @@ struct HostSync {   // pinned read-back of the last select + eigen-solve
   GridCtl ctl;
   unsigned long long phase_ns[4];
   int tc_err;
-  GridCtl lq;         // control block of the FP64 form's LQ and FP32 solves
+  GridCtl lq[2];      // control blocks of the FP64 form's LQ step and of its FP32 start
   GridCtl eig[8];     // FP64 eigen-solves of the last mixed factorisation
   int chol_status;    // Cholesky QR pivot status of the last mixed factorisation
   int chol_pass[2];   // status words after a Cholesky QR pass (cholqr_factor_kernel)
@@ -83,8 +83,9 @@ struct OzWork {
 };
 
 // Workspace of the LQ-preconditioned SVD: the reflectors (z, m x ccap) with their
-// factors and first entries (f, zd), three m x m matrices, the control block of
-// the LQ and FP32 solves.
+// factors and first entries (f, zd), three m x m matrices, the control blocks of
+// the LQ step and of the FP32 start (a launch zeroes its own, so one block for
+// both would lose the first one's errors).
 struct LqWork {
   double2 *z = nullptr, *w = nullptr, *s = nullptr, *v = nullptr, *zd = nullptr;
   double* f = nullptr;
@@ -399,8 +400,8 @@ constexpr int kLqMinRows = 8;
 constexpr int kPreMinRows = 32;
 
 // X (r x c, r <= c) <- the rows Sigma V^H, vecs (r x r) <- rows conj(column of
-// U), w <- sigma^2 (lq_kernel). q.ctl and ctl receive the barrier errors of the
-// first two kernels and of the FP64 solve.
+// U), w <- sigma^2 (lq_kernel). q.ctl[0], q.ctl[1] and ctl receive the barrier
+// errors of the LQ step, of the FP32 start and of the FP64 solve.
 static cudaError_t launch_lq_jacobi(cudaStream_t st, double2* X, int r, int c, int ldx, double2* vecs, double* w,
                                     const LqWork& q, OSCtl* ctl, int max_sweeps, double timeout_s, int num_sms) {
   const bool small = c <= 2 * OSJ_NT;
@@ -410,7 +411,7 @@ static cudaError_t launch_lq_jacobi(cudaStream_t st, double2* X, int r, int c, i
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const int blocks = std::max(1, std::min(std::min(per_sm, 4) * num_sms, r));
-  e = cudaMemsetAsync(q.ctl, 0, sizeof(OSCtl), st);
+  e = cudaMemsetAsync(q.ctl, 0, 2 * sizeof(OSCtl), st);
   if (e != cudaSuccess) return e;
   long long timeout_ns = (long long)(timeout_s * 1e9);
   LqWork k = q;
@@ -429,7 +430,7 @@ static cudaError_t launch_lq_jacobi(cudaStream_t st, double2* X, int r, int c, i
     max_exp_kernel<<<grid_for(n, num_sms), 256, 0, st>>>(vecs, n, q.ex);
     scale_fp32_kernel<<<grid_for(n, num_sms), 256, 0, st>>>(vecs, n, q.ex, a32);
     // a start only: sixteen sweeps at most, and no failure if they run out
-    e = launch_fp32_jacobi(st, a32, r, r, r, u32, (float*)w, q.ctl, 16, timeout_s, num_sms, 0.0);
+    e = launch_fp32_jacobi(st, a32, r, r, r, u32, (float*)w, q.ctl + 1, 16, timeout_s, num_sms, 0.0);
     if (e != cudaSuccess) return e;
     transpose_kernel<float2><<<tg, tb, 0, st>>>(u32, r, r, q.v);                       // W, row-major
     if ((e = cgemm<double>(st, r, r, r, q.v, r, 1, q.v, r, 0, X, r)) != cudaSuccess) return e;   // W^H W (X is free: Z holds the matrix)
@@ -978,10 +979,11 @@ static int svd_select(mpo_ctx* h, cplx<T>* X, int r, int c, int ldx, int cap, bo
   CK(h, cudaMemcpyAsync(&h->hs->ctl, &h->osctl->g, sizeof(GridCtl), cudaMemcpyDeviceToHost, h->st));
   if (h->prof) CK(h, cudaMemcpyAsync(h->hs->phase_ns, h->osctl->phase_ns, sizeof(h->hs->phase_ns), cudaMemcpyDeviceToHost, h->st));
   CK(h, cudaMemcpyAsync(&h->hs->tc_err, h->tc_status, sizeof(int), cudaMemcpyDeviceToHost, h->st));
-  h->hs->lq.err = 0;
-  if (h->vecs_conj) CK(h, cudaMemcpyAsync(&h->hs->lq, &h->lq.ctl->g, sizeof(GridCtl), cudaMemcpyDeviceToHost, h->st));
+  h->hs->lq[0].err = h->hs->lq[1].err = 0;
+  if (h->vecs_conj)
+    CK(h, cudaMemcpy2DAsync(h->hs->lq, sizeof(GridCtl), &h->lq.ctl->g, sizeof(OSCtl), sizeof(GridCtl), 2, cudaMemcpyDeviceToHost, h->st));
   CK(h, cudaStreamSynchronize(h->st));
-  if (h->hs->lq.err) return fail(h, MPO_ERR_TIMEOUT, "grid barrier wait timed out in the SVD");
+  if (h->hs->lq[0].err || h->hs->lq[1].err) return fail(h, MPO_ERR_TIMEOUT, "grid barrier wait timed out in the SVD");
   if (h->hs->tc_err) return fail(h, MPO_ERR_TIMEOUT, "an mbarrier wait timed out in the tensor-core GEMM");
   if (h->prof) for (int i = 0; i < 3; ++i) h->prof_phase_ns[i] += h->hs->phase_ns[i];
   if (h->hs->ctl.err) return fail(h, MPO_ERR_TIMEOUT, "grid barrier wait timed out in the SVD");
@@ -1619,7 +1621,7 @@ static bool alloc_factor_ws(mpo_ctx* h, int m, int ccap, size_t bj_nch) {
 // Workspace of the FP64 form's LQ step.
 static size_t lq_bytes(int m, int ccap) {
   return ((size_t)m * ccap + 3 * (size_t)m * m) * sizeof(double2) + (size_t)m * (sizeof(double2) + sizeof(double)) +
-         sizeof(OSCtl) + sizeof(int) + 8 * 256;
+         2 * sizeof(OSCtl) + sizeof(int) + 8 * 256;
 }
 
 static bool alloc_lq(mpo_ctx* h, int m, int ccap) {
@@ -1628,7 +1630,7 @@ static bool alloc_lq(mpo_ctx* h, int m, int ccap) {
   return ws_alloc(h, (void**)&q.z, (size_t)m * ccap * sizeof(double2)) && ws_alloc(h, (void**)&q.w, w) &&
          ws_alloc(h, (void**)&q.s, w) && ws_alloc(h, (void**)&q.v, w) &&
          ws_alloc(h, (void**)&q.zd, (size_t)m * sizeof(double2)) && ws_alloc(h, (void**)&q.f, (size_t)m * sizeof(double)) &&
-         ws_alloc(h, (void**)&q.ctl, sizeof(OSCtl)) && ws_alloc(h, (void**)&q.ex, sizeof(int));
+         ws_alloc(h, (void**)&q.ctl, 2 * sizeof(OSCtl)) && ws_alloc(h, (void**)&q.ex, sizeof(int));
 }
 
 // All buffers of a handle: `list(lq)` allocates them, with the LQ workspace if lq
