@@ -535,11 +535,19 @@ __device__ __forceinline__ double osj_pow2(int k) { return __longlong_as_double(
 // rotation leaves 1e-14 of g); c and u come from osj_rsqrt, so c^2 + s^2 and
 // |u| are 1 to FP64 rounding whatever the angle. g is scaled by a power of two
 // first (integer arithmetic on its exponent), so no square over- or underflows.
+// A denormal g has too few bits for a rotation: none is made, and unresolved (if
+// given) is set when it is still above the threshold (rows below ~1e-150), so that
+// the solve ends unconverged instead of taking such rows for orthogonal.
 __device__ __forceinline__ bool osj_rotation(double a, double b, double gr, double gi, double tol2, double floor_abs,
-                                             double& c, double& s, double& ur, double& ui) {
+                                             double& c, double& s, double& ur, double& ui,
+                                             bool* unresolved = nullptr) {
   const int er = (int)((__double_as_longlong(gr) >> 52) & 0x7FF), ei = (int)((__double_as_longlong(gi) >> 52) & 0x7FF);
   const int e = max(er, ei) - 1023;
-  if (e <= -1022 || e >= 1022) return false;      // zero, denormal, infinite or NaN couplings
+  if (e <= -1022) {
+    if (unresolved) *unresolved = fmax(fabs(gr), fabs(gi)) > fmax(sqrt(tol2) * (sqrt(a) * sqrt(b)), floor_abs);
+    return false;
+  }
+  if (e >= 1022) return false;                    // infinite or NaN couplings
   const double sc = osj_pow2(-e);
   const double x = gr * sc, y = gi * sc;
   const double g2 = fma(x, x, y * y);             // in [1, 8)
@@ -838,10 +846,12 @@ __global__ void __launch_bounds__(OSJ_NT) pair_jacobi_kernel(cplx<T>* X, int r, 
         osj_reduce4<T>(a, b, gr, gi, part);
         if (tid < 32) {
           double cs, sn, ur, ui;
-          const bool on = osj_rotation((double)a, (double)b, (double)gr, (double)gi, tol2, floor_abs, cs, sn, ur, ui) &&
-                          (T)sn != T(0);
+          bool unresolved = false;
+          const bool on = osj_rotation((double)a, (double)b, (double)gr, (double)gi, tol2, floor_abs, cs, sn, ur, ui,
+                                       &unresolved) && (T)sn != T(0);
           if (tid == 0) {
             s_rot.on = on;
+            if (unresolved) atomicAdd(&ctl->active[sweep], 1);
             if (on) {
               s_rot.c = (T)cs; s_rot.s = (T)sn;
               s_rot.sur = (T)(sn * ur); s_rot.sui = (T)(sn * ui);
@@ -1226,6 +1236,10 @@ __device__ __forceinline__ double lq_rsqrt(double x) {
 
 // Z (r x c) <- X with row j's reflector z_j left in columns j .. c - 1 (its
 // first entry in zd[j]), H_j = I - f_j z_j^H z_j; Y (r x r) <- L^H. r <= c.
+// A row whose squared norm is not above 1e-300 (less than that, denormal squares
+// cost it its accuracy) counts as zero; ctl->g.sweeps receives the largest biased exponent
+// of such a squared norm plus 1, 0 if there was none but exact zeros, and the caller refuses
+// the factorisation when that is not negligible beside the whole (rows below ~1e-150).
 template <int E>
 __global__ void __launch_bounds__(OSJ_NT) lq_kernel(const double2* __restrict__ X, int ldx, int r, int c, double2* Z,
                                                     double2* Y, double* f, double2* zd, OSCtl* ctl,
@@ -1236,6 +1250,7 @@ __global__ void __launch_bounds__(OSJ_NT) lq_kernel(const double2* __restrict__ 
   const unsigned nblk = gridDim.x;
   const int tid = threadIdx.x;
   const bool regs = c <= OSJ_NT * E;
+  int dropped = 0;
   for (int i = blockIdx.x; i < r; i += nblk) {
     for (int k = tid; k < c; k += OSJ_NT) stcg(&Z[(size_t)i * c + k], X[(size_t)i * ldx + k]);
     for (int k = tid; k < r; k += OSJ_NT) stcg(&Y[(size_t)i * r + k], czero<double>());
@@ -1295,6 +1310,8 @@ __global__ void __launch_bounds__(OSJ_NT) lq_kernel(const double2* __restrict__ 
           }
           fj = inv * lq_rsqrt(1.0 + au);                       // f = (fj)^2
           fj = fj * fj;
+        } else if (n2 > 0.0) {
+          dropped = max(dropped, (int)(__double_as_longlong(n2) >> 52) + 1);
         }
         const double2 ps = make_double2(ph.x * nrm, ph.y * nrm);
         const double2 z0 = cadd<double>(x0, ps);
@@ -1357,6 +1374,7 @@ __global__ void __launch_bounds__(OSJ_NT) lq_kernel(const double2* __restrict__ 
     }
     if (!grid_barrier(&ctl->g, nblk, timeout_ns)) return;
   }
+  if (blockIdx.x == 0 && tid == 0) ctl->g.sweeps = dropped;
 }
 
 // Row j of the factorisation from the Jacobi result (Y rows Sigma U^H, Wt row j

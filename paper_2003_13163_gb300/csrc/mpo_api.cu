@@ -984,6 +984,9 @@ static int svd_select(mpo_ctx* h, cplx<T>* X, int r, int c, int ldx, int cap, bo
     CK(h, cudaMemcpy2DAsync(h->hs->lq, sizeof(GridCtl), &h->lq.ctl->g, sizeof(OSCtl), sizeof(GridCtl), 2, cudaMemcpyDeviceToHost, h->st));
   CK(h, cudaStreamSynchronize(h->st));
   if (h->hs->lq[0].err || h->hs->lq[1].err) return fail(h, MPO_ERR_TIMEOUT, "grid barrier wait timed out in the SVD");
+  // rows that the LQ step took for zero: refused unless negligible (2^-104 of the whole)
+  if (h->vecs_conj && h->hs->lq[0].sweeps > 0 && std::ldexp(1.0, h->hs->lq[0].sweeps - 1023) > std::ldexp(h->hs->info.total, -104))
+    return fail(h, MPO_ERR_NOCONV, "matrix too small: squared row norms underflow in the SVD");
   if (h->hs->tc_err) return fail(h, MPO_ERR_TIMEOUT, "an mbarrier wait timed out in the tensor-core GEMM");
   if (h->prof) for (int i = 0; i < 3; ++i) h->prof_phase_ns[i] += h->hs->phase_ns[i];
   if (h->hs->ctl.err) return fail(h, MPO_ERR_TIMEOUT, "grid barrier wait timed out in the SVD");
