@@ -233,7 +233,7 @@ __device__ __forceinline__ int rr_player(int pos, int r, int N) {
 //     norm of the factorised matrix, when w holds Ritz values of a subspace
 //     only), kept = sum of the k largest;
 //   - outputs perm[0..k), lam2[0..k) (descending), info->k, info->kept,
-//     info->total; adds (total-kept)/total to *disc_acc and 0.5 log(kept) to
+//     info->total, info->status (1: a value is infinite or NaN); adds (total-kept)/total to *disc_acc and 0.5 log(kept) to
 //     *lognorm when those are non-null;
 //   - with S_out: the MPO entanglement entropy -sum p log2 p, p = lam2/kept
 //     (Sec. 3.3), and the normalised lam2/kept into schmidt_out.
@@ -263,11 +263,12 @@ __global__ void __launch_bounds__(1024) select_kernel(const T* __restrict__ w, i
   __shared__ double s_tot, s_kept, s_max;
   __shared__ int s_k;
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wp = tid >> 5;
+  bool bad = false;
   for (int i = tid; i < P; i += nt) {
-    if (i < m) { double v = (double)w[i]; key[i] = v > 0.0 ? v : 0.0; idx[i] = i; }
+    if (i < m) { double v = (double)w[i]; key[i] = v > 0.0 ? v : 0.0; idx[i] = i; bad |= !isfinite(v); }
     else { key[i] = -1.0; idx[i] = 0x7fffffff; }
   }
-  __syncthreads();
+  const int any_bad = __syncthreads_or(bad);
   // bitonic sort, descending by key, ascending index on ties
   for (int size = 2; size <= P; size <<= 1) {
     for (int stride = size >> 1; stride > 0; stride >>= 1) {
@@ -338,6 +339,7 @@ __global__ void __launch_bounds__(1024) select_kernel(const T* __restrict__ w, i
   }
   if (tid == 0) {
     info->k = k;
+    info->status = any_bad ? 1 : 0;
     info->kept = kept;
     info->total = s_tot;
     info->inv_sqrt_kept = kept > 0.0 ? 1.0 / sqrt(kept) : 0.0;

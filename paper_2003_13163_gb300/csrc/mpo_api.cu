@@ -934,6 +934,8 @@ static int msvd_select(mpo_ctx* h, double2* X, int r, int c, int ldx, int cap, b
   if (h->hs->eig[0].err) return fail(h, MPO_ERR_TIMEOUT, "grid barrier wait timed out in the FP64 Rayleigh-Ritz eigen-solve");
   if (h->hs->eig[0].status)
     return fail(h, MPO_ERR_NOCONV, "FP64 Rayleigh-Ritz eigen-solve reached eig_max_sweeps (m = " + std::to_string(mp) + ")");
+  // NaN couplings end the solves above without a rotation
+  if (h->hs->info.status) return fail(h, MPO_ERR_NOCONV, "infinite or NaN values in the FP64 Rayleigh-Ritz eigen-solve");
   *k = h->hs->info.k;
   return MPO_OK;
 }
