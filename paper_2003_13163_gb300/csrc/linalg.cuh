@@ -1182,9 +1182,12 @@ __global__ void __launch_bounds__(QJ_NT) quad_jacobi_kernel(float2* X, int r, in
 // FP32 start. From kPreMinRows rows on, the FP32 solver first runs on fl32(R)
 // (scaled to a largest entry near 1), and the FP64 solve starts from W^H R and W,
 // W the FP32 left factor made orthonormal to FP64 rounding: with E = (I - W^H W)
-// / 2, W (I + E + 3/2 E^2 + 5/2 E^3) is off by 35/8 E^4 (E is at most ~5e-5, the
-// drift of the FP32 rotations). The FP64
-// unit runs at 1/64 of the FP32 rate, so its sweeps are what the solve costs, and
+// / 2, W (I + E + 3/2 E^2 + 5/2 E^3) is off by 35/8 E^4. E is the drift of the FP32
+// rotations and grows with the rows: 2-norm 1.1e-4 at 1024, 4.3e-4 at 4096, where
+// 35/8 E^4 left rows of X off by 2.8e-13. The host therefore reads its largest row
+// sum (a bound of the 2-norm, 2.5 to 3.5 times as large here) while the products
+// above run, and above kStartOnce takes one Newton-Schulz step more, above
+// kStartMax no start at all. The FP64 unit runs at 1/64 of the FP32 rate, so its sweeps are what the solve costs, and
 // five (the last of them quiet) remain of eleven; it stops by the same test as
 // without the start. Truncated SVD, LQ only -> with the start: 64 x 64 4.1 -> 2.8 ms,
 // 256 x 256 21.5 -> 17.5 ms, 577 x 600 116 -> 88 ms, 1024 x 1024 542 -> 350 ms;
@@ -1211,6 +1214,29 @@ __global__ void __launch_bounds__(256) scale_fp32_kernel(const double2* __restri
   for (size_t e = (size_t)blockIdx.x * 256 + threadIdx.x; e < n; e += (size_t)gridDim.x * 256) {
     const double2 x = R[e];
     out[e] = make_float2((float)(x.x * sc), (float)(x.y * sc));
+  }
+}
+
+// G (m x m, a Gram matrix) <- E = (I - G) / 2, one CTA per row; *out = the largest
+// row sum of |E_ij| (FP32 bits, zeroed before the launch; a NaN stays one).
+__global__ void __launch_bounds__(256) start_defect_kernel(double2* __restrict__ G, int m, unsigned int* __restrict__ out) {
+  __shared__ float part[8];
+  const int i = blockIdx.x;
+  float sum = 0.0f;
+  for (int j = threadIdx.x; j < m; j += 256) {
+    double2 g = G[(size_t)i * m + j];
+    g.x = 0.5 * ((i == j ? 1.0 : 0.0) - g.x);
+    g.y = -0.5 * g.y;
+    G[(size_t)i * m + j] = g;
+    const float x = (float)g.x, y = (float)g.y;
+    sum += sqrtf(fmaf(x, x, y * y));
+  }
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = sum;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int q = 1; q < 8; ++q) sum += part[q];
+    atomicMax(out, __float_as_uint(fabsf(sum)));
   }
 }
 

@@ -61,6 +61,7 @@ struct HostSync {   // pinned read-back of the last select + eigen-solve
   unsigned long long phase_ns[4];
   int tc_err;
   GridCtl lq[2];      // control blocks of the FP64 form's LQ step and of its FP32 start
+  float lq_defect;    // orthonormality defect of the FP32 start's left factor (start_defect_kernel)
   GridCtl eig[8];     // FP64 eigen-solves of the last mixed factorisation
   int chol_status;    // Cholesky QR pivot status of the last mixed factorisation
   int chol_pass[2];   // status words after a Cholesky QR pass (cholqr_factor_kernel)
@@ -90,7 +91,8 @@ struct LqWork {
   double2 *z = nullptr, *w = nullptr, *s = nullptr, *v = nullptr, *zd = nullptr;
   double* f = nullptr;
   OSCtl* ctl = nullptr;
-  int* ex = nullptr;
+  int* ex = nullptr;               // [0] the FP32 start's exponent, [1] its defect (FP32 bits)
+  cudaEvent_t ev = nullptr;        // the defect has been read back
 };
 
 struct mpo_ctx {
@@ -399,11 +401,20 @@ constexpr int kLqMinRows = 8;
 // Rows from which the FP32 start pays.
 constexpr int kPreMinRows = 32;
 
+// Defect of the start's left factor (a bound of the 2-norm of E) up to which the
+// four-term correction is enough: 35/8 E^4 <= 4.6e-14 for the bound, 1e-15 for the
+// norm itself; the FP64 solve leaves 2e-14 at the rows (1100) where it is met.
+constexpr float kStartOnce = 3.2e-4f;
+// Up to which one more Newton-Schulz step is enough: the first correction leaves a
+// defect of 35/4 E^4 = 3.6e-8, the step its square. Never met: 2.5e-3 at 8192 rows.
+constexpr float kStartMax = 8e-3f;
+
 // X (r x c, r <= c) <- the rows Sigma V^H, vecs (r x r) <- rows conj(column of
 // U), w <- sigma^2 (lq_kernel). q.ctl[0], q.ctl[1] and ctl receive the barrier
-// errors of the LQ step, of the FP32 start and of the FP64 solve.
+// errors of the LQ step, of the FP32 start and of the FP64 solve; *defect (pinned)
+// its left factor's defect, for which the host waits once.
 static cudaError_t launch_lq_jacobi(cudaStream_t st, double2* X, int r, int c, int ldx, double2* vecs, double* w,
-                                    const LqWork& q, OSCtl* ctl, int max_sweeps, double timeout_s, int num_sms) {
+                                    const LqWork& q, OSCtl* ctl, float* defect, int max_sweeps, double timeout_s, int num_sms) {
   const bool small = c <= 2 * OSJ_NT;
   const void* fn = small ? (const void*)lq_kernel<2> : (const void*)lq_kernel<8>;
   int per_sm = 0;
@@ -420,12 +431,12 @@ static cudaError_t launch_lq_jacobi(cudaStream_t st, double2* X, int r, int c, i
   if (e != cudaSuccess) return e;
   const double2* Y = vecs;       // what the FP64 solve works on, and its accumulated left factor
   double2* Wt = q.w;
-  const bool pre = r >= kPreMinRows;
+  bool pre = r >= kPreMinRows;
   if (pre) {
     const size_t n = (size_t)r * r;
     const dim3 tg((r + 31) / 32, (r + 31) / 32), tb(32, 8);
     float2 *a32 = (float2*)q.s, *u32 = a32 + n;
-    e = cudaMemsetAsync(q.ex, 0, sizeof(int), st);
+    e = cudaMemsetAsync(q.ex, 0, 2 * sizeof(int), st);
     if (e != cudaSuccess) return e;
     max_exp_kernel<<<grid_for(n, num_sms), 256, 0, st>>>(vecs, n, q.ex);
     scale_fp32_kernel<<<grid_for(n, num_sms), 256, 0, st>>>(vecs, n, q.ex, a32);
@@ -434,16 +445,30 @@ static cudaError_t launch_lq_jacobi(cudaStream_t st, double2* X, int r, int c, i
     if (e != cudaSuccess) return e;
     transpose_kernel<float2><<<tg, tb, 0, st>>>(u32, r, r, q.v);                       // W, row-major
     if ((e = cgemm<double>(st, r, r, r, q.v, r, 1, q.v, r, 0, X, r)) != cudaSuccess) return e;   // W^H W (X is free: Z holds the matrix)
-    ns_multiplier_kernel<<<grid_for(n, num_sms), 256, 0, st>>>(X, r);                  // E
+    start_defect_kernel<<<r, 256, 0, st>>>(X, r, (unsigned int*)q.ex + 1);             // E
+    if ((e = cudaMemcpyAsync(defect, q.ex + 1, sizeof(float), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
+    if ((e = cudaEventRecord(q.ev, st)) != cudaSuccess) return e;
     if ((e = cudaMemcpyAsync(q.s, X, n * sizeof(double2), cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
     if ((e = cgemm<double>(st, r, r, r, X, r, 0, X, r, 0, q.s, r, nullptr, 5.0 / 3.0, 1)) != cudaSuccess) return e;   // T = E + 5/3 E^2
     if ((e = cudaMemcpyAsync(Wt, X, n * sizeof(double2), cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
     if ((e = cgemm<double>(st, r, r, r, X, r, 0, q.s, r, 0, Wt, r, nullptr, 1.5, 1)) != cudaSuccess) return e;   // E + 3/2 E T
     if ((e = cudaMemcpyAsync(X, q.v, n * sizeof(double2), cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
     if ((e = cgemm<double>(st, r, r, r, q.v, r, 0, Wt, r, 0, X, r, nullptr, 1.0, 1)) != cudaSuccess) return e;   // W
-    if ((e = cgemm<double>(st, r, r, r, X, r, 1, vecs, r, 0, q.v, r)) != cudaSuccess) return e;                  // W^H R
-    transpose_kernel<double2><<<tg, tb, 0, st>>>(X, r, r, Wt);
-    Y = q.v;
+    if ((e = cudaEventSynchronize(q.ev)) != cudaSuccess) return e;      // the three products above run meanwhile
+    pre = *defect <= kStartMax;      // else (or NaN) the FP64 solve starts from R and the identity
+    const double2* W = X;
+    if (pre && *defect > kStartOnce) {
+      if ((e = cgemm<double>(st, r, r, r, X, r, 1, X, r, 0, q.v, r)) != cudaSuccess) return e;
+      ns_multiplier_kernel<<<grid_for(n, num_sms), 256, 0, st>>>(q.v, r);
+      if ((e = cudaMemcpyAsync(q.s, X, n * sizeof(double2), cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
+      if ((e = cgemm<double>(st, r, r, r, X, r, 0, q.v, r, 0, q.s, r, nullptr, 1.0, 1)) != cudaSuccess) return e;
+      W = q.s;
+    }
+    if (pre) {
+      if ((e = cgemm<double>(st, r, r, r, W, r, 1, vecs, r, 0, q.v, r)) != cudaSuccess) return e;                // W^H R
+      transpose_kernel<double2><<<tg, tb, 0, st>>>(W, r, r, Wt);
+      Y = q.v;
+    }
   }
   // the columns of U come from the rows of the result, so these are made
   // orthogonal relative to their own size down to 1e-14 of the largest each
@@ -964,7 +989,7 @@ static int svd_select(mpo_ctx* h, cplx<T>* X, int r, int c, int ldx, int cap, bo
                                    h->opts.barrier_timeout_s, h->num_sms));
     else if (h->lq.z && r >= kLqMinRows && r <= c) {
       if constexpr (std::is_same<T, double>::value) {
-        CK(h, launch_lq_jacobi(h->st, X, r, c, ldx, (double2*)h->vecs, w, h->lq, h->osctl, h->opts.eig_max_sweeps,
+        CK(h, launch_lq_jacobi(h->st, X, r, c, ldx, (double2*)h->vecs, w, h->lq, h->osctl, &h->hs->lq_defect, h->opts.eig_max_sweeps,
                                h->opts.barrier_timeout_s, h->num_sms));
         h->vecs_conj = true;
       }
@@ -1626,7 +1651,7 @@ static bool alloc_factor_ws(mpo_ctx* h, int m, int ccap, size_t bj_nch) {
 // Workspace of the FP64 form's LQ step.
 static size_t lq_bytes(int m, int ccap) {
   return ((size_t)m * ccap + 3 * (size_t)m * m) * sizeof(double2) + (size_t)m * (sizeof(double2) + sizeof(double)) +
-         2 * sizeof(OSCtl) + sizeof(int) + 8 * 256;
+         2 * sizeof(OSCtl) + 2 * sizeof(int) + 8 * 256;
 }
 
 static bool alloc_lq(mpo_ctx* h, int m, int ccap) {
@@ -1635,7 +1660,7 @@ static bool alloc_lq(mpo_ctx* h, int m, int ccap) {
   return ws_alloc(h, (void**)&q.z, (size_t)m * ccap * sizeof(double2)) && ws_alloc(h, (void**)&q.w, w) &&
          ws_alloc(h, (void**)&q.s, w) && ws_alloc(h, (void**)&q.v, w) &&
          ws_alloc(h, (void**)&q.zd, (size_t)m * sizeof(double2)) && ws_alloc(h, (void**)&q.f, (size_t)m * sizeof(double)) &&
-         ws_alloc(h, (void**)&q.ctl, 2 * sizeof(OSCtl)) && ws_alloc(h, (void**)&q.ex, sizeof(int));
+         ws_alloc(h, (void**)&q.ctl, 2 * sizeof(OSCtl)) && ws_alloc(h, (void**)&q.ex, 2 * sizeof(int));
 }
 
 // All buffers of a handle: `list(lq)` allocates them, with the LQ workspace if lq
@@ -1645,7 +1670,9 @@ static bool ws_build_lq(mpo_ctx* h, int m, int ccap, size_t need, size_t room, c
   size_t freeb = 0, totb = 0;
   const size_t lq = lq_bytes(m, ccap);
   if (h->prec == MPO_FP64 && lq <= room && cudaMemGetInfo(&freeb, &totb) == cudaSuccess && need + lq <= freeb) {
-    if (ws_build(h, [&]() { return list(true); })) return true;
+    if (ws_build(h, [&]() { return list(true); }) &&
+        cudaEventCreateWithFlags(&h->lq.ev, cudaEventDisableTiming) == cudaSuccess)
+      return true;
     cudaFree(h->ws_base);
     h->ws_base = nullptr;
     h->lq = LqWork();
@@ -1811,6 +1838,7 @@ void mpo_free(mpo_handle h) {
   if (h->ws_base) cudaFree(h->ws_base);
   else if (h->hs) cudaStreamSynchronize(h->st);
   hostsync_put(h->hs);
+  if (h->lq.ev) cudaEventDestroy(h->lq.ev);
   for (auto& q : h->pend) { cudaEventDestroy(q.a); cudaEventDestroy(q.b); }
   for (auto e : h->evpool) cudaEventDestroy(e);
   delete h;
