@@ -1219,7 +1219,7 @@ __global__ void __launch_bounds__(256) scale_fp32_kernel(const double2* __restri
 
 // G (m x m, a Gram matrix) <- E = (I - G) / 2, one CTA per row; *out = the largest
 // row sum of |E_ij| (FP32 bits, zeroed before the launch; a NaN stays one).
-__global__ void __launch_bounds__(256) start_defect_kernel(double2* __restrict__ G, int m, unsigned int* __restrict__ out) {
+__global__ void __launch_bounds__(256) half_defect_kernel(double2* __restrict__ G, int m, unsigned int* __restrict__ out) {
   __shared__ float part[8];
   const int i = blockIdx.x;
   float sum = 0.0f;

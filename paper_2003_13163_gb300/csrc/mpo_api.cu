@@ -61,7 +61,8 @@ struct HostSync {   // pinned read-back of the last select + eigen-solve
   unsigned long long phase_ns[4];
   int tc_err;
   GridCtl lq[2];      // control blocks of the FP64 form's LQ step and of its FP32 start
-  float lq_defect;    // orthonormality defect of the FP32 start's left factor (start_defect_kernel)
+  float defect;       // largest row sum of |E| from half_defect_kernel: the FP32 start's left
+                      // factor (FP64 form), the basis of the FP64 Rayleigh-Ritz step (precision form)
   GridCtl eig[8];     // FP64 eigen-solves of the last mixed factorisation
   int chol_status;    // Cholesky QR pivot status of the last mixed factorisation
   int chol_pass[2];   // status words after a Cholesky QR pass (cholqr_factor_kernel)
@@ -92,7 +93,6 @@ struct LqWork {
   double* f = nullptr;
   OSCtl* ctl = nullptr;
   int* ex = nullptr;               // [0] the FP32 start's exponent, [1] its defect (FP32 bits)
-  cudaEvent_t ev = nullptr;        // the defect has been read back
 };
 
 struct mpo_ctx {
@@ -121,6 +121,7 @@ struct mpo_ctx {
   OSCtl* osctl = nullptr;          // control block of the Jacobi launches (barriers, status, counts)
   void *bj_gpart = nullptr, *bj_j = nullptr;   // block Jacobi partial Grams and pair rotations
   int* bj_act = nullptr;                        // block Jacobi integer state (bj_state_ints)
+  cudaEvent_t ev = nullptr;        // HostSync::defect has arrived (not in the complex64 form)
   LqWork lq;                       // FP64 form; all NULL when it did not fit (then no LQ step)
   size_t bj_slots = 0, bj_act_ints = 0;
   int block_min_rows = 0;
@@ -168,7 +169,7 @@ struct mpo_ctx {
   long long prof_steps = 0;        // subspace steps since profiling was switched on
   JRot<double>* mx_rot = nullptr;  // rotation tables of that eigen-solve (two rounds in turn)
   OSCtl* mx_eosctl = nullptr;      // control block of the FP64 Rayleigh-Ritz eigen-solve
-  int* mx_chst = nullptr;          // set when a Cholesky pivot was not positive
+  int* mx_chst = nullptr;          // [0], [1] status of cholqr_factor_kernel, [2] defect (FP32 bits) of half_defect_kernel
   OzWork oz;                       // FP64-accurate tensor-core GEMM scratch (precision form)
   bool use_oz = false;
   bool prof = false;
@@ -414,7 +415,7 @@ constexpr float kStartMax = 8e-3f;
 // errors of the LQ step, of the FP32 start and of the FP64 solve; *defect (pinned)
 // its left factor's defect, for which the host waits once.
 static cudaError_t launch_lq_jacobi(cudaStream_t st, double2* X, int r, int c, int ldx, double2* vecs, double* w,
-                                    const LqWork& q, OSCtl* ctl, float* defect, int max_sweeps, double timeout_s, int num_sms) {
+                                    const LqWork& q, OSCtl* ctl, float* defect, cudaEvent_t ev, int max_sweeps, double timeout_s, int num_sms) {
   const bool small = c <= 2 * OSJ_NT;
   const void* fn = small ? (const void*)lq_kernel<2> : (const void*)lq_kernel<8>;
   int per_sm = 0;
@@ -445,16 +446,16 @@ static cudaError_t launch_lq_jacobi(cudaStream_t st, double2* X, int r, int c, i
     if (e != cudaSuccess) return e;
     transpose_kernel<float2><<<tg, tb, 0, st>>>(u32, r, r, q.v);                       // W, row-major
     if ((e = cgemm<double>(st, r, r, r, q.v, r, 1, q.v, r, 0, X, r)) != cudaSuccess) return e;   // W^H W (X is free: Z holds the matrix)
-    start_defect_kernel<<<r, 256, 0, st>>>(X, r, (unsigned int*)q.ex + 1);             // E
+    half_defect_kernel<<<r, 256, 0, st>>>(X, r, (unsigned int*)q.ex + 1);             // E
     if ((e = cudaMemcpyAsync(defect, q.ex + 1, sizeof(float), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
-    if ((e = cudaEventRecord(q.ev, st)) != cudaSuccess) return e;
+    if ((e = cudaEventRecord(ev, st)) != cudaSuccess) return e;
     if ((e = cudaMemcpyAsync(q.s, X, n * sizeof(double2), cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
     if ((e = cgemm<double>(st, r, r, r, X, r, 0, X, r, 0, q.s, r, nullptr, 5.0 / 3.0, 1)) != cudaSuccess) return e;   // T = E + 5/3 E^2
     if ((e = cudaMemcpyAsync(Wt, X, n * sizeof(double2), cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
     if ((e = cgemm<double>(st, r, r, r, X, r, 0, q.s, r, 0, Wt, r, nullptr, 1.5, 1)) != cudaSuccess) return e;   // E + 3/2 E T
     if ((e = cudaMemcpyAsync(X, q.v, n * sizeof(double2), cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
     if ((e = cgemm<double>(st, r, r, r, q.v, r, 0, Wt, r, 0, X, r, nullptr, 1.0, 1)) != cudaSuccess) return e;   // W
-    if ((e = cudaEventSynchronize(q.ev)) != cudaSuccess) return e;      // the three products above run meanwhile
+    if ((e = cudaEventSynchronize(ev)) != cudaSuccess) return e;      // the three products above run meanwhile
     pre = *defect <= kStartMax;      // else (or NaN) the FP64 solve starts from R and the identity
     const double2* W = X;
     if (pre && *defect > kStartOnce) {
@@ -658,9 +659,10 @@ static cudaError_t mx_gram(mpo_ctx* h, int n, int k, const double2* Y, int ldy, 
 // of 2^-42 then scales with the small E instead of with Y (an isometry defect
 // of 2e-12 came from forming Y (3 I - Y^H Y) / 2 in one product). That product
 // splits Y before it writes C, so it adds to Y in place; the SIMT one adds to
-// a copy (the two buffers are then swapped).
+// a copy (the two buffers are then swapped). With first_defect the largest row sum
+// of the first step's |E| goes to hs->defect (h->ev records its arrival).
 static int mx_newton_schulz(mpo_ctx* h, double2*& Y, double2*& spare, int rows, int m, int iters,
-                            double* defect_dev = nullptr) {
+                            double* defect_dev = nullptr, bool first_defect = false) {
   for (int it = 0; it < iters; ++it) {
     CK(h, mx_gram(h, m, rows, Y, m, 1, h->mx_G, m));
     if (defect_dev && it == iters - 1) {   // |Y^H Y - I| entering the last step
@@ -668,7 +670,13 @@ static int mx_newton_schulz(mpo_ctx* h, double2*& Y, double2*& spare, int rows, 
       defect_kernel<<<grid_for((size_t)m * m, h->num_sms), 256, 0, h->st>>>(h->mx_G, m, defect_dev);
       CK(h, cudaGetLastError());
     }
-    {
+    if (first_defect && it == 0) {
+      CK(h, cudaMemsetAsync(h->mx_chst + 2, 0, sizeof(int), h->st));
+      half_defect_kernel<<<m, 256, 0, h->st>>>(h->mx_G, m, (unsigned int*)h->mx_chst + 2);
+      CK(h, cudaGetLastError());
+      CK(h, cudaMemcpyAsync(&h->hs->defect, h->mx_chst + 2, sizeof(float), cudaMemcpyDeviceToHost, h->st));
+      CK(h, cudaEventRecord(h->ev, h->st));
+    } else {
       ProfScope ps(h, PK_REFINE, 0.0, 2.0 * m * m * sizeof(double2));
       ns_multiplier_kernel<<<grid_for((size_t)m * m, h->num_sms), 256, 0, h->st>>>(h->mx_G, m);
       CK(h, cudaGetLastError());
@@ -919,8 +927,18 @@ static int msvd_select(mpo_ctx* h, double2* X, int r, int c, int ldx, int cap, b
     CK(h, cudaMemcpy2DAsync(Qp, (size_t)mp * sizeof(double2), Vp, (size_t)ldv * sizeof(double2),
                             (size_t)mp * sizeof(double2), r, cudaMemcpyDeviceToDevice, h->st));
   }
-  rc = mx_newton_schulz(h, Qp, Qsp, r, mp, 3);
+  rc = mx_newton_schulz(h, Qp, Qsp, r, mp, 3, nullptr, true);
   if (rc) return rc;
+  // three steps take a defect of up to 0.016 to FP64 rounding (d -> 3/4 d^2 + d^3 / 4,
+  // d = 2 |E|); what the correction leaves is far below (E_PP entries up to 1e-3, but
+  // of random phase), which the host checks while the steps run
+  CK(h, cudaEventSynchronize(h->ev));
+  double d = 2.0 * (double)h->hs->defect;
+  for (int it = 0; d > 1e-15; ++it) {
+    if (it >= 12) return fail(h, MPO_ERR_NOCONV, "basis of the FP64 Rayleigh-Ritz step too far from orthonormal");
+    if (it >= 3 && (rc = mx_newton_schulz(h, Qp, Qsp, r, mp, 1))) return rc;
+    d = d * d * (0.75 + 0.25 * d);
+  }
   // 4. FP64 Rayleigh-Ritz (stage 2): B' = Q'^H X, H' = B' B'^H, nearly
   // diagonal, and the FP64 Hermitian Jacobi eigen-solve H' = V diag(w) V^H
   CK(h, mx_gemm(h, mp, c, r, Qp, mp, 1, X, ldx, 0, h->mx_B, c));            // B' (mp x c)
@@ -989,7 +1007,7 @@ static int svd_select(mpo_ctx* h, cplx<T>* X, int r, int c, int ldx, int cap, bo
                                    h->opts.barrier_timeout_s, h->num_sms));
     else if (h->lq.z && r >= kLqMinRows && r <= c) {
       if constexpr (std::is_same<T, double>::value) {
-        CK(h, launch_lq_jacobi(h->st, X, r, c, ldx, (double2*)h->vecs, w, h->lq, h->osctl, &h->hs->lq_defect, h->opts.eig_max_sweeps,
+        CK(h, launch_lq_jacobi(h->st, X, r, c, ldx, (double2*)h->vecs, w, h->lq, h->osctl, &h->hs->defect, h->ev, h->opts.eig_max_sweeps,
                                h->opts.barrier_timeout_s, h->num_sms));
         h->vecs_conj = true;
       }
@@ -1642,7 +1660,7 @@ static bool alloc_factor_ws(mpo_ctx* h, int m, int ccap, size_t bj_nch) {
     ok = ok && alloc((void**)&h->mx_Q0, (size_t)m * mm * sizeof(double2));
     ok = ok && alloc((void**)&h->mx_A32, mm * mm * sizeof(float2));
     ok = ok && alloc((void**)&h->mx_Li32, mm * mm * sizeof(float2));
-    ok = ok && alloc((void**)&h->mx_chst, 2 * sizeof(int));
+    ok = ok && alloc((void**)&h->mx_chst, 3 * sizeof(int));
     if (!h->ws_plan) ok = ok && cudaMemsetAsync(h->ctl, 0, sizeof(GridCtl), h->st) == cudaSuccess;
   }
   return ok;
@@ -1669,10 +1687,12 @@ static bool alloc_lq(mpo_ctx* h, int m, int ccap) {
 static bool ws_build_lq(mpo_ctx* h, int m, int ccap, size_t need, size_t room, const std::function<bool(bool)>& list) {
   size_t freeb = 0, totb = 0;
   const size_t lq = lq_bytes(m, ccap);
+  if (h->prec != MPO_FP32 && cudaEventCreateWithFlags(&h->ev, cudaEventDisableTiming) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
   if (h->prec == MPO_FP64 && lq <= room && cudaMemGetInfo(&freeb, &totb) == cudaSuccess && need + lq <= freeb) {
-    if (ws_build(h, [&]() { return list(true); }) &&
-        cudaEventCreateWithFlags(&h->lq.ev, cudaEventDisableTiming) == cudaSuccess)
-      return true;
+    if (ws_build(h, [&]() { return list(true); })) return true;
     cudaFree(h->ws_base);
     h->ws_base = nullptr;
     h->lq = LqWork();
@@ -1838,7 +1858,7 @@ void mpo_free(mpo_handle h) {
   if (h->ws_base) cudaFree(h->ws_base);
   else if (h->hs) cudaStreamSynchronize(h->st);
   hostsync_put(h->hs);
-  if (h->lq.ev) cudaEventDestroy(h->lq.ev);
+  if (h->ev) cudaEventDestroy(h->ev);
   for (auto& q : h->pend) { cudaEventDestroy(q.a); cudaEventDestroy(q.b); }
   for (auto e : h->evpool) cudaEventDestroy(e);
   delete h;
