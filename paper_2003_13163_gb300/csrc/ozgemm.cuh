@@ -475,6 +475,7 @@ __global__ void __launch_bounds__(oz::NT, 1) oz_mma_kernel(OzTiles tl, OzOp a, O
         ok = __all_sync(0xffffffffu, tcg::wait_parity(tcg::saddr(&part_done), pphase, timeout_ns));
         if (!ok) break;
         if (tid == 0) {
+          __threadfence();      // the other warps' stores, known here through the mbarrier, before the count
           s_last = atomicAdd(&counters[tile], 1) == tl.splits - 1;
           asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(tcg::saddr(&last_known)) : "memory");
         }
