@@ -346,6 +346,9 @@ __global__ void __launch_bounds__(oz::NT, 1) oz_mma_kernel(OzTiles tl, OzOp a, O
   const uint32_t tbase = tmem_base;
   const int ntiles = tl.count() * tl.splits;
   volatile int* fail = &s_fail;
+  // limit of the waits for this CTA's own copies and MMAs at the end: microseconds,
+  // which a caller's shorter limit must not cut
+  const long long drain_ns = max(timeout_ns, 1000000000ll);
 
   if (warp == NDRAIN) {
     // ---- producer: three bulk copies per stage --------------------------
@@ -375,7 +378,7 @@ __global__ void __launch_bounds__(oz::NT, 1) oz_mma_kernel(OzTiles tl, OzOp a, O
       if (!ok) s_fail = 1;
       // copies still in flight land before the CTA may end
       for (int j = max(0, it - NSTAGE); j < it; ++j)
-        (void)tcg::wait_parity(tcg::saddr(&full[j % NSTAGE]), (uint32_t)(j / NSTAGE) & 1u, timeout_ns);
+        (void)tcg::wait_parity(tcg::saddr(&full[j % NSTAGE]), (uint32_t)(j / NSTAGE) & 1u, drain_ns);
     }
   } else if (warp == NDRAIN + 1) {
     // ---- MMA issue --------------------------------------------------------
@@ -420,7 +423,7 @@ __global__ void __launch_bounds__(oz::NT, 1) oz_mma_kernel(OzTiles tl, OzOp a, O
       if (!ok) s_fail = 1;
       // MMAs still in flight finish before TMEM is released
       for (int j = max(0, it - NSTAGE); j < it; ++j)
-        (void)tcg::wait_parity(tcg::saddr(&empty[j % NSTAGE]), (uint32_t)(j / NSTAGE) & 1u, timeout_ns);
+        (void)tcg::wait_parity(tcg::saddr(&empty[j % NSTAGE]), (uint32_t)(j / NSTAGE) & 1u, drain_ns);
     }
   } else {
     // ---- drain and epilogue ------------------------------------------------
