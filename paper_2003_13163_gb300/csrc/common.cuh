@@ -37,7 +37,9 @@ __device__ __forceinline__ unsigned long long global_timer_ns() {
 }
 
 // Control block of a persistent cooperative kernel: a grid barrier plus
-// status words. Zeroed by the host before every launch.
+// status words. Zeroed by the host before every launch, but for the one of
+// cholqr_factor_kernel: a completed barrier leaves the low bits of the word at zero,
+// and a launch that finds err set leaves at once.
 struct GridCtl {
   unsigned int count;   // barrier word: the top bit flips when every CTA has arrived
   unsigned int unused;

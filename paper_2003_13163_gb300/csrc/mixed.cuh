@@ -227,6 +227,12 @@ __global__ void __launch_bounds__(256) cholqr_factor_kernel(const double2* __res
     if ((tid & 31) == 0) atomicMax(&status[1], __float_as_int(mx));
   };
 
+  // after a barrier of an earlier launch that timed out the word holds a partial
+  // count, and barriers would end before all have arrived
+  if (*(volatile int*)&ctl->err) {
+    if (tid == 0) atomicMax(status, 2);
+    return;
+  }
   if (bid == 0 && tid == 0) status[1] = 0;   // before the first barrier; written after it
   // A = fl32(D G D) + shift I, lower tiles
   for (int q = bid; q < nb * (nb + 1) / 2; q += nblk) {

@@ -692,8 +692,8 @@ static int mx_newton_schulz(mpo_ctx* h, double2*& Y, double2*& spare, int rows, 
   return MPO_OK;
 }
 
-// The FP32 shift 8 m u_32 is explained at mx_cholqr_pass. ctl stays zeroed
-// between launches (a barrier leaves its word's low bits at zero).
+// The FP32 shift 8 m u_32 is explained at mx_cholqr_pass. ctl is not zeroed between
+// launches (see GridCtl): up to fifty of them belong to one factorisation.
 static cudaError_t launch_cholqr_factor(cudaStream_t st, const double2* G, int m, float2* A, float2* Li, double2* W,
                                         int* status, GridCtl* ctl, double timeout_s, int num_sms) {
   cudaError_t e = ensure_dynamic_smem((const void*)cholqr_factor_kernel, CHOL_SMEM);
