@@ -55,7 +55,7 @@ thread_local std::string g_last_init_error;
 thread_local int g_last_svd_sweeps = 0;           // statistics of the last mpo_svd on this thread
 thread_local double g_last_svd_phase_ms[3] = {0.0, 0.0, 0.0};
 
-struct HostSync {   // pinned read-back of the last select + eigen-solve
+struct HostSync {   // read-back of the last select + eigen-solve (pinned on a handle)
   SelectInfo info;
   GridCtl ctl;
   unsigned long long phase_ns[4];
@@ -412,7 +412,7 @@ constexpr float kStartMax = 8e-3f;
 
 // X (r x c, r <= c) <- the rows Sigma V^H, vecs (r x r) <- rows conj(column of
 // U), w <- sigma^2 (lq_kernel). q.ctl[0], q.ctl[1] and ctl receive the barrier
-// errors of the LQ step, of the FP32 start and of the FP64 solve; *defect (pinned)
+// errors of the LQ step, of the FP32 start and of the FP64 solve; *defect
 // its left factor's defect, for which the host waits once.
 static cudaError_t launch_lq_jacobi(cudaStream_t st, double2* X, int r, int c, int ldx, double2* vecs, double* w,
                                     const LqWork& q, OSCtl* ctl, float* defect, cudaEvent_t ev, int max_sweeps, double timeout_s, int num_sms) {
@@ -1590,29 +1590,13 @@ static bool ws_build(mpo_ctx* h, const std::function<bool()>& list) {
   return list();
 }
 
-// Pinned read-back blocks, kept for the next handle (at most kHostSyncKeep of
-// them; a pinned allocation and its free cost ~0.2 ms and a device wait).
-constexpr size_t kHostSyncKeep = 16;
-static std::mutex g_hs_mu;
-static std::vector<HostSync*> g_hs_free;
-
-static HostSync* hostsync_get() {
-  {
-    std::lock_guard<std::mutex> lk(g_hs_mu);
-    if (!g_hs_free.empty()) { HostSync* p = g_hs_free.back(); g_hs_free.pop_back(); return p; }
-  }
+// Pinned read-back block of one handle. Not kept for later handles: a block that
+// outlived its own would be a dangling pointer once the host program resets the
+// device. An allocation and its free cost 0.3 ms per handle.
+static HostSync* hostsync_alloc() {
   HostSync* p = nullptr;
-  if (cudaHostAlloc((void**)&p, sizeof(HostSync), cudaHostAllocPortable) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+  if (cudaMallocHost((void**)&p, sizeof(HostSync)) != cudaSuccess) { cudaGetLastError(); return nullptr; }
   return p;
-}
-
-static void hostsync_put(HostSync* p) {
-  if (!p) return;
-  {
-    std::lock_guard<std::mutex> lk(g_hs_mu);
-    if (g_hs_free.size() < kHostSyncKeep) { g_hs_free.push_back(p); return; }
-  }
-  cudaFreeHost(p);
 }
 
 // Workspace of the factorisations (svd_select / msvd_select) for matrices of
@@ -1817,8 +1801,8 @@ int mpo_init(mpo_handle* out, int n, int chi_max, mpo_precision prec, void* stre
     return ok;
   };
   if (!ws_build_lq(h, m, mx_ccap, need, room, list)) return init_fail(h, MPO_ERR_OOM, "cudaMalloc failed");
-  h->hs = hostsync_get();
-  if (!h->hs) return init_fail(h, MPO_ERR_CUDA, "cudaHostAlloc failed");
+  h->hs = hostsync_alloc();
+  if (!h->hs) return init_fail(h, MPO_ERR_CUDA, "cudaMallocHost failed");
   if (h->use_oz && cudaMemsetAsync(h->oz.status, 0, (1 + oz::MAXITEMS) * sizeof(int), h->st) != cudaSuccess)
     return init_fail(h, MPO_ERR_CUDA, "initial state upload failed");
   // product state |0..0><0..0|: every site 1 x 4 x 1 with A[0][0][0] = 1 (Sec. 4.1)
@@ -1856,8 +1840,7 @@ void mpo_free(mpo_handle h) {
   // a handle's buffers and its read-back block may still be in use on its stream
   // after an error or a call that did not wait; cudaFree waits for the device
   if (h->ws_base) cudaFree(h->ws_base);
-  else if (h->hs) cudaStreamSynchronize(h->st);
-  hostsync_put(h->hs);
+  if (h->hs) cudaFreeHost(h->hs);
   if (h->ev) cudaEventDestroy(h->ev);
   for (auto& q : h->pend) { cudaEventDestroy(q.a); cudaEventDestroy(q.b); }
   for (auto e : h->evpool) cudaEventDestroy(e);
@@ -2195,8 +2178,12 @@ int mpo_svd_truncated(int r, int c, const void* A, int cap, mpo_precision prec, 
            (!lq || alloc_lq(h, r, c));
   };
   bool ok = ws_build_lq(h, r, c, 0, h->opts.arena_cap_bytes > 0 ? 0 : ~(size_t)0, list);
-  if (ok && !(h->hs = hostsync_get())) ok = false;
-  if (!ok) { mpo_free(h); g_last_init_error = "mpo_svd_truncated: allocation failed"; return MPO_ERR_OOM; }
+  // the read-back block of one call: plain memory, because pinning one costs 0.3 ms
+  // and its copies 0.1 ms (256 x 256: 14.9 and 14.4 ms); it outlives mpo_free, which waits
+  // for the device, so a copy still under way after an error has landed
+  HostSync hs;
+  h->hs = &hs;
+  if (!ok) { h->hs = nullptr; mpo_free(h); g_last_init_error = "mpo_svd_truncated: allocation failed"; return MPO_ERR_OOM; }
   int rc = MPO_OK, kk = 0;
   auto ck = [&](cudaError_t e) { if (rc == MPO_OK && e != cudaSuccess) { rc = MPO_ERR_CUDA; g_last_init_error = cudaGetErrorString(e); } };
   ck(cudaMemcpyAsync(h->theta, A, (size_t)r * c * h->esz, cudaMemcpyDeviceToDevice, h->st));
@@ -2220,6 +2207,7 @@ int mpo_svd_truncated(int r, int c, const void* A, int cap, mpo_precision prec, 
     ck(cudaStreamSynchronize(h->st));
     *k = kk;
   }
+  h->hs = nullptr;
   mpo_free(h);
   return rc;
 }
