@@ -85,7 +85,8 @@ typedef struct {
                                factorisation [1e-12 for FP64, 1e-6 for FP32: the rounding
                                floor of the one-sided Jacobi SVD; 1e-7 for MPO_MIXED_FP32]; <= 0
                                selects the default */
-  size_t arena_cap_bytes;   /* refuse device allocations above this total [0 = no cap] */
+  size_t arena_cap_bytes;   /* refuse device allocations above this total [0 = no cap]. MPO_FP64:
+                               a cap without room for the LQ workspace (see mpo_init) leaves it out */
   mpo_entropy_mode smode;   /* [MPO_S_ALL_BONDS] */
   double barrier_timeout_s; /* limit of each device-side grid-barrier wait [5.0] */
   int block_jacobi_min_rows;/* factorisations with at least this many rows use the block
@@ -122,7 +123,11 @@ void mpo_default_opts(mpo_opts *o);
  *   opts       : NULL for defaults.
  * Allocates all device memory up front for the worst-case bond dimensions
  * min(chi_max, 4^b, 4^(n-b)); returns MPO_ERR_OOM if that exceeds the device
- * or arena_cap_bytes. */
+ * or arena_cap_bytes. MPO_FP64 handles also take the workspace of the LQ step,
+ * about 64 m^2 bytes for m = 4 chi_max rows (1.1 GB at chi_max = 1024), which makes
+ * the factorisations about three times faster and changes results in rounding
+ * only; it is left out where it is more than a sixteenth of the device memory
+ * that the handle leaves free, or exceeds arena_cap_bytes. */
 int mpo_init(mpo_handle *out, int n_qubits, int chi_max, mpo_precision prec,
              void *cuda_stream, const mpo_opts *opts);
 

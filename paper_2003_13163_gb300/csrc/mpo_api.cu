@@ -1581,11 +1581,16 @@ static bool ws_alloc(mpo_ctx* h, void** p, size_t bytes) {
   return true;
 }
 
-static bool ws_build(mpo_ctx* h, const std::function<bool()>& list) {
+static size_t ws_size(mpo_ctx* h, const std::function<bool()>& list) {
   h->ws_cap = h->ws_off = 0;
   h->ws_plan = true;
   list();
   h->ws_plan = false;
+  return h->ws_cap;
+}
+
+static bool ws_build(mpo_ctx* h, const std::function<bool()>& list) {
+  ws_size(h, list);
   if (cudaMalloc((void**)&h->ws_base, h->ws_cap) != cudaSuccess) { cudaGetLastError(); h->ws_base = nullptr; return false; }
   return list();
 }
@@ -1666,16 +1671,23 @@ static bool alloc_lq(mpo_ctx* h, int m, int ccap) {
 }
 
 // All buffers of a handle: `list(lq)` allocates them, with the LQ workspace if lq
-// is set. That one only saves time, so a handle whose memory limit (`room` bytes
-// left) or device has no room for it goes without.
-static bool ws_build_lq(mpo_ctx* h, int m, int ccap, size_t need, size_t room, const std::function<bool(bool)>& list) {
+// is set. That one only saves time (a 256 x 256 factorisation takes 14 ms with it, 52
+// without), so it must not cost another handle or library its memory: a handle whose
+// memory limit (`room` bytes left) has no room for it goes without, and so does one
+// where it is more than kLqShare of the memory that the handle leaves free on the
+// device.
+constexpr double kLqShare = 1.0 / 16;
+
+static bool ws_build_lq(mpo_ctx* h, int m, int ccap, size_t room, const std::function<bool(bool)>& list) {
   size_t freeb = 0, totb = 0;
   const size_t lq = lq_bytes(m, ccap);
   if (h->prec != MPO_FP32 && cudaEventCreateWithFlags(&h->ev, cudaEventDisableTiming) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  if (h->prec == MPO_FP64 && lq <= room && cudaMemGetInfo(&freeb, &totb) == cudaSuccess && need + lq <= freeb) {
+  const size_t base = ws_size(h, [&]() { return list(false); });
+  if (h->prec == MPO_FP64 && lq <= room && cudaMemGetInfo(&freeb, &totb) == cudaSuccess && base < freeb &&
+      (double)lq <= kLqShare * (double)(freeb - base)) {
     if (ws_build(h, [&]() { return list(true); })) return true;
     cudaFree(h->ws_base);
     h->ws_base = nullptr;
@@ -1800,7 +1812,7 @@ int mpo_init(mpo_handle* out, int n, int chi_max, mpo_precision prec, void* stre
     if (ok && lq) ok = alloc_lq(h, m, mx_ccap);
     return ok;
   };
-  if (!ws_build_lq(h, m, mx_ccap, need, room, list)) return init_fail(h, MPO_ERR_OOM, "cudaMalloc failed");
+  if (!ws_build_lq(h, m, mx_ccap, room, list)) return init_fail(h, MPO_ERR_OOM, "cudaMalloc failed");
   h->hs = hostsync_alloc();
   if (!h->hs) return init_fail(h, MPO_ERR_CUDA, "cudaMallocHost failed");
   if (h->use_oz && cudaMemsetAsync(h->oz.status, 0, (1 + oz::MAXITEMS) * sizeof(int), h->st) != cudaSuccess)
@@ -2177,7 +2189,7 @@ int mpo_svd_truncated(int r, int c, const void* A, int cap, mpo_precision prec, 
            alloc((void**)&h->scal, 8 * sizeof(double)) && (!h->use_oz || alloc_oz(h->oz, c, c, c, h->opts.arena_cap_bytes > 0 ? 0 : oz_part_bytes(c, c, h->num_sms), alloc)) &&
            (!lq || alloc_lq(h, r, c));
   };
-  bool ok = ws_build_lq(h, r, c, 0, h->opts.arena_cap_bytes > 0 ? 0 : ~(size_t)0, list);
+  bool ok = ws_build_lq(h, r, c, h->opts.arena_cap_bytes > 0 ? 0 : ~(size_t)0, list);
   // the read-back block of one call: plain memory, because pinning one costs 0.3 ms
   // and its copies 0.1 ms (256 x 256: 14.9 and 14.4 ms); it outlives mpo_free, which waits
   // for the device, so a copy still under way after an error has landed
