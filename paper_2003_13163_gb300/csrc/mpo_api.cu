@@ -558,6 +558,15 @@ constexpr int kCorrectMin = 32;       // basis size from which an untruncated so
 constexpr int kMixedMaxSteps = 24;    // cap on subspace-iteration steps of one factorisation
 constexpr int kMixedSteps = 4;        // steps before the first convergence check
 
+// K parts per tile. A tile takes ~0.7 us per stage: split K while tiles leave SMs
+// idle, into parts of at least twenty stages (parts of eight made the K = 256 products
+// of a short chain's circuit slower: 222 -> 226 ms; 513 x 300 x 1100: 405 us whole,
+// 349 in three).
+static int oz_splits(const OzTiles& tl, int num_sms) {
+  if (2 * tl.count() > num_sms || num_sms > oz::MAXITEMS) return 1;
+  return std::max(1, std::min(std::min(oz::MAXSPLIT, num_sms / tl.count()), 2 * tl.nkb / 20));
+}
+
 // C (M x N) = alpha op(A) op(B) (+ C), complex128, FP64-accurate on the
 // tensor cores (ozgemm.cuh): exponents, BF16 slices of both operands, then
 // the MMA kernel. Returns cudaErrorInvalidValue if the scratch is too small.
@@ -586,12 +595,8 @@ static cudaError_t oz_gemm(cudaStream_t st, int M, int N, int K, const double2* 
   if (e != cudaSuccess) return e;
   e = ensure_dynamic_smem((const void*)oz_mma_kernel, oz::SMEM_BYTES);
   if (e != cudaSuccess) return e;
-  // a tile takes ~0.7 us per stage: split K while tiles leave SMs idle, into parts
-  // of at least twenty stages (parts of eight made the K = 256 products of a short
-  // chain's circuit slower: 222 -> 226 ms; 513 x 300 x 1100: 405 us whole, 349 in three)
   OzTiles tl{Mp / oz::BM, Nrp / oz::BN, nkb, mode, 1};
-  if (w.part && 2 * tl.count() <= num_sms && num_sms <= oz::MAXITEMS)
-    tl.splits = std::max(1, std::min(std::min(oz::MAXSPLIT, num_sms / tl.count()), 2 * nkb / 20));
+  if (w.part) tl.splits = oz_splits(tl, num_sms);
   oz_mma_kernel<<<std::min(num_sms, tl.count() * tl.splits), oz::NT, oz::SMEM_BYTES, st>>>(tl, a, b, C, ldc, alpha, accumulate, w.part, w.counters,
                                                                                   w.status, (long long)(timeout_s * 1e9));
   return cudaGetLastError();
@@ -2352,8 +2357,12 @@ int mpo_gemm_ex(int M, int N, int K, const void* A, int lda, int opA, const void
   cudaError_t e = cudaSuccess;
   int hs = 0;
   if (prec == MPO_FP64 && engine == 1) {
-    // one allocation, sized for this product
+    // one allocation, sized for this product (with the parts of an unsplit one it
+    // outgrew what the driver keeps at hand: 100 x 100 x 100 0.26 ms, 0.10 without)
     OzWork w;
+    const OzTiles tl{(M + oz::BM - 1) / oz::BM, (2 * N + oz::BN - 1) / oz::BN, (K + 15) / 16, OzTiles::kGeneral, 1};
+    const int splits = oz_splits(tl, sms);
+    const size_t part = splits > 1 ? (size_t)tl.count() * splits * oz::PART_BYTES : 0;
     size_t off = 0;
     char* base = nullptr;
     auto carve = [&](void** p, size_t bytes) -> bool {
@@ -2361,10 +2370,10 @@ int mpo_gemm_ex(int M, int N, int K, const void* A, int lda, int opA, const void
       off += (bytes + 255) & ~(size_t)255;
       return true;
     };
-    alloc_oz(w, M, N, K, oz_part_bytes(M, N, sms), carve);
+    alloc_oz(w, M, N, K, part, carve);
     if (cudaMalloc((void**)&base, off) != cudaSuccess) { cudaGetLastError(); return MPO_ERR_OOM; }
     off = 0;
-    alloc_oz(w, M, N, K, oz_part_bytes(M, N, sms), carve);
+    alloc_oz(w, M, N, K, part, carve);
     e = cudaMemsetAsync(w.status, 0, (1 + oz::MAXITEMS) * sizeof(int), st);
     if (e == cudaSuccess)
       e = oz_gemm(st, M, N, K, (const double2*)A, lda, opA, (const double2*)B, ldb, opB, (double2*)C, ldc, 1.0, 0, w,
