@@ -50,17 +50,17 @@ typedef struct mpo_ctx *mpo_handle;
  *   MPO_FP32:       complex64 site tensors and FP32 contractions and eigen-solves;
  *                   Schmidt-value normalisation, entropy and log-norm stay FP64.
  *                   Fast, but its entropies differ from the FP64 form by ~1e-3.
- *   MPO_MIXED_FP32: the precision form. complex128 site tensors; every truncated
- *                   SVD (App. A) and centre move starts from the FP32 one-sided
- *                   Jacobi SVD of an FP32 copy, whose m = chi_max + oversample
- *                   leading left singular vectors Q are refined in FP64 by one
- *                   Rayleigh-Ritz step: B = Q^H theta' and H = B B^H by
- *                   FP64-accurate products, and the FP64 Hermitian Jacobi
- *                   eigen-solve of H (optionally preceded by refine_steps FP64
- *                   subspace-iteration steps); the singular values, their
+ *   MPO_MIXED_FP32: the precision form. complex128 site tensors; a truncating SVD
+ *                   (App. A) iterates a random subspace of m = chi_max + oversample
+ *                   directions with FP64-accurate products, solves on it in FP32
+ *                   (any other SVD starts with that solve, on theta' itself),
+ *                   corrects the leading vectors to first order and ends with an
+ *                   FP64 Rayleigh-Ritz step: B = Q^H theta', H = B B^H and the FP64
+ *                   Hermitian Jacobi eigen-solve of H. The singular values, their
  *                   normalisation and the entropy are FP64. Matches the FP64
  *                   form to |dS| <= 1e-6 and a kept-theta relative Frobenius
- *                   error <= 1e-7 per gate. */
+ *                   error <= 1e-7 per gate. A matrix that holds infinities or NaN
+ *                   ends with MPO_ERR_NOCONV. */
 typedef enum { MPO_FP64 = 0, MPO_FP32 = 1, MPO_MIXED_FP32 = 2 } mpo_precision;
 
 /* Which bonds mpo_entropy reports.
@@ -101,12 +101,11 @@ typedef struct {
                                MPO_MIXED_FP32: >= 0 runs its FP64 products (theta, the
                                refinement and the projections) on the tensor cores as
                                FP64-accurate BF16 split products [0 = on; < 0 = SIMT FP64] */
-  int oversample;           /* MPO_MIXED_FP32: extra FP32 singular vectors carried into the FP64
-                               Rayleigh-Ritz step of a truncating SVD, beyond chi_max [0 = 64;
-                               < 0 = none] */
-  int refine_steps;         /* MPO_MIXED_FP32: FP64 subspace-iteration steps (shifted CholeskyQR3
-                               after each product) before the Rayleigh-Ritz step of a truncating
-                               SVD [0 or < 0 = none, the default; at most 7] */
+  int oversample;           /* MPO_MIXED_FP32: directions of the iterated subspace of a truncating
+                               SVD beyond chi_max [0 = chi_max; < 0 = none] */
+  int refine_steps;         /* MPO_MIXED_FP32: subspace-iteration steps of a truncating SVD before
+                               its convergence is first checked, which adds steps up to 24 in all
+                               [0 = 4; < 0 = 1; at most 24] */
 } mpo_opts;
 
 /* Fill *o with the defaults. */

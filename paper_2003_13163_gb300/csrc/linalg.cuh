@@ -153,6 +153,8 @@ __global__ void __launch_bounds__(256) cgemm_small_kernel(int M, int N, int K, c
   C[(size_t)r * ldc + c] = v;
 }
 
+constexpr int kTileSms = 152;     // SMs of the part: fewer 16 x 16 tiles than that go as 8 x 8 ones
+
 template <typename T>
 inline cudaError_t cgemm(cudaStream_t st, int M, int N, int K, const cplx<T>* A, int lda, int opA,
                          const cplx<T>* B, int ldb, int opB, cplx<T>* C, int ldc,
@@ -170,7 +172,7 @@ inline cudaError_t cgemm(cudaStream_t st, int M, int N, int K, const cplx<T>* A,
   }
   if constexpr (sizeof(T) == 8) {
     const long nr16 = (M + 15) / 16, nc16 = (N + 15) / 16, nr8 = (M + 7) / 8, nc8 = (N + 7) / 8;
-    if (nr16 * nc16 < 152)      // fewer tiles than the part's SMs
+    if (nr16 * nc16 < kTileSms)
       cgemm_small_kernel<T, 8><<<(unsigned)(nr8 * nc8), 256, 0, st>>>(M, N, K, A, lda, opA, B, ldb, opB, C, ldc, alpha_dev,
                                                                       alpha_host, accumulate, (int)nc8);
     else
@@ -365,6 +367,7 @@ __global__ void __launch_bounds__(1024) select_kernel(const T* __restrict__ w, i
 // Ut    t_p <- c t_p - u* s t_q,  t_q <- s t_p + u* c t_q      (U <- U J)
 // Ordering is round-robin as above; pairs of one round touch disjoint rows,
 // so a round is one phase (one warp per pair) followed by one grid barrier.
+// The complex64 form below its block solver's smallest size.
 // A sweep with no rotation (|g| <= max(tol sqrt(ab), floor)) ends the solve.
 // ---------------------------------------------------------------------------
 struct OSCtl {
@@ -409,8 +412,7 @@ __global__ void __launch_bounds__(256) onesided_jacobi_kernel(cplx<T>* X, int r,
   const unsigned nblk = gridDim.x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwb = blockDim.x >> 5;
   // warp w of CTA b takes the pairs w gridDim + b, ...: neighbouring pairs go to
-  // different SMs, so that a round of fewer pairs than warps uses the FP64
-  // units of every SM (8 neighbours on one SM left 104 of 152 idle at r = 768)
+  // different SMs, so that a round of fewer pairs than warps uses every SM
   const long gwarp = (long)warp * nblk + blockIdx.x, nwarps = (long)nblk * nwb;
   const size_t gtid = (size_t)blockIdx.x * blockDim.x + threadIdx.x, gthreads = (size_t)nblk * blockDim.x;
   if (max_sweeps > 64) max_sweeps = 64;
@@ -497,10 +499,10 @@ __global__ void __launch_bounds__(256) onesided_jacobi_kernel(cplx<T>* X, int r,
 }
 
 // ---------------------------------------------------------------------------
-// The same solver with one CTA (four warps) per row pair, the form every
-// complex128 factorisation and the precision form's FP32 Rayleigh-Ritz step
-// use (onesided_jacobi_kernel above serves the complex64 form, whose results
-// are pinned to its arithmetic).
+// The same solver with one CTA (four warps) per row pair: every complex128
+// factorisation, and the FP32 solves (quad_jacobi_kernel below) of fewer than 32
+// rows or more than 4096 columns. onesided_jacobi_kernel above serves the
+// complex64 form, whose results are pinned to its arithmetic.
 //
 // What bounds it: an FP64 warp instruction occupies its SM partition for 64
 // clocks on this part, so a pair handled by one warp uses a quarter of the
@@ -513,8 +515,7 @@ __global__ void __launch_bounds__(256) onesided_jacobi_kernel(cplx<T>* X, int r,
 // (one read and one write per round instead of two and one).
 // Measured, one warp per pair -> this kernel: complex128 64 x 64 17.2 ->
 // 7.1 ms (20 sweeps), 256 x 256 174 -> 51 ms, 768 x 1024 1363 -> 586 ms
-// (28 sweeps, 27 us per round); complex64 2048 x 2048 in the precision form
-// 557 -> 166 ms.
+// (28 sweeps, 27 us per round).
 // ---------------------------------------------------------------------------
 constexpr int OSJ_NT = 128;
 
@@ -1640,7 +1641,7 @@ __device__ __forceinline__ void bj_rot_params(const cplx<TI>* G, int p, int q, T
   }
 }
 
-// One round of the cyclic parallel Jacobi as 2 x 2 block updates: the round's
+// Pair solve: one round of the cyclic parallel Jacobi as 2 x 2 block updates: the round's
 // JP/2 disjoint rotations partition the indices into pairs, so the JP x JP
 // matrix splits into (JP/2)^2 blocks B_ab = G[{p_a, q_a}][{p_b, q_b}], each
 // updated on its own as B_ab <- R_a^H B_ab R_b. Thread (a, b) derives both

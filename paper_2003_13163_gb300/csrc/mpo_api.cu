@@ -527,28 +527,22 @@ static cudaError_t launch_block_jacobi(cudaStream_t st, cplx<T>* X, int r, int c
 // ---------------------------------------------------------------------------
 // Precision form: truncated SVD of a complex128 matrix X (r x c, r <= c,
 // leading dimension ldx) keeping at most cap singular values (App. A), with
-// the heavy lifting in FP32 and the accuracy won back in FP64.
-//   1. FP32 one-sided Jacobi SVD of fl32(X) -> approximate U (r x r), w.
-//   2. Q (r x m, FP64) = the m = min(r, cap + oversample) leading columns of U,
-//      made orthonormal to FP64 rounding by Newton-Schulz steps.
-//   3. Optional (refine_steps > 0, only when m < r): subspace-iteration steps
-//      W <- orth(X^H Q), Q <- orth(X W) in FP64, each damping the components
-//      of the leading singular vectors outside span(Q) by
-//      (sigma_{m+1} / sigma_j)^2; orth is shifted Cholesky QR followed by two
-//      Cholesky QR passes (shifted CholeskyQR3, stable for condition numbers
-//      up to 1/u), applied after each product so that a basis never carries
-//      more than the condition number sigma_1 / sigma_m; the refined basis is
-//      then turned back towards the FP32 one (Q <- Q W, W the orthonormal
-//      factor of Q^H Q_FP32) so that the Rayleigh-Ritz matrix stays nearly
-//      diagonal.
-//   4. Rayleigh-Ritz in FP64: B = Q^H X (m x c), H = B B^H (m x m), both by
-//      the FP64-class products, and the FP64 Hermitian Jacobi eigen-solve
-//      H = V diag(w) V^H. With Q from the FP32 singular vectors H is nearly
-//      diagonal, so the solve ends after a few sweeps. The Ritz values w are
-//      the squared singular values, Q V the left singular vectors and the rows
-//      of V^H B = Lambda W^H the scaled right ones.
-// Outputs follow the one-sided Jacobi convention of svd_select: rows 0..m-1
-// of X are overwritten with V^H B, h->vecs holds V^H Q^H (m x r, row j = conj
+// the heavy lifting in FP64-accurate tensor-core products and FP32 solves.
+//   1. When m = min(r, cap + oversample) < r: randomized subspace iteration on m
+//      directions, Q <- orth(X orth(X^H Q)) from a seeded Gaussian start, orth by
+//      mixed-precision Cholesky QR (mx_cholqr) and at the end Newton-Schulz steps.
+//   2. FP32 Rayleigh-Ritz: the row Jacobi SVD of M = Q^H X T (m x m, T the last
+//      right basis), or of X itself when m = r. Its Ritz values decide whether the
+//      iteration takes more steps (at most kMixedMaxSteps).
+//   3. First-order correction of its mp = min(m, cap + kMixedMargin) leading vectors
+//      (partition_correction_kernel), then Q' = Q V_P made orthonormal to FP64
+//      rounding by as many Newton-Schulz steps as that takes.
+//   4. Rayleigh-Ritz in FP64: B = Q'^H X (mp x c), H = B B^H by the FP64-class
+//      products, and the two-sided FP64 Jacobi eigen-solve H = V diag(w) V^H of the
+//      nearly diagonal H. The Ritz values w are the squared singular values, Q' V the
+//      left singular vectors and the rows of V^H B = Lambda W^H the scaled right ones.
+// Outputs follow the one-sided Jacobi convention of svd_select: rows 0..mp-1
+// of X are overwritten with V^H B, h->vecs holds V^H Q'^H (mp x r, row j = conj
 // of left singular vector j: h->vecs_conj), h->mx_w the w; the select kernel
 // then sorts and truncates, with the discarded weight taken against the
 // squared Frobenius norm of X (the Ritz values cover span(Q) only).

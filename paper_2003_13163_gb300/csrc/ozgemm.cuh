@@ -19,8 +19,8 @@
 //
 // Accumulation. The products of one level L = t + u are summed in their own
 // TMEM accumulator: within a level every product is an integer multiple of
-// 2^{-7L}, and over a K chunk of KC real terms those integer sums stay far
-// below 2^24, so each chunk's sum is exact whatever the alignment and
+// 2^{-7L}, and over a K chunk of KC real terms those integer sums are at most
+// 2^24, so each chunk's sum is exact whatever the alignment and
 // rounding inside the tensor core's FP32 accumulation (levels of different
 // units must not share an accumulator: their small terms would fall below
 // the accumulator's resolution, an error growing with K). After each chunk
@@ -50,11 +50,12 @@
 // thread the MMAs, eight warps drain the accumulators and write C, so the
 // copies of the next tile run under the epilogue of this one. Every wait is
 // bounded.
-// What bounds it: shared memory bandwidth. A stage of 16 real K takes 768 clocks
-// of the tensor pipe, but the MMAs read 96 KB and the copies write 36 KB of
-// shared memory for it (1056 clocks at 128 B). 4096 x 2048 x 4096: 13.75 ms
-// with cp.async loads one stage ahead and N = 64 MMAs, 4.92 ms now (tensor pipe
-// 54 % active, 55.9 TFLOP/s of FP64-accurate work, L2 reads 7.9 TB/s).
+// What bounds it: most likely L2, whose reads run at 7.9 TB/s. A stage of 16 real K
+// takes 768 clocks of the tensor pipe and 1056 of shared memory (the MMAs read
+// 96 KB, the copies write 36 KB, at 128 B per clock) but 1343 in all, and a CTA pair
+// with 23 % less shared-memory traffic was no faster (6.8 ms per call instead of
+// 6.0). 4096 x 2048 x 4096: 13.75 ms with cp.async loads one stage ahead and N = 64
+// MMAs, 4.92 ms now (tensor pipe 54 % active, 55.9 TFLOP/s of FP64-accurate work).
 #pragma once
 #include <cuda_bf16.h>
 #include "common.cuh"
@@ -67,6 +68,7 @@ constexpr int KS = 16;                       // real K per stage: one MMA deep
 // real K per exact chunk: a level's products sum to at most 2^15 units per K
 // (|a_1| <= 128, |a_t| <= 64: 2 * 2^13 + 4 * 2^12 at level 7), 2^24 per chunk
 constexpr int KC = 512;
+static_assert((long long)KC * (2 * 128 * 64 + (S - 2) * 64 * 64) <= 1ll << 24, "a chunk's sums must be exact in FP32");
 constexpr int SPC = KC / KS;                 // stages per chunk
 constexpr int A_STAGE = S * 2 * BM * 16;     // 24 KB in global and shared memory
 constexpr int B_STAGE = 2 * S * BN * 16;     // 12 KB in global memory
