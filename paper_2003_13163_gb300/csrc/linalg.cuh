@@ -230,7 +230,8 @@ __device__ __forceinline__ int rr_player(int pos, int r, int N) {
 // squared Schmidt values lambda'^2 of the factorised bond) into the kept set.
 //   - bitonic sort of (value desc, index asc) in shared memory (stable order
 //     for exact ties), negative rounding values clamped to 0;
-//   - k = min(cap, #{lambda^2 > cutoff^2 * lambda_max^2}), at least 1;
+//   - k = min(cap, #{lambda^2 > cutoff^2 * lambda_max^2}), at least 1; min(cap, m) when
+//     cutoff2 < 0, also where every value is zero (callers then read all of perm);
 //   - sums in FP64: total = sum lambda^2 (or *total_in, the squared Frobenius
 //     norm of the factorised matrix, when w holds Ritz values of a subspace
 //     only), kept = sum of the k largest;
@@ -302,7 +303,7 @@ __global__ void __launch_bounds__(1024) select_kernel(const T* __restrict__ w, i
     const double thr = cutoff2 * key[0];
     int k = 0;
     const int lim = cap < m ? cap : m;
-    while (k < lim && key[k] > thr) ++k;
+    while (k < lim && (cutoff2 < 0.0 || key[k] > thr)) ++k;
     if (k == 0) k = 1;
     s_k = k;
   }
