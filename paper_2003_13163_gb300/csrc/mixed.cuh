@@ -414,7 +414,9 @@ __global__ void hermitise_kernel(double2* __restrict__ H, int m) {
 // remaining columns (j >= mp) that is what keeps the FP32 solve's couplings out
 // of the kept subspace; pairs with a relative gap below 1e-2 (inside a cluster
 // at the edge, only in the margin beyond the kept directions) get the
-// orthogonality term R_ji / 2 alone. Among the leading columns it saves the FP64
+// orthogonality term R_ji / 2 alone, and so do pairs with |E_ji| > 1e-2: couplings of
+// 3e-5 give at most 3e-3 there, so both values are rounding of zeros (a rank
+// below mp), and E_ji their ratio, of any size. Among the leading columns it saves the FP64
 // eigen-solve that follows a sweep; there a pair is taken where |E_ji| <= 1e-3, so
 // that V_P (I + E_PP) stays within reach of the Newton-Schulz steps, else R_ji / 2.
 // A pair without a gap is never taken: exactly equal values with no coupling
@@ -434,8 +436,8 @@ __global__ void partition_correction_kernel(const double2* __restrict__ S, const
     const double2 rji = make_double2(-g.x, -g.y);      // (I - G)_ji, j != i
     const double gap = li - lj;
     const double2 num = make_double2(s.x + li * rji.x, s.y + li * rji.y);
-    const bool far = j < mp ? fabs(gap) > 0.0 && fmax(fabs(num.x), fabs(num.y)) <= 1e-3 * fabs(gap)
-                            : fabs(gap) > 1e-2 * fmax(fabs(li), fabs(lj));
+    const double an = fmax(fabs(num.x), fabs(num.y)), ag = fabs(gap);
+    const bool far = j < mp ? ag > 0.0 && an <= 1e-3 * ag : ag > 1e-2 * fmax(fabs(li), fabs(lj)) && an <= 1e-2 * ag;
     E[e] = far ? make_double2(num.x / gap, num.y / gap) : make_double2(0.5 * rji.x, 0.5 * rji.y);
   }
 }
