@@ -73,7 +73,8 @@ enum {
   MPO_ERR_ARG = -1,     /* invalid argument (sizes, parity, NULL)              */
   MPO_ERR_CUDA = -2,    /* a CUDA call failed, or no device                    */
   MPO_ERR_OOM = -3,     /* device allocation failed or exceeded arena_cap_bytes */
-  MPO_ERR_NOCONV = -4,  /* an SVD / eigen-solve hit its sweep cap unconverged   */
+  MPO_ERR_NOCONV = -4,  /* an SVD / eigen-solve hit its sweep cap unconverged, or
+                           cannot resolve its input (underflow; NaN, rank: precision form) */
   MPO_ERR_TIMEOUT = -5, /* a bounded device-side wait gave up                   */
   MPO_ERR_STATE = -6    /* handle is in an error state or call order is wrong   */
 };
